@@ -79,6 +79,29 @@ Geo make_geo(const fvm_params& p, const LevelShape& s) {
   return g;
 }
 
+// first level of the coarse tail (fvm_tail.cu): the finest one below level 0
+// (or level 0 when there is no other) from which all levels fit; -1 when not
+// even the coarsest does.  pack: bytes of its packed coefficients
+template <typename T>
+int tail_first_of(const fvm_params& p, const LevelShape* lv, int nl, size_t* pack) {
+  MGLevel<T> Ls[kMaxLevels];
+  for (int l = 0; l < nl; ++l) {
+    Ls[l] = MGLevel<T>();
+    Ls[l].geo = make_geo(p, lv[l]);
+    for (int d = 0; d < 3; ++d) Ls[l].f[d] = lv[l].f[d];
+  }
+  TailArgs<T> A;
+  size_t smem = 0;
+  for (int l = nl > 1 ? 1 : 0; l < nl; ++l)
+    if (tail_layout<T>(Ls + l, nl - l, A, &smem, pack)) return l;
+  *pack = 0;
+  return -1;
+}
+int tail_first(const fvm_params& p, const LevelShape* lv, int nl, size_t* pack) {
+  return p.precision == FVM_MIXED ? tail_first_of<float>(p, lv, nl, pack)
+                                  : tail_first_of<double>(p, lv, nl, pack);
+}
+
 const char* check_params(const fvm_params* p) {
   if (!p) return "params is NULL";
   if (p->nx < 1 || p->ny < 1 || p->nz < 1) return "grid sizes must be >= 1";
@@ -157,6 +180,8 @@ struct fvm_ctx {
   void* lb[kMaxLevels];
   void* lbeta[kMaxLevels][3];
   void* cg[3];
+  int tail;              // first level of the coarse tail, -1: none
+  void* pack;            // the tail's packed coefficients (null: formed in every cycle)
   // reduction scratch
   double* partial;
   double* scal;          // 16 doubles
@@ -276,6 +301,9 @@ size_t plan_workspace(const fvm_params& p, fvm_ctx* c) {
   long long nc = (long long)lv[nl - 1].n[0] * lv[nl - 1].n[1] * lv[nl - 1].n[2];
   size_t o_cg[3];   // r, d and (Ad, x) in double
   for (int q = 0; q < 3; ++q) o_cg[q] = pl.take((q == 2 ? 2 : 1) * nc * sizeof(double));
+  size_t pack_bytes = 0;
+  const int tail = tail_first(p, lv, nl, &pack_bytes);
+  const size_t o_pack = pl.take(pack_bytes);
   size_t o_part = pl.take(2 * kRedBlocks * sizeof(double));
   size_t o_scal = pl.take(16 * sizeof(double));
   size_t o_max = pl.take(8 * sizeof(unsigned long long));
@@ -316,6 +344,8 @@ size_t plan_workspace(const fvm_params& p, fvm_ctx* c) {
       for (int q = 0; q < 3; ++q) c->lbeta[l][q] = w + o_lbeta[l][q];
     }
     for (int q = 0; q < 3; ++q) c->cg[q] = w + o_cg[q];
+    c->tail = tail;
+    c->pack = pack_bytes ? w + o_pack : nullptr;
     c->partial = (double*)(w + o_part);
     c->scal = (double*)(w + o_scal);
     c->maxbits = (unsigned long long*)(w + o_max);
@@ -397,12 +427,6 @@ void hierarchy(fvm_ctx* c, T* x0, T* b0, T* const* beta0, MGLevel<T>* Ls) {
   }
 }
 
-template <typename T>
-void coarsen_betas(fvm_ctx* c, MGLevel<T>* Ls) {
-  for (int l = 0; l + 1 < c->nlev; ++l)
-    TIMED(c, FVM_K_BETA, 1, launch_beta_coarsen<T>(Ls[l], Ls[l + 1], c->stream));
-}
-
 // what the sweeps of one smoothing step fold in
 template <typename T>
 struct SweepFold {
@@ -453,20 +477,38 @@ int coarse_post(const fvm_ctx* c) {
   return c->prm.mg_coarse_sweeps > 0 ? c->prm.mg_coarse_sweeps : c->prm.mg_post;
 }
 
-// first level of the one-CTA coarse tail (at most kTailCells cells, not the
-// finest, at least one level above the coarsest), or -1
-int tail_start(const fvm_ctx* c) {
-  for (int l = 1; l < c->nlev - 1; ++l) {
-    const LevelShape& q = c->shp[l];
-    if ((long long)q.n[0] * q.n[1] * q.n[2] <= kTailCells)
-      return c->nlev - l <= kTailLevels ? l : -1;
+// the arguments of the tail that starts at level l = c->tail
+template <typename T>
+size_t tail_args(fvm_ctx* c, const MGLevel<T>* Ls, double rtol, TailArgs<T>& A) {
+  size_t smem = 0, pack = 0;
+  tail_layout<T>(Ls + c->tail, c->nlev - c->tail, A, &smem, &pack);
+  A.pack = c->pack;
+  A.rtol = rtol;
+  A.maxit = c->prm.coarse_maxit;
+  A.pre = coarse_pre(c);
+  A.post = coarse_post(c);
+  // at most 32 coarsest cells are solved by a packed inverse, unless the caller
+  // cuts the conjugate gradients short
+  const long long nc = Ls[c->nlev - 1].geo.N;
+  A.direct = c->pack && nc > 1 && nc <= 32 && A.maxit >= nc;
+  return smem;
+}
+
+// the face coefficients of every level, and the tail's packed form of them
+template <typename T>
+void coarsen_betas(fvm_ctx* c, MGLevel<T>* Ls) {
+  for (int l = 0; l + 1 < c->nlev; ++l)
+    TIMED(c, FVM_K_BETA, 1, launch_beta_coarsen<T>(Ls[l], Ls[l + 1], c->stream));
+  if (c->tail >= 0 && c->pack) {
+    TailArgs<T> A;
+    tail_args<T>(c, Ls, 0.0, A);
+    TIMED(c, FVM_K_BETA, 1, launch_tail_pack<T>(A, c->stream));
   }
-  return -1;
 }
 
 // V(pre, post) cycle: red-black sweeps before the coarse correction,
-// black-red after, CG on the coarsest level; the levels from tail_start()
-// down run in one kernel
+// black-red after, CG on the coarsest level; the levels from c->tail down
+// run in one kernel
 // How the finest level's x starts: as it is, at 0 (not yet zeroed), with the
 // first sweep already taken (by k_residual64 in the mixed form, or skipped
 // because it would repeat the previous cycle's last sweep), or with that skip
@@ -504,24 +546,16 @@ void vcycle(fvm_ctx* c, MGLevel<T>* Ls, int l, double coarse_rtol, int start = k
   cudaStream_t s = c->stream;
   const int pre = l == 0 ? c->prm.mg_pre : coarse_pre(c);
   const int post = l == 0 ? c->prm.mg_post : coarse_post(c);
-  const bool whole = l == tail_start(c) || l == c->nlev - 1;   // no sweeps of its own here
+  const bool whole = l == c->tail || l == c->nlev - 1;   // no sweeps of its own here
   const bool zero = start == kStartZero;
   if (zero && (whole || pre == 0))
     TIMED(c, FVM_K_MISC, 1, launch_zero<T>(Ls[l].x, Ls[l].geo.N, s));
   const bool fold_zero = zero && !whole && pre > 0;
   const bool fold_add = addp && !whole && post > 0;
-  if (l == tail_start(c)) {
+  if (l == c->tail) {
     TailArgs<T> A;
-    A.nl = c->nlev - l;
-    for (int q = 0; q < A.nl; ++q) A.L[q] = Ls[l + q];
-    A.r = (double*)c->cg[0];
-    A.d = (double*)c->cg[1];
-    A.Ad = (double*)c->cg[2];
-    A.rtol = coarse_rtol;
-    A.maxit = c->prm.coarse_maxit;
-    A.pre = coarse_pre(c);
-    A.post = coarse_post(c);
-    TIMED(c, FVM_K_COARSE_TAIL, 1, launch_coarse_tail<T>(A, s));
+    const size_t smem = tail_args<T>(c, Ls, coarse_rtol, A);
+    TIMED(c, FVM_K_COARSE_TAIL, 1, launch_tail<T>(A, smem, s));
   } else if (l == c->nlev - 1) {
     TIMED(c, FVM_K_COARSE_CG, 1, launch_coarse_cg<T>(Ls[l], (double*)c->cg[0], (double*)c->cg[1], (double*)c->cg[2],
                                                    coarse_rtol, c->prm.coarse_maxit, s));
@@ -537,7 +571,7 @@ void vcycle(fvm_ctx* c, MGLevel<T>* Ls, int l, double coarse_rtol, int start = k
     smooth<T>(c, Ls[l], l, pre, 0, fpre);
     // the next level's first sweep rides on the restriction when that level
     // sweeps on its own (not the tail, not the coarsest)
-    const bool swept = l + 1 != tail_start(c) && l + 1 != c->nlev - 1 && coarse_pre(c) > 0;
+    const bool swept = l + 1 != c->tail && l + 1 != c->nlev - 1 && coarse_pre(c) > 0;
     TIMED(c, l == 0 ? FVM_K_RESTRICT_FINE : FVM_K_RESTRICT_COARSE, 1,
           launch_residual_restrict<T>(Ls[l], Ls[l + 1], s, swept));
     vcycle<T>(c, Ls, l + 1, coarse_rtol, swept ? kStartFirstSwept : kStartAsIs);
@@ -1628,7 +1662,16 @@ size_t plan_noalloc(const fvm_params& p, fvm_ctx* c, char* base) {
   for (int q = 0; q < 3; ++q) o_cg[q] = pl.take((q == 2 ? 2 : 1) * nc * sizeof(double));
   size_t o_part = pl.take(2 * kRedBlocks * sizeof(double));
   size_t o_scal = pl.take(16 * sizeof(double));
+  // the tail's packed coefficients where they fit as well (else every cycle
+  // forms them from beta: no grid is refused for them)
+  size_t pack_bytes = 0;
+  const int tail = tail_first(p, lv, nl, &pack_bytes);
+  size_t o_pack = 0;
+  if (pl.off + pack_bytes <= kNoAllocScratchBytes) o_pack = pl.take(pack_bytes);
+  else pack_bytes = 0;
   if (c) {
+    c->tail = tail;
+    c->pack = pack_bytes ? base + o_pack : nullptr;
     c->b = (double*)(base + o_b);
     for (int q = 0; q < 3; ++q) c->beta0[q] = base + o_beta[q];
     c->e32 = mixed ? (float*)(base + o_e) : nullptr;

@@ -159,21 +159,49 @@ void launch_gs_zero(const MGLevel<T>& L, int colour, cudaStream_t s);
 void launch_gs_addp(const MGLevel<float>& L, int colour, double* p, cudaStream_t s);
 template <typename T>
 void launch_beta_coarsen(const MGLevel<T>& F, const MGLevel<T>& C, cudaStream_t s);
-// The coarse tail of a V-cycle (levels of at most kTailCells cells, the
-// coarsest solved by CG) in one CTA
-constexpr int kTailCells = 4096;
-constexpr int kTailLevels = 8;
+// The coarse tail of a V-cycle (fvm_tail.cu): the levels from the first one
+// that fits down to the coarsest, in one launch of one cluster of kTailCTAs
+// CTAs.
+constexpr int kTailCTAs = 16;
+constexpr int kTailLevels = 16;
+constexpr int kTailMaxCells = 32768;        // of the tail's first level
+constexpr int kTailSmem = 220 * 1024;       // shared memory of a CTA
+constexpr int kTailCells32 = 512, kTailCells64 = 256;   // cells a CTA should have (float, double)
+constexpr int kTailCgCells = 64, kTailCgSingle = 400;    // the same for the coarsest level's CG
 template <typename T>
-struct TailArgs {
-  int nl;                      // levels in the tail, the last one the coarsest
-  MGLevel<T> L[kTailLevels];
-  double *r, *d, *Ad;          // CG vectors (as launch_coarse_cg)
-  double rtol;
-  int maxit, pre, post;
+struct TailLevel {
+  int n[3], f[3];              // cells per axis, coarsening factor to the next level
+  int hx, pitch, rows;         // column pairs of a row, stored row length, rows (ny nz)
+  int rpc, nact, cap;          // rows per CTA, CTAs with rows, stored cells per CTA
+  int ox, ob, oa, otab;        // byte offsets in shared memory: x, b, coefficients, row table
+  int cb;                      // bytes of a CTA's coefficients
+  bool wall[3];
+  T w[3];                      // 1 / hd^2
+  const T* beta[3];
+  const T* b;                  // the first level's right-hand side and solution
+  T* x;
+  size_t opack;                // byte offset of the level's blocks in the packed coefficients
 };
 template <typename T>
-void launch_coarse_tail(const TailArgs<T>& A, cudaStream_t s);
-// CG vectors are double in both precisions (the coarsest level is small)
+struct TailArgs {
+  int nl;                      // levels, the last one the coarsest
+  TailLevel<T> L[kTailLevels];
+  int oscr, ocg, ored;         // byte offsets: fine residuals, CG vectors, reductions
+  const void* pack;            // coefficients of launch_tail_pack (null: formed from beta)
+  double rtol;
+  int maxit, pre, post;
+  bool direct;                 // the coarsest level by its packed inverse instead of CG
+};
+// lay out levels Ls[0 .. nl-1]; false when they do not fit.  smem: bytes per
+// CTA, pack: bytes of the packed coefficients
+template <typename T>
+bool tail_layout(const MGLevel<T>* Ls, int nl, TailArgs<T>& A, size_t* smem, size_t* pack);
+template <typename T>
+void launch_tail_pack(const TailArgs<T>& A, cudaStream_t s);
+template <typename T>
+void launch_tail(const TailArgs<T>& A, size_t smem, cudaStream_t s);
+// CG on a coarsest level too large for the tail, vectors in global memory
+// (double in both precisions)
 template <typename T>
 void launch_coarse_cg(const MGLevel<T>& L, double* r, double* d, double* Ad, double rtol,
                       int maxit, cudaStream_t s);

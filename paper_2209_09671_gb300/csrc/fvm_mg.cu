@@ -7,7 +7,8 @@
 //   k_gs_prolong        the first sweep after the correction with the prolongation folded in
 //   k_gs_zero, k_gs_addp the first sweep from x = 0 and the last one adding x to p (mixed form)
 //   k_beta_coarsen      coarse face beta = mean of the fine faces it covers
-//   k_coarse_cg         conjugate gradients on the coarsest level, one CTA
+//   k_coarse_cg         conjugate gradients on a coarsest level too large for the tail
+//                       of fvm_tail.cu, one CTA
 //   k_residual_norm2    ||b - L x||^2 partial sums
 //   k_residual64        mixed form: r = b - L p in double, stored as float
 // The paper names no linear solver; this is the reading used throughout the
@@ -503,153 +504,13 @@ __device__ void coarse_cg_block(const MGLevel<T>& L, double* __restrict__ r,
   for (int c = threadIdx.x; c < N; c += blockDim.x) L.x[c] = (T)(x[c] - xm);
 }
 
-// The coarsest-level CG of a single CTA is bound by the latency of every
-// iteration's dependent phases (operator, two reductions, updates); when the
-// level is small its vectors and face coefficients are kept in shared
-// memory instead of global memory (the same arithmetic in the same order).
-constexpr int kCgSmemCells = 640;
-struct CgSmem {
-  double v[4][kCgSmemCells];   // r, d, Ad, x
-  double beta[3][kCgSmemCells];
-};
-
-template <typename T>
-__device__ void coarse_cg_dispatch(const MGLevel<T>& L, double* r, double* dd, double* Ad,
-                                   double rtol, int maxit, double* sh, CgSmem& cs) {
-  const int N = (int)L.geo.N;
-  if (N > kCgSmemCells || sizeof(T) > sizeof(double)) {
-    coarse_cg_block(L, r, dd, Ad, rtol, maxit, sh);
-    return;
-  }
-  // face coefficients staged in the level's precision T; the operator then
-  // reads them through a copy of the level whose beta points to them
-  T* bs = reinterpret_cast<T*>(&cs.beta[0][0]);
-  MGLevel<T> S = L;
-  for (int q = 0; q < 3; ++q) {
-    S.beta[q] = bs + q * kCgSmemCells;
-    for (int c = threadIdx.x; c < N; c += blockDim.x) S.beta[q][c] = L.beta[q][c];
-  }
-  __syncthreads();
-  coarse_cg_block(S, cs.v[0], cs.v[1], cs.v[2], rtol, maxit, sh);
-}
-
 template <typename T>
 __global__ void __launch_bounds__(1024) k_coarse_cg(MGLevel<T> L, double* __restrict__ r,
                                                     double* __restrict__ dd,
                                                     double* __restrict__ Ad, double rtol,
                                                     int maxit) {
   __shared__ double sh[33];
-  __shared__ CgSmem cs;
-  coarse_cg_dispatch(L, r, dd, Ad, rtol, maxit, sh, cs);
-}
-
-// The coarse tail of a V-cycle in one CTA: levels small enough that a kernel
-// launch per sweep costs more than the sweep.  The same point updates as the
-// per-level kernels, in the same order of phases (pre-sweeps red first,
-// residual restriction, ..., CG on the coarsest level, ..., prolongation,
-// post-sweeps black first), separated by block barriers; within one colour
-// sweep (and within restriction and prolongation) the points are
-// independent, so the result equals that of the per-level kernels bit for bit.
-// one colour sweep of a tail level by the CTA: thread t takes the t-th cell
-// of the colour (rows of ceil(nx/2) such cells); the row and plane indices
-// come from float reciprocals, exact for the at most 4096 cells of a tail
-// level, instead of integer divisions
-template <typename T>
-__device__ __forceinline__ void tail_colour(const MGLevel<T>& L, int col) {
-  const Geo& g = L.geo;
-  const int hx = (g.n[0] + 1) >> 1;
-  const int half = hx * g.n[1] * g.n[2];
-  const float ihx = 1.0f / (float)hx, iny = 1.0f / (float)g.n[1];
-  for (int t = threadIdx.x; t < half; t += blockDim.x) {
-    const int q = (int)(((float)t + 0.5f) * ihx);   // row j + ny k
-    const int i2 = t - q * hx;
-    const int k = (int)(((float)q + 0.5f) * iny);
-    const int j = q - k * g.n[1];
-    const int i = 2 * i2 + ((col + j + k) & 1);
-    if (i < g.n[0]) gs_point(L, i, j, k);
-  }
-}
-
-template <typename T>
-__device__ void tail_body(const MGLevel<T>* Ls, int nl, double* r, double* d, double* Ad,
-                          double rtol, int maxit, int pre, int post, double* sh, CgSmem& cs) {
-  const int last = nl - 1;
-  for (int l = 0; l < last; ++l) {
-    const MGLevel<T>& L = Ls[l];
-    for (int it = 0; it < pre; ++it)
-      for (int col = 0; col < 2; ++col) {
-        tail_colour(L, col);
-        __syncthreads();
-      }
-    for (int cc = threadIdx.x; cc < (int)Ls[l + 1].geo.N; cc += blockDim.x)
-      restrict_point(L, Ls[l + 1], cc);
-    __syncthreads();
-  }
-  coarse_cg_dispatch(Ls[last], r, d, Ad, rtol, maxit, sh, cs);
-  __syncthreads();
-  for (int l = last - 1; l >= 0; --l) {
-    const MGLevel<T>& L = Ls[l];
-    const Geo& g = L.geo;
-    for (int c = threadIdx.x; c < (int)g.N; c += blockDim.x) prolong_point(L, Ls[l + 1], c);
-    __syncthreads();
-    for (int it = 0; it < post; ++it)
-      for (int col = 0; col < 2; ++col) {
-        tail_colour(L, 1 - col);
-        __syncthreads();
-      }
-  }
-}
-
-// staged: the tail levels' x, b and betas are copied into dynamic shared
-// memory first (x and b of the top level, the betas of every level; the
-// lower levels' x and b are set by the restrictions inside the tail), the
-// tail runs on those copies, and the top level's x is copied back for the
-// prolongation.  The arithmetic is the same as on the global arrays; only the
-// latency of each sweep's loads changes.
-template <typename T>
-__global__ void __launch_bounds__(1024) k_coarse_tail(TailArgs<T> A, int staged) {
-  __shared__ double sh[33];
-  __shared__ CgSmem cs;
-  extern __shared__ __align__(16) unsigned char tail_smem[];
-  if (!staged) {
-    tail_body(A.L, A.nl, A.r, A.d, A.Ad, A.rtol, A.maxit, A.pre, A.post, sh, cs);
-    return;
-  }
-  MGLevel<T> L[kTailLevels];
-  T* base = reinterpret_cast<T*>(tail_smem);
-  for (int q = 0; q < A.nl; ++q) {
-    L[q] = A.L[q];
-    const int n = (int)L[q].geo.N;
-    L[q].x = base;
-    L[q].b = base + n;
-    for (int d = 0; d < 3; ++d) L[q].beta[d] = base + (2 + d) * n;
-    base += 5 * n;
-    for (int c = threadIdx.x; c < n; c += blockDim.x) {
-      for (int d = 0; d < 3; ++d) L[q].beta[d][c] = A.L[q].beta[d][c];
-      if (q == 0) {
-        L[0].x[c] = A.L[0].x[c];
-        L[0].b[c] = A.L[0].b[c];
-      }
-    }
-  }
-  __syncthreads();
-  tail_body(L, A.nl, A.r, A.d, A.Ad, A.rtol, A.maxit, A.pre, A.post, sh, cs);
-  __syncthreads();
-  for (int c = threadIdx.x; c < (int)L[0].geo.N; c += blockDim.x) A.L[0].x[c] = L[0].x[c];
-}
-
-template <typename T>
-void launch_coarse_tail(const TailArgs<T>& A, cudaStream_t s) {
-  // stage the levels of the FP64 form when they fit beside the kernel's
-  // static shared memory (the float tail was slower staged, 112 -> 124 us per
-  // call at 256^3, and reads the global arrays)
-  size_t bytes = 0;
-  for (int q = 0; q < A.nl; ++q) bytes += 5 * (size_t)A.L[q].geo.N * sizeof(T);
-  const size_t limit = 227 * 1024 - sizeof(CgSmem) - 33 * sizeof(double) - 1024;
-  const bool staged = sizeof(T) == sizeof(double) && bytes <= limit;
-  if (staged)
-    cudaFuncSetAttribute(k_coarse_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  k_coarse_tail<T><<<1, 1024, staged ? bytes : 0, s>>>(A, staged ? 1 : 0);
+  coarse_cg_block(L, r, dd, Ad, rtol, maxit, sh);
 }
 
 template <typename T>
@@ -840,7 +701,6 @@ void launch_ctl_store(const SolveCtl* ctl, SolveCtl* rec, int* sticky, cudaStrea
   template void launch_gs_prolong<T>(const MGLevel<T>&, const MGLevel<T>&, int, cudaStream_t); \
   template void launch_gs_zero<T>(const MGLevel<T>&, int, cudaStream_t);                      \
   template void launch_beta_coarsen<T>(const MGLevel<T>&, const MGLevel<T>&, cudaStream_t);  \
-  template void launch_coarse_tail<T>(const TailArgs<T>&, cudaStream_t);                     \
   template void launch_coarse_cg<T>(const MGLevel<T>&, double*, double*, double*, double,  \
                                     int, cudaStream_t);                                      \
   template void launch_residual_norm2<T>(const MGLevel<T>&, double*, double*, cudaStream_t);

@@ -1,0 +1,721 @@
+// The coarse levels of a V-cycle in one launch of one thread-block cluster.
+//
+// A coarse level is too small to fill the GPU: a colour sweep of 32^3 cells
+// takes 2.6 us as a launch of its own (almost all of it launch and drain), and
+// a V-cycle makes a dozen of them per level.  On one CTA the same levels
+// are bound by that SM instead.  Here kTailCTAs CTAs of one cluster keep every
+// level of the tail in their shared memory, each a run of rows of it; a sweep
+// reads the rows of other CTAs through distributed shared memory and ends
+// with a cluster barrier (475 clocks; a remote load is 240).  Levels small
+// enough for one CTA run on CTA 0 between block barriers (44 clocks) while the
+// others wait.
+//
+// Per cell a level holds x, b, the six face coefficients beta / h_d^2 and the
+// reciprocal of their sum (7 numbers prepared once per solve by k_tail_pack,
+// so that a sweep divides nothing), the coarsest level its coefficients and
+// conjugate-gradient vectors in double.  A row is stored with its even
+// columns first, then the odd ones: the cells of one colour are consecutive
+// and their loads free of bank conflicts.
+//
+// Measured per V-cycle against the levels of at most 4096 cells on one CTA and
+// the larger ones as launches: 256^3 float (32^3 cells and below) 51 against
+// 134 + 45 us, 128^3 double 105 against 344 + 60 us, the 64^2 double drop 53
+// against 156 us; bound by the barriers and the latencies between them.
+#include "fvm_device.cuh"
+
+namespace fvm {
+
+namespace {
+
+constexpr int kTailThreads = 512;
+
+__device__ __forceinline__ unsigned smem_u32(const void* p) {
+  return (unsigned)__cvta_generic_to_shared(p);
+}
+// address of the same shared-memory location in CTA `rank` of the cluster
+__device__ __forceinline__ unsigned map_rank(unsigned a, unsigned rank) {
+  unsigned r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void ld_cl(unsigned a, float& v) {
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a));
+}
+__device__ __forceinline__ void ld_cl(unsigned a, double& v) {
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a));
+}
+__device__ __forceinline__ void st_cl(unsigned a, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
+                   : "memory");
+}
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+
+// what a CTA knows of one level
+template <typename T>
+struct View {
+  const TailLevel<T>& L;
+  char* sm;
+  int rank, nrows;      // rows of this CTA
+  __device__ View(const TailLevel<T>& l, char* s, int r) : L(l), sm(s), rank(r) {
+    const int r0 = r * l.rpc;
+    nrows = r0 >= l.rows ? 0 : (l.rows - r0 < l.rpc ? l.rows - r0 : l.rpc);
+  }
+  __device__ T* x() const { return reinterpret_cast<T*>(sm + L.ox); }
+  __device__ T* b() const { return reinterpret_cast<T*>(sm + L.ob); }
+  template <typename C>
+  __device__ C* a() const { return reinterpret_cast<C*>(sm + L.oa); }
+  __device__ int4* tab() const { return reinterpret_cast<int4*>(sm + L.otab); }
+};
+
+// quotient t / d for 0 <= t < 2^20 (id = 1 / d)
+__device__ __forceinline__ int quot(int t, float id) { return (int)(((float)t + 0.5f) * id); }
+
+// position of column i in a stored row: even columns, then odd ones
+__device__ __forceinline__ int row_pos(int i, int hx) { return (i & 1) * hx + (i >> 1); }
+
+// shared-cluster address of row R of an array at byte offset `off` (elements
+// of `esize` bytes)
+template <typename T>
+__device__ __forceinline__ unsigned row_addr(const TailLevel<T>& L, unsigned base, int off, int R,
+                                             int esize) {
+  const int rk = quot(R, 1.0f / (float)L.rpc);
+  return map_rank(base + off + (R - rk * L.rpc) * L.pitch * esize, rk);
+}
+
+// the six coefficients of cell (i, row R) and the reciprocal of their sum
+template <typename T, typename C>
+__device__ __forceinline__ C cell_coefs(const TailLevel<T>& L, int i, int R, C* a) {
+  const int nx = L.n[0], ny = L.n[1], nz = L.n[2];
+  const int k = quot(R, 1.0f / (float)ny), j = R - k * ny;
+  const int c = R * nx + i;
+  const int idx[3] = {i, j, k}, st[3] = {1, nx, nx * ny};
+  C den = C(0);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    a[2 * d] = a[2 * d + 1] = C(0);
+    const int n = L.n[d];
+    if (n == 1) continue;
+    const bool last = idx[d] == n - 1;
+    const int hi = last ? c - (n - 1) * st[d] : c + st[d];
+    a[2 * d] = (C)L.beta[d][c] * (C)L.w[d];
+    a[2 * d + 1] = (last && L.wall[d]) ? C(0) : (C)L.beta[d][hi] * (C)L.w[d];
+    den += a[2 * d] + a[2 * d + 1];
+  }
+  return C(1) / den;
+}
+
+// fill the coefficient block of CTA `rank` (layout of shared memory and of
+// the packed copy in global memory)
+template <typename T>
+__device__ void fill_coefs(const TailLevel<T>& L, bool coarsest, void* dst, int rank, int tid,
+                           int nthr) {
+  const int r0 = rank * L.rpc;
+  const int nrows = max(0, min(L.rpc, L.rows - r0));
+  for (int t = tid; t < nrows * L.pitch; t += nthr) {
+    const int q = quot(t, 1.0f / (float)L.pitch), pos = t - q * L.pitch;
+    const int i = pos < L.hx ? 2 * pos : 2 * (pos - L.hx) + 1;
+    if (i >= L.n[0]) continue;
+    if (coarsest) {
+      double a[6];
+      cell_coefs<T, double>(L, i, r0 + q, a);
+      for (int m = 0; m < 6; ++m) ((double*)dst)[m * L.cap + t] = a[m];
+    } else {
+      T a[6];
+      const T inv = cell_coefs<T, T>(L, i, r0 + q, a);
+      for (int m = 0; m < 6; ++m) ((T*)dst)[m * L.cap + t] = a[m];
+      ((T*)dst)[6 * L.cap + t] = inv;
+    }
+  }
+}
+
+// G = (L + s 1 1^T / N)^-1 on a coarsest level of N <= 32 cells, s the mean
+// diagonal: Gauss-Jordan without pivoting (the matrix is symmetric and positive
+// definite: L has the constants as its only null vectors), by one block
+template <typename T>
+__device__ void coarsest_inverse(const TailLevel<T>& L, double* __restrict__ G) {
+  __shared__ double M[32][33];
+  __shared__ double diag[32];
+  const int N = L.rows * L.n[0], nx = L.n[0], ny = L.n[1];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int r = w; r < N; r += nw)
+    if (lane < N) M[r][lane] = 0.0;
+  __syncthreads();
+  if (w == 0 && lane < N) {
+    const int R = lane / nx, i = lane - R * nx, k = R / ny, j = R - k * ny;
+    double a[6], dg = 0.0;
+    cell_coefs<T, double>(L, i, R, a);
+    const int idx[3] = {i, j, k}, st[3] = {1, nx, nx * ny};
+    for (int d = 0; d < 3; ++d) {
+      const int n = L.n[d];
+      if (n == 1) continue;
+      const int lo = idx[d] == 0 ? lane + (n - 1) * st[d] : lane - st[d];
+      const int hi = idx[d] == n - 1 ? lane - (n - 1) * st[d] : lane + st[d];
+      M[lane][lo] -= a[2 * d];
+      M[lane][hi] -= a[2 * d + 1];
+      dg += a[2 * d] + a[2 * d + 1];
+    }
+    M[lane][lane] += dg;
+    diag[lane] = dg;
+  }
+  __syncthreads();
+  double s = 0.0;
+  for (int q = 0; q < N; ++q) s += diag[q];
+  s /= (double)N * (double)N;
+  for (int r = w; r < N; r += nw)
+    if (lane < N) M[r][lane] += s;
+  __syncthreads();
+  for (int p = 0; p < N; ++p) {
+    const double ip = 1.0 / M[p][p];
+    const double mp = lane < N ? M[p][lane] : 0.0;
+    const double rp = lane == p ? ip : mp * ip;      // the scaled pivot row
+    double f[4], v[4];
+    for (int q = 0; q < 4; ++q) {
+      const int r = w + q * nw;
+      if (r < N && lane < N) {
+        f[q] = M[r][p];
+        v[q] = M[r][lane];
+      }
+    }
+    __syncthreads();
+    for (int q = 0; q < 4; ++q) {
+      const int r = w + q * nw;
+      if (r < N && lane < N) {
+        if (r == p) M[r][lane] = rp;
+        else M[r][lane] = lane == p ? -f[q] * ip : fma(-f[q], rp, v[q]);
+      }
+    }
+    __syncthreads();
+  }
+  for (int r = w; r < N; r += nw)
+    if (lane < N) G[r * N + lane] = M[r][lane];
+}
+
+// one Gauss-Seidel sweep of a colour over the CTA's rows
+template <typename T>
+__device__ __forceinline__ void sweep(const View<T>& V, int col) {
+  const TailLevel<T>& L = V.L;
+  T* x = V.x();
+  const T* b = V.b();
+  const T* a = V.template a<T>();
+  const int hx = L.hx, nx = L.n[0], cap = L.cap;
+  const float ihx = 1.0f / (float)hx;
+  for (int t = threadIdx.x; t < V.nrows * hx; t += kTailThreads) {
+    const int q = quot(t, ihx), i2 = t - q * hx;
+    const int4 ra = V.tab()[2 * q];
+    const int s = (col + V.tab()[2 * q + 1].y) & 1;
+    const int i = 2 * i2 + s;
+    if (i >= nx) continue;
+    const int row = q * L.pitch, p = s * hx + i2, c = row + p;
+    T ym, yp, zm, zp;
+    const unsigned o = p * (unsigned)sizeof(T);
+    ld_cl(ra.x + o, ym);
+    ld_cl(ra.y + o, yp);
+    ld_cl(ra.z + o, zm);
+    ld_cl(ra.w + o, zp);
+    const T xm = x[row + row_pos(i == 0 ? nx - 1 : i - 1, hx)];
+    const T xp = x[row + row_pos(i == nx - 1 ? 0 : i + 1, hx)];
+    T num = b[c];
+    num += a[c] * xm + a[cap + c] * xp;
+    num += a[2 * cap + c] * ym + a[3 * cap + c] * yp;
+    num += a[4 * cap + c] * zm + a[5 * cap + c] * zp;
+    x[c] = num * a[6 * cap + c];
+  }
+}
+
+// r = b - L x over the CTA's rows
+template <typename T>
+__device__ __forceinline__ void residual(const View<T>& V, T* r) {
+  const TailLevel<T>& L = V.L;
+  const T* x = V.x();
+  const T* b = V.b();
+  const T* a = V.template a<T>();
+  const int hx = L.hx, nx = L.n[0], cap = L.cap;
+  const float ip = 1.0f / (float)L.pitch;
+  for (int t = threadIdx.x; t < V.nrows * L.pitch; t += kTailThreads) {
+    const int q = quot(t, ip), p = t - q * L.pitch;
+    const int i = p < hx ? 2 * p : 2 * (p - hx) + 1;
+    if (i >= nx) continue;
+    const int4 ra = V.tab()[2 * q];
+    const int row = q * L.pitch;
+    T ym, yp, zm, zp;
+    const unsigned o = p * (unsigned)sizeof(T);
+    ld_cl(ra.x + o, ym);
+    ld_cl(ra.y + o, yp);
+    ld_cl(ra.z + o, zm);
+    ld_cl(ra.w + o, zp);
+    const T xc = x[t];
+    const T xm = x[row + row_pos(i == 0 ? nx - 1 : i - 1, hx)];
+    const T xp = x[row + row_pos(i == nx - 1 ? 0 : i + 1, hx)];
+    T out = a[t] * (xc - xm) + a[cap + t] * (xc - xp);
+    out += a[2 * cap + t] * (xc - ym) + a[3 * cap + t] * (xc - yp);
+    out += a[4 * cap + t] * (xc - zm) + a[5 * cap + t] * (xc - zp);
+    r[t] = b[t] - out;
+  }
+}
+
+// x from a start of 0 with the first colour-0 sweep taken (it needs only b)
+template <typename T>
+__device__ __forceinline__ T first_x(const View<T>& V, int c, int i, int parity, T b, bool sweep0) {
+  return sweep0 && ((i + parity) & 1) == 0 ? b * V.template a<T>()[6 * V.L.cap + c] : T(0);
+}
+
+// b of the coarse level = mean over the children of the fine residual
+template <typename T>
+__device__ __forceinline__ void restrict_rows(const View<T>& F, const View<T>& C, unsigned base,
+                                              int oscr, bool coarsest, bool sweep0) {
+  const TailLevel<T>& L = C.L;
+  const int fx = F.L.f[0], fy = F.L.f[1], fz = F.L.f[2];
+  const T scale = T(1) / (T)(fx * fy * fz);   // a power of two
+  const float ip = 1.0f / (float)L.pitch, iny = 1.0f / (float)L.n[1];
+  for (int t = threadIdx.x; t < C.nrows * L.pitch; t += kTailThreads) {
+    const int q = quot(t, ip), p = t - q * L.pitch;
+    const int I = p < L.hx ? 2 * p : 2 * (p - L.hx) + 1;
+    if (I >= L.n[0]) continue;
+    const int R = C.rank * L.rpc + q;
+    const int K = quot(R, iny), J = R - K * L.n[1];
+    T acc = T(0);
+    for (int dz = 0; dz < fz; ++dz)
+      for (int dy = 0; dy < fy; ++dy) {
+        const unsigned ra = row_addr(F.L, base, oscr, (K * fz + dz) * F.L.n[1] + J * fy + dy,
+                                     (int)sizeof(T));
+        for (int dx = 0; dx < fx; ++dx) {
+          T v;
+          ld_cl(ra + row_pos(I * fx + dx, F.L.hx) * (unsigned)sizeof(T), v);
+          acc += v;
+        }
+      }
+    const T b = acc * scale;
+    C.b()[t] = b;
+    if (!coarsest) C.x()[t] = first_x(C, t, I, J + K, b, sweep0);
+  }
+}
+
+// x += the coarse correction of the parent cell
+template <typename T>
+__device__ __forceinline__ void prolong_rows(const View<T>& F, const TailLevel<T>& C) {
+  const TailLevel<T>& L = F.L;
+  const int hx = L.hx;
+  const float ip = 1.0f / (float)L.pitch;
+  for (int t = threadIdx.x; t < F.nrows * L.pitch; t += kTailThreads) {
+    const int q = quot(t, ip), p = t - q * L.pitch;
+    const int i = p < hx ? 2 * p : 2 * (p - hx) + 1;
+    if (i >= L.n[0]) continue;
+    const unsigned pa = (unsigned)F.tab()[2 * q + 1].x;
+    T v;
+    ld_cl(pa + row_pos(L.f[0] == 2 ? i >> 1 : i, C.hx) * (unsigned)sizeof(T), v);
+    F.x()[t] += v;
+  }
+}
+
+__device__ __forceinline__ double warp_sum_all(double v, int steps) {
+  for (int o = 1 << (steps - 1); steps > 0; o >>= 1, --steps) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Sums over the cells of a level spread over `nact` CTAs (CTA 0 alone when nact
+// is 1, else the whole cluster takes part), in a fixed order.  The first warp
+// adds the threads' values from shared memory and works out the scalars of
+// the iteration: the FP64 pipe of an SM does 2 lanes a clock, so shuffling,
+// dividing or taking roots in every warp keeps it busy for thousands of clocks
+// (25 x 25 cells: 1160 instead of 870 us per V-cycle).
+struct Reduce {
+  double* vals;     // kTailThreads
+  double* slots;    // 2 sets of kTailCTAs, written by the other CTAs
+  double* out;      // the scalar handed to every thread
+  unsigned base_slots;
+  int nact, rank, used;   // used: threads of this CTA with a value
+  int phase;
+  // the sum of v over all cells goes through `f` in warp 0 (the same numbers
+  // in every CTA); every thread gets f's value
+  template <typename F>
+  __device__ __forceinline__ double run(double v, F f) {
+    const int tid = threadIdx.x;
+    if (tid < used) vals[tid] = v;
+    __syncthreads();
+    if (nact == 1) {
+      if (tid < 32) {
+        double s = 0.0;
+        for (int q = tid; q < used; q += 32) s += vals[q];
+        s = f(warp_sum_all(s, used > 16 ? 5 : (used > 8 ? 4 : 3)));
+        if (tid == 0) *out = s;
+      }
+    } else {
+      const int set = (phase++ & 1) * kTailCTAs;
+      if (tid < 32) {
+        double s = 0.0;
+        for (int q = tid; q < used; q += 32) s += vals[q];
+        s = warp_sum_all(s, used > 16 ? 5 : (used > 8 ? 4 : 3));
+        if (tid < kTailCTAs) st_cl(map_rank(base_slots + (set + rank) * 8, tid), s);
+      }
+      cluster_sync();
+      if (tid < 32) {
+        double s = f(warp_sum_all(tid < nact ? slots[set + tid] : 0.0, 4));
+        if (tid == 0) *out = s;
+      }
+    }
+    __syncthreads();
+    return *out;   // (rewritten only after the next call's first barrier)
+  }
+};
+
+// conjugate gradients on the coarsest level: mean-free right-hand side,
+// x0 = 0, stop at ||r|| <= rtol ||b|| or on breakdown, mean-free result; the
+// vectors are double in both precisions
+template <typename T>
+__device__ void coarsest_cg(const View<T>& V, const TailArgs<T>& A, Reduce& red) {
+  const TailLevel<T>& L = V.L;
+  const int cap = L.cap, hx = L.hx, nx = L.n[0];
+  const double* a = V.template a<double>();
+  double* d = reinterpret_cast<double*>(V.sm + A.ocg);
+  double *r = d + cap, *x = r + cap, *Ad = x + cap;
+  const int nc = V.nrows * L.pitch;
+  const float ip = 1.0f / (float)L.pitch;
+  const double N = (double)L.rows * nx;
+  // columns beyond nx in a padded row hold 0 in every vector
+  auto column = [&](int t) {
+    const int q = quot(t, ip), p = t - q * L.pitch;
+    return p < hx ? 2 * p : 2 * (p - hx) + 1;
+  };
+  double acc = 0.0;
+  for (int t = threadIdx.x; t < nc; t += kTailThreads)
+    if (column(t) < nx) acc += (double)V.b()[t];
+  const double mean = red.run(acc, [&](double s) { return s / N; });
+  acc = 0.0;
+  for (int t = threadIdx.x; t < nc; t += kTailThreads) {
+    const double v = column(t) < nx ? (double)V.b()[t] - mean : 0.0;
+    r[t] = d[t] = v;
+    x[t] = 0.0;
+    acc += v * v;
+  }
+  // rr and the stopping threshold live in warp 0; (the barrier also publishes d)
+  double rr = 0.0, stop = 0.0;   // ||r||^2 and its threshold
+  double go = red.run(acc, [&](double s) {
+    rr = s;
+    stop = A.rtol * A.rtol * s;
+    return s != 0.0 && !(s <= stop) ? 1.0 : 0.0;
+  });
+  for (int it = 0; it < A.maxit && go != 0.0; ++it) {
+    acc = 0.0;
+    for (int t = threadIdx.x; t < nc; t += kTailThreads) {
+      const int q = quot(t, ip), p = t - q * L.pitch;
+      const int i = p < hx ? 2 * p : 2 * (p - hx) + 1;
+      if (i >= nx) continue;
+      const int4 ra = V.tab()[2 * q];
+      const int row = q * L.pitch;
+      const unsigned o = p * 8u;
+      const double dc = d[t];
+      double v0, v1, v2, v3;
+      ld_cl(ra.x + o, v0);
+      ld_cl(ra.y + o, v1);
+      ld_cl(ra.z + o, v2);
+      ld_cl(ra.w + o, v3);
+      // an axis of one cell has coefficients 0; three short chains, as an FP64
+      // operation takes 63 clocks from issue to result
+      double ox = a[t] * (dc - d[row + row_pos(i == 0 ? nx - 1 : i - 1, hx)]);
+      double oy = a[2 * cap + t] * (dc - v0);
+      double oz = 0.0;
+      ox = fma(a[cap + t], dc - d[row + row_pos(i == nx - 1 ? 0 : i + 1, hx)], ox);
+      oy = fma(a[3 * cap + t], dc - v1, oy);
+      if (L.n[2] > 1) {
+        oz = a[4 * cap + t] * (dc - v2);
+        oz = fma(a[5 * cap + t], dc - v3, oz);
+      }
+      const double out = (ox + oy) + oz;
+      Ad[t] = out;
+      acc = fma(dc, out, acc);
+    }
+    // step length; 0 on breakdown (exhausted direction or rounding)
+    const double al = red.run(acc, [&](double s) { return s > 0.0 ? rr / s : 0.0; });
+    if (al == 0.0) break;
+    acc = 0.0;
+    for (int t = threadIdx.x; t < nc; t += kTailThreads) {
+      if (column(t) >= nx) continue;
+      x[t] = fma(al, d[t], x[t]);
+      const double v = fma(-al, Ad[t], r[t]);
+      r[t] = v;
+      acc = fma(v, v, acc);
+    }
+    // direction update, negative when ||r|| has reached the threshold
+    const double beta = red.run(acc, [&](double s) {
+      const double q = s / rr;
+      rr = s;
+      return s <= stop ? -1.0 : q;
+    });
+    if (beta < 0.0) break;
+    for (int t = threadIdx.x; t < nc; t += kTailThreads) d[t] = fma(beta, d[t], r[t]);
+    if (red.nact > 1) cluster_sync();
+    else __syncthreads();
+  }
+  acc = 0.0;
+  for (int t = threadIdx.x; t < nc; t += kTailThreads) acc += x[t];
+  const double xm = red.run(acc, [&](double s) { return s / N; });
+  for (int t = threadIdx.x; t < nc; t += kTailThreads) V.x()[t] = (T)(x[t] - xm);
+}
+
+// The coarsest level of at most 32 cells: x = G (b - mean b) with the inverse
+// G of L + s 1 1^T / N formed once per solve (coarsest_inverse).  On mean-free
+// right-hand sides that is the mean-free solution of L x = b to rounding,
+// where conjugate gradients would run their iterations' dependent reductions,
+// divisions and roots in every cycle.  One lane per cell.
+template <typename T>
+__device__ void coarsest_direct(const View<T>& V) {
+  const TailLevel<T>& L = V.L;
+  const int N = L.rows * L.n[0], lane = threadIdx.x;
+  if (lane >= 32) return;
+  const double* G = V.template a<double>();
+  const int q = quot(lane, 1.0f / (float)L.n[0]), c = q * L.pitch + row_pos(lane - q * L.n[0], L.hx);
+  double b = lane < N ? (double)V.b()[c] : 0.0;
+  const double mean = warp_sum_all(b, 5) / (double)N;
+  b = lane < N ? b - mean : 0.0;
+  double s0 = 0.0, s1 = 0.0;
+  for (int m = 0; m < N; m += 2) {
+    const double b0 = __shfl_sync(0xffffffffu, b, m), b1 = __shfl_sync(0xffffffffu, b, (m + 1) & 31);
+    if (lane < N) {
+      s0 = fma(G[m * N + lane], b0, s0);
+      if (m + 1 < N) s1 = fma(G[(m + 1) * N + lane], b1, s1);
+    }
+  }
+  if (lane < N) V.x()[c] = (T)(s0 + s1);
+}
+
+// row tables: addresses of the rows beside each own row (the array a sweep or
+// the conjugate gradients read there), the parent row, the row's parity
+template <typename T>
+__device__ void fill_table(const TailArgs<T>& A, int l, char* sm, unsigned base, int rank) {
+  const TailLevel<T>& L = A.L[l];
+  const View<T> V(L, sm, rank);
+  const bool cg = l == A.nl - 1;
+  const int off = cg ? A.ocg : L.ox, es = cg ? 8 : (int)sizeof(T);
+  const int ny = L.n[1], nz = L.n[2];
+  for (int q = threadIdx.x; q < V.nrows; q += kTailThreads) {
+    const int R = rank * L.rpc + q;
+    const int k = quot(R, 1.0f / (float)ny), j = R - k * ny;
+    int4 ra, rb;
+    ra.x = (int)row_addr(L, base, off, k * ny + (j == 0 ? ny - 1 : j - 1), es);
+    ra.y = (int)row_addr(L, base, off, k * ny + (j == ny - 1 ? 0 : j + 1), es);
+    ra.z = (int)row_addr(L, base, off, (k == 0 ? nz - 1 : k - 1) * ny + j, es);
+    ra.w = (int)row_addr(L, base, off, (k == nz - 1 ? 0 : k + 1) * ny + j, es);
+    rb.x = rb.z = rb.w = 0;
+    rb.y = (j + k) & 1;
+    if (!cg) {
+      const TailLevel<T>& C = A.L[l + 1];
+      rb.x = (int)row_addr(C, base, C.ox, (L.f[2] == 2 ? k >> 1 : k) * C.n[1] + (L.f[1] == 2 ? j >> 1 : j),
+                           (int)sizeof(T));
+    }
+    V.tab()[2 * q] = ra;
+    V.tab()[2 * q + 1] = rb;
+  }
+}
+
+}  // namespace
+
+template <typename T>
+__global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ TailArgs<T> A) {
+  extern __shared__ __align__(16) char sm[];
+  const int rank = (int)cluster_rank();
+  const unsigned base = smem_u32(sm);
+  const int last = A.nl - 1;
+  // coefficients: the packed copy, or from the betas
+  for (int l = 0; l <= last; ++l) {
+    const TailLevel<T>& L = A.L[l];
+    if (rank >= L.nact) continue;
+    const int bytes = L.cb;
+    if (A.pack) {
+      const int4* src = reinterpret_cast<const int4*>((const char*)A.pack + L.opack + (size_t)rank * bytes);
+      int4* dst = reinterpret_cast<int4*>(sm + L.oa);
+      for (int t = threadIdx.x; t < bytes / 16; t += kTailThreads) dst[t] = __ldg(src + t);
+    } else {
+      fill_coefs(L, l == last, sm + L.oa, rank, threadIdx.x, kTailThreads);
+    }
+    fill_table(A, l, sm, base, rank);
+  }
+  Reduce red;
+  red.vals = reinterpret_cast<double*>(sm + A.ored);
+  red.slots = red.vals + kTailThreads;
+  red.out = red.slots + 2 * kTailCTAs;
+  red.base_slots = base + A.ored + kTailThreads * 8;
+  red.nact = A.L[last].nact;
+  red.rank = rank;
+  red.phase = 0;
+  red.used = min(View<T>(A.L[last], sm, rank).nrows * A.L[last].pitch, kTailThreads);
+  __syncthreads();
+  {
+    // the top level's right-hand side; x starts at 0
+    const View<T> V(A.L[0], sm, rank);
+    const TailLevel<T>& L = V.L;
+    const float ip = 1.0f / (float)L.pitch;
+    for (int t = threadIdx.x; t < V.nrows * L.pitch; t += kTailThreads) {
+      const int q = quot(t, ip), p = t - q * L.pitch;
+      const int i = p < L.hx ? 2 * p : 2 * (p - L.hx) + 1;
+      if (i >= L.n[0]) continue;
+      const T b = __ldg(L.b + (rank * L.rpc + q) * L.n[0] + i);
+      V.b()[t] = b;
+      if (last > 0) V.x()[t] = first_x(V, t, i, V.tab()[2 * q + 1].y, b, A.pre > 0);
+    }
+  }
+  cluster_sync();
+  int single = 0;   // first level that CTA 0 holds alone
+  while (single <= last && A.L[single].nact > 1) ++single;
+  auto sync = [&](int l) {
+    if (l < single) cluster_sync();
+    else __syncthreads();
+  };
+  T* scr = reinterpret_cast<T*>(sm + A.oscr);
+  for (int l = 0; l < last; ++l) {
+    if (l >= single && rank) break;
+    const View<T> V(A.L[l], sm, rank);
+    for (int h = 1; h < 2 * A.pre; ++h) {   // the first half-sweep came with b
+      sweep(V, h & 1);
+      sync(l);
+    }
+    residual(V, scr);
+    sync(l);
+    restrict_rows(V, View<T>(A.L[l + 1], sm, rank), base, A.oscr, l + 1 == last, A.pre > 0);
+    sync(l);
+  }
+  if (last < single || rank == 0) {
+    const View<T> V(A.L[last], sm, rank);
+    if (A.direct) coarsest_direct(V);
+    else coarsest_cg(V, A, red);
+  }
+  for (int l = last - 1; l >= 0; --l) {
+    if (l >= single && rank) continue;
+    const View<T> V(A.L[l], sm, rank);
+    sync(l);
+    prolong_rows(V, A.L[l + 1]);
+    sync(l);
+    for (int h = 0; h < 2 * A.post; ++h) {
+      sweep(V, 1 - (h & 1));
+      sync(l);
+    }
+  }
+  if (last == 0) __syncthreads();
+  {
+    const View<T> V(A.L[0], sm, rank);
+    const TailLevel<T>& L = V.L;
+    const float in = 1.0f / (float)L.n[0];
+    for (int t = threadIdx.x; t < V.nrows * L.n[0]; t += kTailThreads) {
+      const int q = quot(t, in), i = t - q * L.n[0];
+      L.x[(rank * L.rpc) * L.n[0] + t] = V.x()[q * L.pitch + row_pos(i, L.hx)];
+    }
+  }
+}
+
+// the coefficient blocks of every level and CTA, once per solve
+template <typename T>
+__global__ void k_tail_pack(const __grid_constant__ TailArgs<T> A) {
+  const int l = blockIdx.y, rank = blockIdx.x;
+  const TailLevel<T>& L = A.L[l];
+  if (rank >= L.nact) return;
+  const bool coarsest = l == A.nl - 1;
+  char* dst = (char*)A.pack + L.opack + (size_t)rank * L.cb;
+  if (coarsest && A.direct) {
+    if (blockIdx.z == 0) coarsest_inverse(L, (double*)dst);
+    return;
+  }
+  fill_coefs(L, coarsest, dst, rank, threadIdx.x + blockIdx.z * blockDim.x,
+             blockDim.x * gridDim.z);
+}
+
+// Layout of a tail that starts at level Ls[0] with nl levels; false when it
+// does not fit.  The cells a CTA should have: enough that a sweep's work is
+// no smaller than the barrier that ends it.
+template <typename T>
+bool tail_layout(const MGLevel<T>* Ls, int nl, TailArgs<T>& A, size_t* smem, size_t* pack) {
+  if (nl < 1 || nl > kTailLevels) return false;
+  A.nl = nl;
+  int off = 0;
+  size_t po = 0;
+  auto take = [&](size_t bytes) {
+    const int o = off;
+    off += (int)((bytes + 15) / 16 * 16);
+    return o;
+  };
+  size_t scr = 0;
+  for (int l = 0; l < nl; ++l) {
+    const MGLevel<T>& M = Ls[l];
+    TailLevel<T>& L = A.L[l];
+    const bool coarsest = l == nl - 1;
+    if (M.geo.N > kTailMaxCells) return false;
+    for (int d = 0; d < 3; ++d) {
+      L.n[d] = M.geo.n[d];
+      L.wall[d] = M.geo.bc[d] == WALL;
+      L.f[d] = M.f[d];
+      L.w[d] = M.w[d];
+      L.beta[d] = M.beta[d];
+    }
+    L.x = M.x;
+    L.b = M.b;
+    L.hx = (L.n[0] + 1) / 2;
+    L.pitch = 2 * L.hx;
+    L.rows = L.n[1] * L.n[2];
+    const int per = coarsest ? kTailCgCells : (sizeof(T) == 8 ? kTailCells64 : kTailCells32);
+    int want = (int)((M.geo.N + per - 1) / per);
+    if (coarsest && M.geo.N <= kTailCgSingle) want = 1;
+    want = want > kTailCTAs ? kTailCTAs : want;
+    if (l > 0 && want > A.L[l - 1].nact) want = A.L[l - 1].nact;
+    L.rpc = (L.rows + want - 1) / want;
+    L.nact = (L.rows + L.rpc - 1) / L.rpc;
+    if (l > 0 && L.nact > A.L[l - 1].nact) return false;
+    L.cap = (L.rpc * L.pitch + 3) / 4 * 4;
+    size_t cb = (size_t)L.cap * (coarsest ? 6 * sizeof(double) : 7 * sizeof(T));
+    if (coarsest && M.geo.N <= 32) cb = cb > M.geo.N * M.geo.N * 8 ? cb : (size_t)(M.geo.N * M.geo.N * 8 + 15) / 16 * 16;
+    if (cb + 2 * L.cap * sizeof(T) > (size_t)kTailSmem) return false;
+    L.cb = (int)cb;
+    L.ox = take(L.cap * sizeof(T));
+    L.ob = take(L.cap * sizeof(T));
+    L.oa = take(cb);
+    L.otab = take((size_t)L.rpc * 32);
+    L.opack = po;
+    po += cb * L.nact;
+    if (coarsest) A.ocg = take((size_t)L.cap * 4 * sizeof(double));
+    else if (L.cap * sizeof(T) > scr) scr = L.cap * sizeof(T);
+    if (off > kTailSmem) return false;
+  }
+  A.oscr = take(scr);
+  A.ored = take((kTailThreads + 2 * kTailCTAs + 1) * sizeof(double));
+  *smem = off;
+  *pack = po;
+  return off <= kTailSmem;
+}
+
+template <typename T>
+void launch_tail_pack(const TailArgs<T>& A, cudaStream_t s) {
+  k_tail_pack<T><<<dim3(kTailCTAs, A.nl, 2), 256, 0, s>>>(A);
+}
+
+template <typename T>
+void launch_tail(const TailArgs<T>& A, size_t smem, cudaStream_t s) {
+  cudaFuncSetAttribute(k_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncSetAttribute(k_tail<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kTailCTAs);
+  cfg.blockDim = dim3(kTailThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kTailCTAs;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k_tail<T>, A);
+}
+
+#define FVM_TAIL_INST(T)                                                                        \
+  template bool tail_layout<T>(const MGLevel<T>*, int, TailArgs<T>&, size_t*, size_t*);         \
+  template void launch_tail_pack<T>(const TailArgs<T>&, cudaStream_t);                          \
+  template void launch_tail<T>(const TailArgs<T>&, size_t, cudaStream_t);
+
+FVM_TAIL_INST(double)
+FVM_TAIL_INST(float)
+
+}  // namespace fvm
