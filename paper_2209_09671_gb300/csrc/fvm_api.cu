@@ -79,27 +79,36 @@ Geo make_geo(const fvm_params& p, const LevelShape& s) {
   return g;
 }
 
-// first level of the coarse tail (fvm_tail.cu): the finest one below level 0
-// (or level 0 when there is no other) from which all levels fit; -1 when not
-// even the coarsest does.  pack: bytes of its packed coefficients
+// the coarse tail (fvm_tail.cu) of a hierarchy: its first level, the finest
+// one below level 0 (or level 0 when there is no other) from which all
+// levels fit, -1 when not even the coarsest does; the bytes of its packed
+// coefficients and of the two matrices of the coarsest level's float inverse
+struct TailPlan {
+  int first;
+  bool inverse;          // the coarsest level is solved with a float inverse
+  size_t pack, inv;
+};
 template <typename T>
-int tail_first_of(const fvm_params& p, const LevelShape* lv, int nl, size_t* pack) {
+TailPlan plan_tail_of(const fvm_params& p, const LevelShape* lv, int nl, bool inverse) {
   MGLevel<T> Ls[kMaxLevels];
   for (int l = 0; l < nl; ++l) {
     Ls[l] = MGLevel<T>();
     Ls[l].geo = make_geo(p, lv[l]);
     for (int d = 0; d < 3; ++d) Ls[l].f[d] = lv[l].f[d];
   }
+  // conjugate gradients that the caller cuts short stay conjugate gradients
+  const long long nc = Ls[nl - 1].geo.N;
+  inverse = inverse && nc > 32 && nc <= kTailInvMax && p.coarse_maxit >= nc;
   TailArgs<T> A;
-  size_t smem = 0;
+  size_t smem = 0, pack = 0;
   for (int l = nl > 1 ? 1 : 0; l < nl; ++l)
-    if (tail_layout<T>(Ls + l, nl - l, A, &smem, pack)) return l;
-  *pack = 0;
-  return -1;
+    if (tail_layout<T>(Ls + l, nl - l, inverse, A, &smem, &pack))
+      return {l, inverse, pack, (size_t)A.np * A.np * 2 * sizeof(float) + (inverse ? 256 : 0)};
+  return {-1, false, 0, 0};
 }
-int tail_first(const fvm_params& p, const LevelShape* lv, int nl, size_t* pack) {
-  return p.precision == FVM_MIXED ? tail_first_of<float>(p, lv, nl, pack)
-                                  : tail_first_of<double>(p, lv, nl, pack);
+TailPlan plan_tail(const fvm_params& p, const LevelShape* lv, int nl, bool inverse) {
+  return p.precision == FVM_MIXED ? plan_tail_of<float>(p, lv, nl, inverse)
+                                  : plan_tail_of<double>(p, lv, nl, inverse);
 }
 
 const char* check_params(const fvm_params* p) {
@@ -180,8 +189,9 @@ struct fvm_ctx {
   void* lb[kMaxLevels];
   void* lbeta[kMaxLevels][3];
   void* cg[3];
-  int tail;              // first level of the coarse tail, -1: none
+  TailPlan tail;
   void* pack;            // the tail's packed coefficients (null: formed in every cycle)
+  char* inv;             // the scale and the two matrices of the float inverse
   // reduction scratch
   double* partial;
   double* scal;          // 16 doubles
@@ -301,9 +311,9 @@ size_t plan_workspace(const fvm_params& p, fvm_ctx* c) {
   long long nc = (long long)lv[nl - 1].n[0] * lv[nl - 1].n[1] * lv[nl - 1].n[2];
   size_t o_cg[3];   // r, d and (Ad, x) in double
   for (int q = 0; q < 3; ++q) o_cg[q] = pl.take((q == 2 ? 2 : 1) * nc * sizeof(double));
-  size_t pack_bytes = 0;
-  const int tail = tail_first(p, lv, nl, &pack_bytes);
-  const size_t o_pack = pl.take(pack_bytes);
+  const TailPlan tail = plan_tail(p, lv, nl, true);
+  const size_t o_pack = pl.take(tail.pack);
+  const size_t o_inv = pl.take(tail.inv);
   size_t o_part = pl.take(2 * kRedBlocks * sizeof(double));
   size_t o_scal = pl.take(16 * sizeof(double));
   size_t o_max = pl.take(8 * sizeof(unsigned long long));
@@ -345,7 +355,8 @@ size_t plan_workspace(const fvm_params& p, fvm_ctx* c) {
     }
     for (int q = 0; q < 3; ++q) c->cg[q] = w + o_cg[q];
     c->tail = tail;
-    c->pack = pack_bytes ? w + o_pack : nullptr;
+    c->pack = tail.pack ? w + o_pack : nullptr;
+    c->inv = tail.inv ? w + o_inv : nullptr;
     c->partial = (double*)(w + o_part);
     c->scal = (double*)(w + o_scal);
     c->maxbits = (unsigned long long*)(w + o_max);
@@ -477,12 +488,19 @@ int coarse_post(const fvm_ctx* c) {
   return c->prm.mg_coarse_sweeps > 0 ? c->prm.mg_coarse_sweeps : c->prm.mg_post;
 }
 
-// the arguments of the tail that starts at level l = c->tail
+// the two matrices of the coarsest level's float inverse, behind its scale
+float* tail_matrix(fvm_ctx* c, int np, int which) {
+  return (float*)(c->inv + 256) + (size_t)which * np * np;
+}
+
+// the arguments of the tail
 template <typename T>
 size_t tail_args(fvm_ctx* c, const MGLevel<T>* Ls, double rtol, TailArgs<T>& A) {
   size_t smem = 0, pack = 0;
-  tail_layout<T>(Ls + c->tail, c->nlev - c->tail, A, &smem, &pack);
+  tail_layout<T>(Ls + c->tail.first, c->nlev - c->tail.first, c->tail.inverse, A, &smem, &pack);
   A.pack = c->pack;
+  A.G = c->inv ? tail_matrix(c, A.np, inverse_blocks(A) & 1) : nullptr;
+  A.gscale = (const double*)c->inv;
   A.rtol = rtol;
   A.maxit = c->prm.coarse_maxit;
   A.pre = coarse_pre(c);
@@ -499,15 +517,19 @@ template <typename T>
 void coarsen_betas(fvm_ctx* c, MGLevel<T>* Ls) {
   for (int l = 0; l + 1 < c->nlev; ++l)
     TIMED(c, FVM_K_BETA, 1, launch_beta_coarsen<T>(Ls[l], Ls[l + 1], c->stream));
-  if (c->tail >= 0 && c->pack) {
+  if (c->tail.first >= 0 && c->pack) {
     TailArgs<T> A;
     tail_args<T>(c, Ls, 0.0, A);
     TIMED(c, FVM_K_BETA, 1, launch_tail_pack<T>(A, c->stream));
+    if (c->inv)
+      TIMED(c, FVM_K_BETA, 1 + inverse_blocks(A),
+            launch_tail_inverse<T>(A, tail_matrix(c, A.np, 0), tail_matrix(c, A.np, 1),
+                                   (double*)c->inv, c->stream));
   }
 }
 
 // V(pre, post) cycle: red-black sweeps before the coarse correction,
-// black-red after, CG on the coarsest level; the levels from c->tail down
+// black-red after, CG on the coarsest level; the levels from the tail's first down
 // run in one kernel
 // How the finest level's x starts: as it is, at 0 (not yet zeroed), with the
 // first sweep already taken (by k_residual64 in the mixed form, or skipped
@@ -546,13 +568,13 @@ void vcycle(fvm_ctx* c, MGLevel<T>* Ls, int l, double coarse_rtol, int start = k
   cudaStream_t s = c->stream;
   const int pre = l == 0 ? c->prm.mg_pre : coarse_pre(c);
   const int post = l == 0 ? c->prm.mg_post : coarse_post(c);
-  const bool whole = l == c->tail || l == c->nlev - 1;   // no sweeps of its own here
+  const bool whole = l == c->tail.first || l == c->nlev - 1;   // no sweeps of its own here
   const bool zero = start == kStartZero;
   if (zero && (whole || pre == 0))
     TIMED(c, FVM_K_MISC, 1, launch_zero<T>(Ls[l].x, Ls[l].geo.N, s));
   const bool fold_zero = zero && !whole && pre > 0;
   const bool fold_add = addp && !whole && post > 0;
-  if (l == c->tail) {
+  if (l == c->tail.first) {
     TailArgs<T> A;
     const size_t smem = tail_args<T>(c, Ls, coarse_rtol, A);
     TIMED(c, FVM_K_COARSE_TAIL, 1, launch_tail<T>(A, smem, s));
@@ -571,7 +593,7 @@ void vcycle(fvm_ctx* c, MGLevel<T>* Ls, int l, double coarse_rtol, int start = k
     smooth<T>(c, Ls[l], l, pre, 0, fpre);
     // the next level's first sweep rides on the restriction when that level
     // sweeps on its own (not the tail, not the coarsest)
-    const bool swept = l + 1 != c->tail && l + 1 != c->nlev - 1 && coarse_pre(c) > 0;
+    const bool swept = l + 1 != c->tail.first && l + 1 != c->nlev - 1 && coarse_pre(c) > 0;
     TIMED(c, l == 0 ? FVM_K_RESTRICT_FINE : FVM_K_RESTRICT_COARSE, 1,
           launch_residual_restrict<T>(Ls[l], Ls[l + 1], s, swept));
     vcycle<T>(c, Ls, l + 1, coarse_rtol, swept ? kStartFirstSwept : kStartAsIs);
@@ -1662,16 +1684,19 @@ size_t plan_noalloc(const fvm_params& p, fvm_ctx* c, char* base) {
   for (int q = 0; q < 3; ++q) o_cg[q] = pl.take((q == 2 ? 2 : 1) * nc * sizeof(double));
   size_t o_part = pl.take(2 * kRedBlocks * sizeof(double));
   size_t o_scal = pl.take(16 * sizeof(double));
-  // the tail's packed coefficients where they fit as well (else every cycle
-  // forms them from beta: no grid is refused for them)
-  size_t pack_bytes = 0;
-  const int tail = tail_first(p, lv, nl, &pack_bytes);
-  size_t o_pack = 0;
-  if (pl.off + pack_bytes <= kNoAllocScratchBytes) o_pack = pl.take(pack_bytes);
-  else pack_bytes = 0;
+  // the tail's packed coefficients and float inverse where they fit as well
+  // (else every cycle forms the coefficients from beta and the coarsest level
+  // takes conjugate gradients: no grid is refused for them)
+  const size_t room = kNoAllocScratchBytes - (pl.off < kNoAllocScratchBytes ? pl.off : kNoAllocScratchBytes);
+  TailPlan tail = plan_tail(p, lv, nl, true);
+  if (tail.pack + tail.inv + 2 * kAlign > room) tail = plan_tail(p, lv, nl, false);
+  if (tail.pack + kAlign > room) tail.pack = 0;
+  const size_t o_pack = pl.take(tail.pack);
+  const size_t o_inv = pl.take(tail.inv);
   if (c) {
     c->tail = tail;
-    c->pack = pack_bytes ? base + o_pack : nullptr;
+    c->pack = tail.pack ? base + o_pack : nullptr;
+    c->inv = tail.inv ? base + o_inv : nullptr;
     c->b = (double*)(base + o_b);
     for (int q = 0; q < 3; ++q) c->beta0[q] = base + o_beta[q];
     c->e32 = mixed ? (float*)(base + o_e) : nullptr;

@@ -168,6 +168,8 @@ constexpr int kTailMaxCells = 32768;        // of the tail's first level
 constexpr int kTailSmem = 220 * 1024;       // shared memory of a CTA
 constexpr int kTailCells32 = 512, kTailCells64 = 256;   // cells a CTA should have (float, double)
 constexpr int kTailCgCells = 64, kTailCgSingle = 400;    // the same for the coarsest level's CG
+constexpr int kTailInvCells = 32;           // the same for the coarsest level by a float inverse
+constexpr int kTailInvMax = 1000;           // cells of a coarsest level solved with one
 template <typename T>
 struct TailLevel {
   int n[3], f[3];              // cells per axis, coarsening factor to the next level
@@ -186,7 +188,10 @@ template <typename T>
 struct TailArgs {
   int nl;                      // levels, the last one the coarsest
   TailLevel<T> L[kTailLevels];
-  int oscr, ocg, ored;         // byte offsets: fine residuals, CG vectors, reductions
+  int oscr, ocg, ored, ovec;   // byte offsets: fine residuals, CG vectors, reductions, float residual
+  int np;                      // order of the float inverse (a multiple of 64; 0: none)
+  const float* G;              // the inverse of the coarsest operator / *gscale (null: CG)
+  const double* gscale;
   const void* pack;            // coefficients of launch_tail_pack (null: formed from beta)
   double rtol;
   int maxit, pre, post;
@@ -194,8 +199,20 @@ struct TailArgs {
 };
 // lay out levels Ls[0 .. nl-1]; false when they do not fit.  smem: bytes per
 // CTA, pack: bytes of the packed coefficients
+// (inverse: the coarsest level is solved with a float inverse, A.np set)
 template <typename T>
-bool tail_layout(const MGLevel<T>* Ls, int nl, TailArgs<T>& A, size_t* smem, size_t* pack);
+bool tail_layout(const MGLevel<T>* Ls, int nl, bool inverse, TailArgs<T>& A, size_t* smem,
+                 size_t* pack);
+// the float inverse takes one launch per block of 32 pivots and ends in W0 when
+// their number is even, else in W1
+template <typename T>
+int inverse_blocks(const TailArgs<T>& A) {
+  const TailLevel<T>& L = A.L[A.nl - 1];
+  return (L.rows * L.n[0] + 31) / 32;
+}
+template <typename T>
+void launch_tail_inverse(const TailArgs<T>& A, float* W0, float* W1, double* gscale,
+                         cudaStream_t s);
 template <typename T>
 void launch_tail_pack(const TailArgs<T>& A, cudaStream_t s);
 template <typename T>

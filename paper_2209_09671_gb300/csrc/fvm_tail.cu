@@ -314,9 +314,14 @@ __device__ __forceinline__ void prolong_rows(const View<T>& F, const TailLevel<T
   }
 }
 
-__device__ __forceinline__ double warp_sum_all(double v, int steps) {
-  for (int o = 1 << (steps - 1); steps > 0; o >>= 1, --steps) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+// the sums of s and of t over the warp, in every lane (two chains at once: an
+// FP64 addition takes 63 clocks from issue to result)
+__device__ __forceinline__ void warp_sum2(double& s, double& t) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+    t += __shfl_xor_sync(0xffffffffu, t, o);
+  }
 }
 
 // Sums over the cells of a level spread over `nact` CTAs (CTA 0 alone when nact
@@ -326,42 +331,54 @@ __device__ __forceinline__ double warp_sum_all(double v, int steps) {
 // dividing or taking roots in every warp keeps it busy for thousands of clocks
 // (25 x 25 cells: 1160 instead of 870 us per V-cycle).
 struct Reduce {
-  double* vals;     // kTailThreads
-  double* slots;    // 2 sets of kTailCTAs, written by the other CTAs
-  double* out;      // the scalar handed to every thread
+  double* vals;     // 2 x kTailThreads
+  double* slots;    // 2 sets of 2 x kTailCTAs, written by the other CTAs
+  double* out;      // the scalar handed to every thread, and three for its user
   unsigned base_slots;
   int nact, rank, used;   // used: threads of this CTA with a value
   int phase;
-  // the sum of v over all cells goes through `f` in warp 0 (the same numbers
-  // in every CTA); every thread gets f's value
+  // the sums of v and u over all cells go through `f` in warp 0 (the same
+  // numbers in every CTA); every thread gets f's value
   template <typename F>
-  __device__ __forceinline__ double run(double v, F f) {
+  __device__ __forceinline__ double run2(double v, double u, F f) {
     const int tid = threadIdx.x;
-    if (tid < used) vals[tid] = v;
+    if (tid < used) {
+      vals[tid] = v;
+      vals[kTailThreads + tid] = u;
+    }
     __syncthreads();
-    if (nact == 1) {
-      if (tid < 32) {
-        double s = 0.0;
-        for (int q = tid; q < used; q += 32) s += vals[q];
-        s = f(warp_sum_all(s, used > 16 ? 5 : (used > 8 ? 4 : 3)));
-        if (tid == 0) *out = s;
+    double s = 0.0, t = 0.0;
+    if (tid < 32) {
+      for (int q = tid; q < used; q += 32) {
+        s += vals[q];
+        t += vals[kTailThreads + q];
       }
-    } else {
-      const int set = (phase++ & 1) * kTailCTAs;
-      if (tid < 32) {
-        double s = 0.0;
-        for (int q = tid; q < used; q += 32) s += vals[q];
-        s = warp_sum_all(s, used > 16 ? 5 : (used > 8 ? 4 : 3));
-        if (tid < kTailCTAs) st_cl(map_rank(base_slots + (set + rank) * 8, tid), s);
+      warp_sum2(s, t);
+    }
+    if (nact > 1) {
+      const int set = (phase++ & 1) * 2 * kTailCTAs;
+      if (tid < kTailCTAs) {
+        const unsigned to = map_rank(base_slots + (set + rank) * 8, tid);
+        st_cl(to, s);
+        st_cl(to + kTailCTAs * 8, t);
       }
       cluster_sync();
       if (tid < 32) {
-        double s = f(warp_sum_all(tid < nact ? slots[set + tid] : 0.0, 4));
-        if (tid == 0) *out = s;
+        s = tid < nact ? slots[set + tid] : 0.0;
+        t = tid < nact ? slots[set + kTailCTAs + tid] : 0.0;
+        warp_sum2(s, t);
       }
+    }
+    if (tid < 32) {
+      s = f(s, t);
+      if (tid == 0) *out = s;
     }
     __syncthreads();
     return *out;   // (rewritten only after the next call's first barrier)
+  }
+  template <typename F>
+  __device__ __forceinline__ double run(double v, F f) {
+    return run2(v, 0.0, [&](double s, double) { return f(s); });
   }
 };
 
@@ -459,6 +476,151 @@ __device__ void coarsest_cg(const View<T>& V, const TailArgs<T>& A, Reduce& red)
   for (int t = threadIdx.x; t < nc; t += kTailThreads) V.x()[t] = (T)(x[t] - xm);
 }
 
+// The coarsest level by defect correction: dx = G r with the float inverse G
+// of the level's operator (launch_tail_inverse, once per solve), r -= L dx in
+// double, until ||r|| <= rtol ||b||: each step gains what the float inverse
+// resolves (four to six digits), where conjugate gradients take 50 to 170
+// iterations of two dependent sums each (5 us an iteration).  The whole tail
+// per V-cycle: 25 x 25 coarsest cells 870 -> 65 us (to 1e-12), 11 x 18 x 5
+// 364 -> 88 us (to 1e-6).  The result
+// meets the same double residual; its mean is left as it comes (a constant
+// is no correction).  Returns false when a step gains less than a factor
+// of two (an operator too ill-conditioned for float, or not a number): the
+// caller then runs conjugate gradients.
+template <typename T>
+__device__ bool coarsest_refine(const View<T>& V, const TailArgs<T>& A, Reduce& red) {
+  const TailLevel<T>& L = V.L;
+  const int cap = L.cap, hx = L.hx, nx = L.n[0], np = A.np;
+  const double* a = V.template a<double>();
+  double* d = reinterpret_cast<double*>(V.sm + A.ocg);
+  double *r = d + cap, *x = r + cap;
+  float* mine = reinterpret_cast<float*>(V.sm + A.ovec);   // own part of the scaled residual
+  float* full = mine + (L.rpc * nx + 3) / 4 * 4;           // all of it
+  const unsigned mine_a = smem_u32(mine);
+  const int nc = V.nrows * L.pitch, own = V.nrows * nx, chunk = L.rpc * nx;
+  const int ncell = L.rows * nx;
+  const float ip = 1.0f / (float)L.pitch, ic = 1.0f / (float)chunk;
+  const double N = (double)ncell;
+  auto column = [&](int t) {
+    const int q = quot(t, ip), p = t - q * L.pitch;
+    return p < hx ? 2 * p : 2 * (p - hx) + 1;
+  };
+  double acc = 0.0, sq = 0.0;
+  for (int t = threadIdx.x; t < nc; t += kTailThreads) {
+    const double v = column(t) < nx ? (double)V.b()[t] : 0.0;
+    acc += v;
+    sq = fma(v, v, sq);
+  }
+  double rr = 0.0, stop = 0.0;   // ||r||^2 and its threshold, in warp 0
+  // (the mean of a restricted residual is small beside its size, so that its
+  // square is subtracted from the sum without cancellation)
+  double mean = 0.0;
+  double* bmean = red.out + 1;
+  double sc = red.run2(acc, sq, [&](double s, double t) {
+    mean = s / N;
+    if (threadIdx.x == 0) *bmean = mean;
+    rr = t - s * mean;
+    stop = A.rtol * A.rtol * rr;
+    return rr > stop ? 1.0 : 0.0;
+  });
+  mean = *bmean;
+  for (int t = threadIdx.x; t < nc; t += kTailThreads) {
+    r[t] = column(t) < nx ? (double)V.b()[t] - mean : 0.0;
+    x[t] = 0.0;
+  }
+  bool ok = true;
+  while (sc != 0.0) {
+    // scale so that the residual's norm is of order one in float: half its
+    // exponent, a power of two
+    if (threadIdx.x == 0) {
+      const int e = (int)((__double2hiint(rr) >> 20) & 0x7ff) - 1023;
+      bmean[1] = __hiloint2double((1023 - (e >> 1)) << 20, 0);
+      bmean[2] = 1.0 / (bmean[1] * __ldg(A.gscale));
+    }
+    __syncthreads();
+    const double scale = bmean[1], back = bmean[2];
+    for (int t = threadIdx.x; t < nc; t += kTailThreads) {
+      const int q = quot(t, ip), i = column(t);
+      if (i < nx) mine[q * nx + i] = (float)(r[t] * scale);
+    }
+    if (red.nact > 1) cluster_sync();
+    else __syncthreads();
+    for (int c = threadIdx.x; c < np; c += kTailThreads) {
+      float v = 0.f;
+      if (c < ncell) {
+        const int rk = quot(c, ic);
+        ld_cl(map_rank(mine_a + (c - rk * chunk) * 4u, rk), v);
+      }
+      full[c] = v;
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const float4* f4 = reinterpret_cast<const float4*>(full);
+    for (int r0 = w * 4; r0 < own; r0 += kTailThreads / 8) {
+      float s[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int c = lane; c < np / 4; c += 32) {
+        const float4 v = f4[c];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          if (r0 + m >= own) continue;
+          const float4 g = __ldg(reinterpret_cast<const float4*>(
+                                     A.G + (size_t)(V.rank * chunk + r0 + m) * np) + c);
+          s[m] += g.x * v.x + g.y * v.y + g.z * v.z + g.w * v.w;
+        }
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s[m] += __shfl_xor_sync(0xffffffffu, s[m], o);
+      if (lane < 4 && r0 + lane < own) {
+        const float v = lane == 0 ? s[0] : (lane == 1 ? s[1] : (lane == 2 ? s[2] : s[3]));
+        const int q = quot(r0 + lane, 1.0f / (float)nx);
+        d[q * L.pitch + row_pos(r0 + lane - q * nx, hx)] = (double)v * back;
+      }
+    }
+    if (red.nact > 1) cluster_sync();
+    else __syncthreads();
+    acc = 0.0;
+    for (int t = threadIdx.x; t < nc; t += kTailThreads) {
+      const int q = quot(t, ip), p = t - q * L.pitch;
+      const int i = p < hx ? 2 * p : 2 * (p - hx) + 1;
+      if (i >= nx) continue;
+      const int4 ra = V.tab()[2 * q];
+      const int row = q * L.pitch;
+      const unsigned o = p * 8u;
+      const double dc = d[t];
+      double v0, v1, v2, v3;
+      ld_cl(ra.x + o, v0);
+      ld_cl(ra.y + o, v1);
+      ld_cl(ra.z + o, v2);
+      ld_cl(ra.w + o, v3);
+      double ox = a[t] * (dc - d[row + row_pos(i == 0 ? nx - 1 : i - 1, hx)]);
+      double oy = a[2 * cap + t] * (dc - v0);
+      double oz = a[4 * cap + t] * (dc - v2);
+      ox = fma(a[cap + t], dc - d[row + row_pos(i == nx - 1 ? 0 : i + 1, hx)], ox);
+      oy = fma(a[3 * cap + t], dc - v1, oy);
+      oz = fma(a[5 * cap + t], dc - v3, oz);
+      const double rn = r[t] - ((ox + oy) + oz);
+      r[t] = rn;
+      x[t] += dc;
+      acc = fma(rn, rn, acc);
+    }
+    // 0: done, 1: another step, 2: no gain (or not a number)
+    sc = red.run(acc, [&](double s) {
+      const double was = rr;
+      rr = s;
+      return s <= stop ? 0.0 : (s <= 0.25 * was ? 1.0 : 2.0);
+    });
+    if (sc == 2.0) {
+      ok = false;
+      break;
+    }
+  }
+  if (ok)
+    for (int t = threadIdx.x; t < nc; t += kTailThreads) V.x()[t] = (T)x[t];
+  return ok;
+}
+
 // The coarsest level of at most 32 cells: x = G (b - mean b) with the inverse
 // G of L + s 1 1^T / N formed once per solve (coarsest_inverse).  On mean-free
 // right-hand sides that is the mean-free solution of L x = b to rounding,
@@ -472,7 +634,9 @@ __device__ void coarsest_direct(const View<T>& V) {
   const double* G = V.template a<double>();
   const int q = quot(lane, 1.0f / (float)L.n[0]), c = q * L.pitch + row_pos(lane - q * L.n[0], L.hx);
   double b = lane < N ? (double)V.b()[c] : 0.0;
-  const double mean = warp_sum_all(b, 5) / (double)N;
+  double bs = b, none = 0.0;
+  warp_sum2(bs, none);
+  const double mean = bs / (double)N;
   b = lane < N ? b - mean : 0.0;
   double s0 = 0.0, s1 = 0.0;
   for (int m = 0; m < N; m += 2) {
@@ -538,9 +702,9 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
   }
   Reduce red;
   red.vals = reinterpret_cast<double*>(sm + A.ored);
-  red.slots = red.vals + kTailThreads;
-  red.out = red.slots + 2 * kTailCTAs;
-  red.base_slots = base + A.ored + kTailThreads * 8;
+  red.slots = red.vals + 2 * kTailThreads;
+  red.out = red.slots + 4 * kTailCTAs;
+  red.base_slots = base + A.ored + 2 * kTailThreads * 8;
   red.nact = A.L[last].nact;
   red.rank = rank;
   red.phase = 0;
@@ -583,7 +747,7 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
   if (last < single || rank == 0) {
     const View<T> V(A.L[last], sm, rank);
     if (A.direct) coarsest_direct(V);
-    else coarsest_cg(V, A, red);
+    else if (!A.G || !coarsest_refine(V, A, red)) coarsest_cg(V, A, red);
   }
   for (int l = last - 1; l >= 0; --l) {
     if (l >= single && rank) continue;
@@ -624,11 +788,157 @@ __global__ void k_tail_pack(const __grid_constant__ TailArgs<T> A) {
              blockDim.x * gridDim.z);
 }
 
+// ---------------------------------------------------------------------------
+// The float inverse of the coarsest operator, (L + s 1 1^T / N) / s with s the
+// mean diagonal, by block Gauss-Jordan elimination over the whole GPU: one
+// launch per block of 32 pivots, from one matrix into the other (every tile
+// of a step reads the pivot rows and columns of the step before).  Symmetric
+// and positive definite, so no pivoting.  Rows beyond N hold the identity.
+// 32 x 32 tiles, whose CTAs are more and each repeat the pivot block's
+// inverse, took 17 us per block for 625 cells, 32 us for 990.
+template <typename T>
+__global__ void k_inv_init(const __grid_constant__ TailLevel<T> L, float* __restrict__ W, int np,
+                           double* __restrict__ gscale) {
+  __shared__ float part[8];
+  const int nx = L.n[0], N = L.rows * nx;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float a[6], sum = 0.f;
+  for (int c = threadIdx.x; c < N; c += 256) {
+    const int R = c / nx;
+    cell_coefs<T, float>(L, c - R * nx, R, a);
+    sum += (a[0] + a[1]) + (a[2] + a[3]) + (a[4] + a[5]);
+  }
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (lane == 0) part[w] = sum;
+  __syncthreads();
+  sum = 0.f;
+  for (int q = 0; q < 8; ++q) sum += part[q];
+  const float s = sum / (float)N, is = 1.0f / s;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *gscale = (double)s;
+  const int r = blockIdx.x * 8 + w;
+  float* row = W + (size_t)r * np;
+  if (r >= N) {
+    for (int c = lane; c < np; c += 32) row[c] = c == r ? 1.f : 0.f;
+    return;
+  }
+  for (int c = lane; c < np; c += 32) row[c] = c < N ? 1.0f / (float)N : 0.f;
+  __syncwarp();
+  if (lane == 0) {
+    const int ny = L.n[1], R = r / nx, i = r - R * nx, k = R / ny, j = R - k * ny;
+    cell_coefs<T, float>(L, i, R, a);
+    const int idx[3] = {i, j, k}, st[3] = {1, nx, nx * ny};
+    float dg = 0.f;
+    for (int d = 0; d < 3; ++d) {
+      const int n = L.n[d];
+      if (n == 1) continue;
+      row[idx[d] == 0 ? r + (n - 1) * st[d] : r - st[d]] -= a[2 * d] * is;
+      row[idx[d] == n - 1 ? r - (n - 1) * st[d] : r + st[d]] -= a[2 * d + 1] * is;
+      dg += a[2 * d] + a[2 * d + 1];
+    }
+    row[r] += dg * is;
+  }
+}
+
+// one block of 32 pivots (rows and columns b * 32 ...) on a 64 x 64 tile: every
+// CTA inverts the pivot block D itself (2 us; as a launch of its own it would
+// cost the gap between launches as well), forms X = D^-1 A[pivots, tile] and
+// subtracts A[tile, pivots] X
+__global__ void __launch_bounds__(256) k_inv_step(const float* __restrict__ A,
+                                                  float* __restrict__ B, int np, int b) {
+  __shared__ float D[2][32][33];
+  __shared__ __align__(16) float Ct[32][68], R[32][64], X[32][64];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int i0 = blockIdx.y * 64, j0 = blockIdx.x * 64, p0 = b * 32;
+  const int tx = tid & 15, ty = tid >> 4;
+  const bool pc = ((j0 + tx * 4) >> 5) == b;    // the thread's columns are pivots
+  const bool pr = ((i0 + ty * 4) >> 5) == b;    // the thread's rows are pivots
+  float4 t[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    t[q] = *reinterpret_cast<const float4*>(A + (size_t)(i0 + ty * 4 + q) * np + j0 + tx * 4);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) D[0][w + 8 * q][lane] = A[(size_t)(p0 + w + 8 * q) * np + p0 + lane];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    Ct[lane][w + 8 * q] = A[(size_t)(i0 + w + 8 * q) * np + p0 + lane];
+    R[w + 8 * (q >> 1)][lane + 32 * (q & 1)] =
+        A[(size_t)(p0 + w + 8 * (q >> 1)) * np + j0 + lane + 32 * (q & 1)];
+  }
+  __syncthreads();
+  // D <- D^-1, from one copy into the other
+  for (int p = 0; p < 32; ++p) {
+    const float(*S)[33] = D[p & 1];
+    float(*O)[33] = D[(p & 1) ^ 1];
+    const float ip = __fdividef(1.0f, S[p][p]);
+    const float rp = lane == p ? ip : S[p][lane] * ip;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = w + 8 * q;
+      const float f = S[r][p], v = S[r][lane];
+      O[r][lane] = r == p ? rp : (lane == p ? -f * ip : v - f * rp);
+    }
+    __syncthreads();
+  }
+  {
+    const float(*V)[33] = D[0];
+    const int r = ty * 2;
+    float4 x0 = {0.f, 0.f, 0.f, 0.f}, x1 = x0;
+    if (pc) {
+      const int c = (j0 + tx * 4) & 31;
+      x0 = {V[r][c], V[r][c + 1], V[r][c + 2], V[r][c + 3]};
+      x1 = {V[r + 1][c], V[r + 1][c + 1], V[r + 1][c + 2], V[r + 1][c + 3]};
+    } else {
+#pragma unroll 8
+      for (int m = 0; m < 32; ++m) {
+        const float4 v = *reinterpret_cast<const float4*>(&R[m][tx * 4]);
+        const float d0 = V[r][m], d1 = V[r + 1][m];
+        x0.x += d0 * v.x; x0.y += d0 * v.y; x0.z += d0 * v.z; x0.w += d0 * v.w;
+        x1.x += d1 * v.x; x1.y += d1 * v.y; x1.z += d1 * v.z; x1.w += d1 * v.w;
+      }
+    }
+    *reinterpret_cast<float4*>(&X[r][tx * 4]) = x0;
+    *reinterpret_cast<float4*>(&X[r + 1][tx * 4]) = x1;
+  }
+  __syncthreads();
+  if (pr) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      t[q] = *reinterpret_cast<const float4*>(&X[(i0 + ty * 4 + q) & 31][tx * 4]);
+  } else {
+    if (pc)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) t[q] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+    for (int m = 0; m < 32; ++m) {
+      const float4 v = *reinterpret_cast<const float4*>(&X[m][tx * 4]);
+      const float4 c = *reinterpret_cast<const float4*>(&Ct[m][ty * 4]);
+      const float cc[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        t[q].x -= cc[q] * v.x; t[q].y -= cc[q] * v.y; t[q].z -= cc[q] * v.z; t[q].w -= cc[q] * v.w;
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    *reinterpret_cast<float4*>(B + (size_t)(i0 + ty * 4 + q) * np + j0 + tx * 4) = t[q];
+}
+
+template <typename T>
+void launch_tail_inverse(const TailArgs<T>& A, float* W0, float* W1, double* gscale,
+                         cudaStream_t s) {
+  const int nb = inverse_blocks(A), nt = A.np / 64;
+  k_inv_init<T><<<A.np / 8, 256, 0, s>>>(A.L[A.nl - 1], W0, A.np, gscale);
+  for (int b = 0; b < nb; ++b)
+    k_inv_step<<<dim3(nt, nt), 256, 0, s>>>(b & 1 ? W1 : W0, b & 1 ? W0 : W1, A.np, b);
+}
+
 // Layout of a tail that starts at level Ls[0] with nl levels; false when it
 // does not fit.  The cells a CTA should have: enough that a sweep's work is
 // no smaller than the barrier that ends it.
 template <typename T>
-bool tail_layout(const MGLevel<T>* Ls, int nl, TailArgs<T>& A, size_t* smem, size_t* pack) {
+bool tail_layout(const MGLevel<T>* Ls, int nl, bool inverse, TailArgs<T>& A, size_t* smem,
+                 size_t* pack) {
   if (nl < 1 || nl > kTailLevels) return false;
   A.nl = nl;
   int off = 0;
@@ -656,9 +966,12 @@ bool tail_layout(const MGLevel<T>* Ls, int nl, TailArgs<T>& A, size_t* smem, siz
     L.hx = (L.n[0] + 1) / 2;
     L.pitch = 2 * L.hx;
     L.rows = L.n[1] * L.n[2];
-    const int per = coarsest ? kTailCgCells : (sizeof(T) == 8 ? kTailCells64 : kTailCells32);
+    // the float inverse is read by rows, from all CTAs at once
+    const bool inv = coarsest && inverse && M.geo.N > 32;
+    const int per = inv ? kTailInvCells
+                        : (coarsest ? kTailCgCells : (sizeof(T) == 8 ? kTailCells64 : kTailCells32));
     int want = (int)((M.geo.N + per - 1) / per);
-    if (coarsest && M.geo.N <= kTailCgSingle) want = 1;
+    if (coarsest && !inv && M.geo.N <= kTailCgSingle) want = 1;
     want = want > kTailCTAs ? kTailCTAs : want;
     if (l > 0 && want > A.L[l - 1].nact) want = A.L[l - 1].nact;
     L.rpc = (L.rows + want - 1) / want;
@@ -675,12 +988,16 @@ bool tail_layout(const MGLevel<T>* Ls, int nl, TailArgs<T>& A, size_t* smem, siz
     L.otab = take((size_t)L.rpc * 32);
     L.opack = po;
     po += cb * L.nact;
-    if (coarsest) A.ocg = take((size_t)L.cap * 4 * sizeof(double));
+    if (coarsest) {
+      A.ocg = take((size_t)L.cap * 4 * sizeof(double));
+      A.np = inv ? (int)((M.geo.N + 63) / 64 * 64) : 0;
+      A.ovec = take(inv ? ((size_t)(L.rpc * L.n[0] + 3) / 4 * 4 + A.np) * sizeof(float) : 0);
+    }
     else if (L.cap * sizeof(T) > scr) scr = L.cap * sizeof(T);
     if (off > kTailSmem) return false;
   }
   A.oscr = take(scr);
-  A.ored = take((kTailThreads + 2 * kTailCTAs + 1) * sizeof(double));
+  A.ored = take((2 * kTailThreads + 4 * kTailCTAs + 4) * sizeof(double));
   *smem = off;
   *pack = po;
   return off <= kTailSmem;
@@ -711,7 +1028,8 @@ void launch_tail(const TailArgs<T>& A, size_t smem, cudaStream_t s) {
 }
 
 #define FVM_TAIL_INST(T)                                                                        \
-  template bool tail_layout<T>(const MGLevel<T>*, int, TailArgs<T>&, size_t*, size_t*);         \
+  template bool tail_layout<T>(const MGLevel<T>*, int, bool, TailArgs<T>&, size_t*, size_t*);   \
+  template void launch_tail_inverse<T>(const TailArgs<T>&, float*, float*, double*, cudaStream_t); \
   template void launch_tail_pack<T>(const TailArgs<T>&, cudaStream_t);                          \
   template void launch_tail<T>(const TailArgs<T>&, size_t, cudaStream_t);
 

@@ -1,7 +1,8 @@
 """The multigrid levels that run in one cluster launch, on hierarchies that
 take each of its forms: a level on one CTA or spread over the cluster, rows of
 odd length, axes of one cell, periodic wrap, the coarsest level by its inverse
-(at most 32 cells), by conjugate gradients on one CTA or on the cluster, a tail
+(at most 32 cells), by a float inverse in defect correction or by conjugate
+gradients, on one CTA or on the cluster, a tail
 of the coarsest level alone, and the scratch-limited solve whose coefficients
 are formed in every cycle.  FP64 with a fixed cycle count against the oracle's
 V-cycles at the FP64 parity bound; mixed to 1e-12 against the FP64 solution."""
@@ -22,9 +23,9 @@ GRIDS = [
     (64, 64, 1, (W, W, P_)),      # 2D
     (64, 1, 1, (W, P_, P_)),      # one row
     (1, 48, 1, (P_, W, P_)),      # one column
-    (28, 20, 12, (W, W, W)),      # odd rows at the coarsest level, CG on one CTA
+    (28, 20, 12, (W, W, W)),      # odd rows at the coarsest level
     (12, 12, 12, (P_, P_, P_)),   # coarsening stopped by the periodic colouring
-    (66, 50, 1, (W, W, P_)),      # 825 coarsest cells: CG on the cluster
+    (66, 50, 1, (W, W, P_)),      # 825 coarsest cells
     (44, 20, 20, (W, P_, W)),     # coarsest level with wrap
 ]
 
@@ -52,6 +53,18 @@ def _solve(P, p, alpha, rhs):
 def test_f64_cycles_equal_oracle(nx, ny, nz, bc):
     P = need_gpu()
     p, alpha, rhs = _problem(nx, ny, nz, bc, mg_fixed_cycles=4)
+    ref, _, _ = O.poisson_solve(alpha, rhs, np.zeros(p.shape), p)
+    got, _ = _solve(P, p, alpha, rhs)
+    assert rel_l2(got, ref.numpy()) <= 1e-11
+
+
+@pytest.mark.parametrize("nx,ny,nz,bc,maxit", [(28, 20, 12, (W, W, W), 104), (66, 50, 1, (W, W, P_), 800),
+                                               (130, 34, 1, (W, P_, P_), 1000)])
+def test_f64_cycles_with_conjugate_gradients(nx, ny, nz, bc, maxit):
+    """An iteration cap below the cell count (or more than 1000 coarsest cells)
+    keeps the coarsest level on conjugate gradients, which end before it."""
+    P = need_gpu()
+    p, alpha, rhs = _problem(nx, ny, nz, bc, mg_fixed_cycles=4, coarse_maxit=maxit)
     ref, _, _ = O.poisson_solve(alpha, rhs, np.zeros(p.shape), p)
     got, _ = _solve(P, p, alpha, rhs)
     assert rel_l2(got, ref.numpy()) <= 1e-11
