@@ -188,6 +188,7 @@ struct fvm_ctx {
   void* lx[kMaxLevels];
   void* lb[kMaxLevels];
   void* lbeta[kMaxLevels][3];
+  void* linv[kMaxLevels];    // reciprocal diagonals of the levels above the tail (double; null: none)
   void* cg[3];
   TailPlan tail;
   void* pack;            // the tail's packed coefficients (null: formed in every cycle)
@@ -301,17 +302,19 @@ size_t plan_workspace(const fvm_params& p, fvm_ctx* c) {
     o_e = pl.take(N * sizeof(float));
     o_r = pl.take(N * sizeof(float));
   }
-  size_t o_lx[kMaxLevels], o_lb[kMaxLevels], o_lbeta[kMaxLevels][3];
+  const TailPlan tail = plan_tail(p, lv, nl, true);
+  const int above = tail.first < 0 ? nl - 1 : tail.first;   // levels that sweep on their own
+  size_t o_lx[kMaxLevels], o_lb[kMaxLevels], o_lbeta[kMaxLevels][3], o_linv[kMaxLevels];
   for (int l = 1; l < nl; ++l) {
     long long n = (long long)lv[l].n[0] * lv[l].n[1] * lv[l].n[2];
     o_lx[l] = pl.take(n * ms);
     o_lb[l] = pl.take(n * ms);
     for (int q = 0; q < 3; ++q) o_lbeta[l][q] = pl.take(n * ms);
+    o_linv[l] = !mixed && l < above ? pl.take(n * ms) : 0;
   }
   long long nc = (long long)lv[nl - 1].n[0] * lv[nl - 1].n[1] * lv[nl - 1].n[2];
   size_t o_cg[3];   // r, d and (Ad, x) in double
   for (int q = 0; q < 3; ++q) o_cg[q] = pl.take((q == 2 ? 2 : 1) * nc * sizeof(double));
-  const TailPlan tail = plan_tail(p, lv, nl, true);
   const size_t o_pack = pl.take(tail.pack);
   const size_t o_inv = pl.take(tail.inv);
   size_t o_part = pl.take(2 * kRedBlocks * sizeof(double));
@@ -352,7 +355,10 @@ size_t plan_workspace(const fvm_params& p, fvm_ctx* c) {
       c->lx[l] = w + o_lx[l];
       c->lb[l] = w + o_lb[l];
       for (int q = 0; q < 3; ++q) c->lbeta[l][q] = w + o_lbeta[l][q];
+      c->linv[l] = !mixed && l < above ? w + o_linv[l] : nullptr;
     }
+    // the finest level's fills the buffer that the solves leave free
+    c->linv[0] = !mixed && above > 0 ? c->tmp : nullptr;
     for (int q = 0; q < 3; ++q) c->cg[q] = w + o_cg[q];
     c->tail = tail;
     c->pack = tail.pack ? w + o_pack : nullptr;
@@ -414,6 +420,18 @@ fvm_status read_scalar(fvm_ctx* c, const double* dsrc, double* host) {
   return FVM_OK;
 }
 
+// the common weight of the coupled axes, 0 when they differ
+template <typename T>
+T uniform_weight(const T* w) {
+  T u = T(0);
+  for (int d = 0; d < 3; ++d) {
+    if (w[d] == T(0)) continue;
+    if (u != T(0) && w[d] != u) return T(0);
+    u = w[d];
+  }
+  return u;
+}
+
 template <typename T>
 MGLevel<T> mg_level(fvm_ctx* c, int l, T* x, T* b, T* const* beta) {
   MGLevel<T> L;
@@ -424,6 +442,8 @@ MGLevel<T> mg_level(fvm_ctx* c, int l, T* x, T* b, T* const* beta) {
     L.beta[q] = beta[q];
     L.w[q] = (T)L.geo.w[q];
   }
+  L.wu = uniform_weight(L.w);
+  L.inv = sizeof(T) == sizeof(double) ? (T*)c->linv[l] : nullptr;
   for (int d = 0; d < 3; ++d) L.f[d] = c->shp[l].f[d];
   return L;
 }
@@ -517,6 +537,8 @@ template <typename T>
 void coarsen_betas(fvm_ctx* c, MGLevel<T>* Ls) {
   for (int l = 0; l + 1 < c->nlev; ++l)
     TIMED(c, FVM_K_BETA, 1, launch_beta_coarsen<T>(Ls[l], Ls[l + 1], c->stream));
+  for (int l = 0; l < c->nlev; ++l)
+    if (Ls[l].inv) TIMED(c, FVM_K_BETA, 1, launch_inv_diag<T>(Ls[l], c->stream));
   if (c->tail.first >= 0 && c->pack) {
     TailArgs<T> A;
     tail_args<T>(c, Ls, 0.0, A);
@@ -595,7 +617,8 @@ void vcycle(fvm_ctx* c, MGLevel<T>* Ls, int l, double coarse_rtol, int start = k
     // sweeps on its own (not the tail, not the coarsest)
     const bool swept = l + 1 != c->tail.first && l + 1 != c->nlev - 1 && coarse_pre(c) > 0;
     TIMED(c, l == 0 ? FVM_K_RESTRICT_FINE : FVM_K_RESTRICT_COARSE, 1,
-          launch_residual_restrict<T>(Ls[l], Ls[l + 1], s, swept));
+          launch_residual_restrict<T>(Ls[l], Ls[l + 1], s, swept,
+                                        pre > 0 && sizeof(T) == sizeof(double)));
     vcycle<T>(c, Ls, l + 1, coarse_rtol, swept ? kStartFirstSwept : kStartAsIs);
     if (post > 0) {
       // the prolongation rides on the first post-smoothing sweep
@@ -1687,13 +1710,21 @@ size_t plan_noalloc(const fvm_params& p, fvm_ctx* c, char* base) {
   // the tail's packed coefficients and float inverse where they fit as well
   // (else every cycle forms the coefficients from beta and the coarsest level
   // takes conjugate gradients: no grid is refused for them)
-  const size_t room = kNoAllocScratchBytes - (pl.off < kNoAllocScratchBytes ? pl.off : kNoAllocScratchBytes);
+  size_t room = kNoAllocScratchBytes - (pl.off < kNoAllocScratchBytes ? pl.off : kNoAllocScratchBytes);
   TailPlan tail = plan_tail(p, lv, nl, true);
   if (tail.pack + tail.inv + 2 * kAlign > room) tail = plan_tail(p, lv, nl, false);
   if (tail.pack + kAlign > room) tail.pack = 0;
   const size_t o_pack = pl.take(tail.pack);
   const size_t o_inv = pl.take(tail.inv);
+  // likewise the reciprocal diagonals, finest level first
+  const int above = tail.first < 0 ? nl - 1 : tail.first;
+  size_t o_linv[kMaxLevels];
+  for (int l = 0; l < above; ++l) {
+    const size_t n = (size_t)lv[l].n[0] * lv[l].n[1] * lv[l].n[2] * ms;
+    o_linv[l] = !mixed && pl.off + n + kAlign <= kNoAllocScratchBytes ? pl.take(n) : 0;
+  }
   if (c) {
+    for (int l = 0; l < above; ++l) c->linv[l] = o_linv[l] ? base + o_linv[l] : nullptr;
     c->tail = tail;
     c->pack = tail.pack ? base + o_pack : nullptr;
     c->inv = tail.inv ? base + o_inv : nullptr;

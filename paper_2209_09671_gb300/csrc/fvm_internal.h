@@ -69,6 +69,8 @@ struct MGLevel {
   T* b;
   T* beta[3];
   T w[3];            // 1 / hd^2 in the level's precision (0: no coupling)
+  T wu;              // the one weight of every coupled axis, 0 when they differ
+  T* inv;            // reciprocal diagonal per cell (null: the sweeps divide)
   int f[3];          // coarsening factor to the next level
 };
 
@@ -142,9 +144,13 @@ void launch_gs(const MGLevel<T>& L, int colour, cudaStream_t s, const int* gate 
                int gate_min = 0);
 
 
+// half: the last sweep was of colour 1, whose cells' residuals are taken as 0
 template <typename T>
 void launch_residual_restrict(const MGLevel<T>& F, const MGLevel<T>& C, cudaStream_t s,
-                              bool sweep = false);
+                              bool sweep = false, bool half = false);
+// L.inv from the betas
+template <typename T>
+void launch_inv_diag(const MGLevel<T>& L, cudaStream_t s);
 template <typename T>
 void launch_prolong(const MGLevel<T>& F, const MGLevel<T>& C, cudaStream_t s);
 // a sweep of `colour` on F reading the other colour plus the coarse

@@ -141,6 +141,16 @@ __device__ __forceinline__ X apply_L_at(const MGLevel<T>& L, const X* __restrict
   const Geo& g = L.geo;
   X xc = x[c];
   X out = X(0);
+  if (L.wu != T(0)) {
+    // one weight for every axis: 13 operations instead of 15
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      if (g.n[d] == 1) continue;
+      out += (X)nb.blo[d] * (xc - x[nb.lo[d]]);
+      out += (X)nb.bhi[d] * (xc - x[nb.hi[d]]);
+    }
+    return out * (X)L.wu;
+  }
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     if (g.n[d] == 1) continue;
@@ -160,19 +170,81 @@ __device__ __forceinline__ void decode_lv(const Geo& g, long long c, int& i, int
 // ---------------------------------------------------------------------------
 // Gauss-Seidel value of one cell from its right-hand side, the face betas
 // and the neighbour values on the low and high side of each axis (axes of
-// one cell carry no coupling)
+// one cell carry no coupling).  wu: the common weight of the axes (0: w per
+// axis).  inv: the cell's reciprocal diagonal, null to form and divide by the
+// diagonal.  A double update is bound by the FP64 pipe (2 lanes a clock per
+// SM): 8 operations with both, about 27 with neither; a colour sweep of
+// 128^3 cells took 50 us before, and the array costs 8 bytes per cell.  In
+// float the sweeps are bound by memory, so they divide.
 template <typename T>
-__device__ __forceinline__ T gs_formula(const Geo& g, const T* w, T b, const T* blo, const T* bhi,
-                                        const T* xlo, const T* xhi) {
-  T num = b;
-  T den = T(0);
+__device__ __forceinline__ T gs_formula(const Geo& g, const T* w, T wu, T b, const T* blo,
+                                        const T* bhi, const T* xlo, const T* xhi,
+                                        const T* inv = nullptr) {
+  T num, den = T(0);
+  if (wu != T(0)) {
+    T sum = T(0);
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    if (g.n[d] == 1) continue;
-    num += (blo[d] * xlo[d] + bhi[d] * xhi[d]) * w[d];
-    den += (blo[d] + bhi[d]) * w[d];
+    for (int d = 0; d < 3; ++d) {
+      if (g.n[d] == 1) continue;
+      sum += blo[d] * xlo[d];
+      sum += bhi[d] * xhi[d];
+    }
+    num = b + sum * wu;
+  } else {
+    num = b;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      if (g.n[d] == 1) continue;
+      num += (blo[d] * xlo[d] + bhi[d] * xhi[d]) * w[d];
+    }
+  }
+  if (inv) return num * *inv;
+  if (wu != T(0)) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      if (g.n[d] == 1) continue;
+      den += blo[d] + bhi[d];
+    }
+    den *= wu;
+  } else {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      if (g.n[d] == 1) continue;
+      den += (blo[d] + bhi[d]) * w[d];
+    }
   }
   return num / den;
+}
+
+template <typename T>
+__device__ __forceinline__ T gs_value(const MGLevel<T>& L, int c, const OpNb<T>& nb, const T* xlo,
+                                      const T* xhi) {
+  return gs_formula(L.geo, L.w, L.wu, L.b[c], nb.blo, nb.bhi, xlo, xhi,
+                    L.inv ? L.inv + c : nullptr);
+}
+
+template <typename T>
+__global__ void k_inv_diag(MGLevel<T> L) {
+  const Geo& g = L.geo;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.y * blockDim.y + threadIdx.y;
+  const int k = blockIdx.z * blockDim.z + threadIdx.z;
+  if (i >= g.n[0] || j >= g.n[1] || k >= g.n[2]) return;
+  const int c = (k * g.n[1] + j) * g.n[0] + i;
+  OpNb<T> nb;
+  neighbours(L, i, j, k, c, nb);
+  T den = T(0);
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+    if (g.n[d] > 1) den += (nb.blo[d] + nb.bhi[d]) * L.w[d];
+  L.inv[c] = T(1) / den;
+}
+
+template <typename T>
+void launch_inv_diag(const MGLevel<T>& L, cudaStream_t s) {
+  const dim3 bs(32, 4, 2);
+  const dim3 gs((L.geo.n[0] + 31) / 32, (L.geo.n[1] + 3) / 4, (L.geo.n[2] + 1) / 2);
+  k_inv_diag<T><<<gs, bs, 0, s>>>(L);
 }
 
 // Gauss-Seidel update of one cell (its colour's neighbours are fixed)
@@ -188,7 +260,7 @@ __device__ __forceinline__ void gs_point(const MGLevel<T>& L, int i, int j, int 
     xlo[d] = L.x[nb.lo[d]];
     xhi[d] = L.x[nb.hi[d]];
   }
-  L.x[c] = gs_formula(g, L.w, L.b[c], nb.blo, nb.bhi, xlo, xhi);
+  L.x[c] = gs_value(L, c, nb, xlo, xhi);
 }
 
 // gate (optional): the sweep does nothing once *gate >= gate_min (the FP64
@@ -215,43 +287,43 @@ void launch_gs(const MGLevel<T>& L, int colour, cudaStream_t s, const int* gate,
   k_gs<T><<<gs, bs, 0, s>>>(L, colour, gate, gate_min);
 }
 
-// coarse b = mean over children of (b - L x) on the fine level; coarse x = 0
+// coarse b = mean over children of (b - L x) on the fine level; coarse x = 0.
+// half: the fine level's last sweep was of colour 1, so the residuals of
+// those cells are 0 up to the rounding of that sweep; only the children of
+// colour 0 are formed (half the FP64 operations: 90 -> 43 us for 128^3 double).
+// Not in float: there that rounding is what keeps the restricted residual's
+// sum 0, and without it a density ratio of 7900 between the phases slows the
+// convergence (1.5e-9 -> 3.1e-8 after five refinements at 256^3).
 template <typename T>
 __device__ __forceinline__ void restrict_point(const MGLevel<T>& F, const MGLevel<T>& C, int I,
-                                               int J, int K) {
+                                               int J, int K, bool half) {
   const long long cc = lin(C.geo, I, J, K);
   T acc = T(0);
-  int cnt = 0;
   for (int dz = 0; dz < F.f[2]; ++dz)
-    for (int dy = 0; dy < F.f[1]; ++dy)
+    for (int dy = 0; dy < F.f[1]; ++dy) {
+      const int j = J * F.f[1] + dy, k = K * F.f[2] + dz;
       for (int dx = 0; dx < F.f[0]; ++dx) {
-        int i = I * F.f[0] + dx, j = J * F.f[1] + dy, k = K * F.f[2] + dz;
+        const int i = I * F.f[0] + dx;
+        if (half && ((i + j + k) & 1)) continue;
         const int c = (k * F.geo.n[1] + j) * F.geo.n[0] + i;
         OpNb<T> nb;
         neighbours(F, i, j, k, c, nb);
         acc += F.b[c] - apply_L_at<T, T>(F, F.x, c, nb);
-        ++cnt;
       }
-  C.b[cc] = acc / (T)cnt;
+    }
+  const int n = F.f[0] * F.f[1] * F.f[2];   // 1, 2, 4 or 8 children
+  C.b[cc] = acc * (n == 8 ? T(0.125) : (n == 4 ? T(0.25) : (n == 2 ? T(0.5) : T(1))));
   C.x[cc] = T(0);
-}
-
-template <typename T>
-__device__ __forceinline__ void restrict_point(const MGLevel<T>& F, const MGLevel<T>& C,
-                                               long long cc) {
-  int I, J, K;
-  decode_lv(C.geo, cc, I, J, K);
-  restrict_point(F, C, I, J, K);
 }
 
 // one thread per coarse cell on a 3D grid (no index division per thread)
 template <typename T>
-__global__ void k_residual_restrict(MGLevel<T> F, MGLevel<T> C, int sweep) {
+__global__ void k_residual_restrict(MGLevel<T> F, MGLevel<T> C, int sweep, int half) {
   const int I = blockIdx.x * blockDim.x + threadIdx.x;
   const int J = blockIdx.y * blockDim.y + threadIdx.y;
   const int K = blockIdx.z * blockDim.z + threadIdx.z;
   if (I >= C.geo.n[0] || J >= C.geo.n[1] || K >= C.geo.n[2]) return;
-  restrict_point(F, C, I, J, K);
+  restrict_point(F, C, I, J, K, half != 0);
   if (sweep && ((I + J + K) & 1) == 0) {
     // the coarse level's first sweep (colour 0 from x = 0) needs only the
     // cell's own right-hand side: taken here, with k_gs's arithmetic
@@ -259,16 +331,17 @@ __global__ void k_residual_restrict(MGLevel<T> F, MGLevel<T> C, int sweep) {
     OpNb<T> nb;
     neighbours(C, I, J, K, cc, nb);
     const T z[3] = {T(0), T(0), T(0)};
-    C.x[cc] = gs_formula(C.geo, C.w, C.b[cc], nb.blo, nb.bhi, z, z);
+    C.x[cc] = gs_value(C, cc, nb, z, z);
   }
 }
 
 // sweep: also take the coarse level's first Gauss-Seidel sweep from x = 0
 template <typename T>
-void launch_residual_restrict(const MGLevel<T>& F, const MGLevel<T>& C, cudaStream_t s, bool sweep) {
+void launch_residual_restrict(const MGLevel<T>& F, const MGLevel<T>& C, cudaStream_t s, bool sweep,
+                              bool half) {
   const dim3 bs(32, 4, 2);
   const dim3 gs((C.geo.n[0] + 31) / 32, (C.geo.n[1] + 3) / 4, (C.geo.n[2] + 1) / 2);
-  k_residual_restrict<T><<<gs, bs, 0, s>>>(F, C, sweep ? 1 : 0);
+  k_residual_restrict<T><<<gs, bs, 0, s>>>(F, C, sweep ? 1 : 0, half ? 1 : 0);
 }
 
 // the coarsening factor of an axis is 1 or 2
@@ -281,14 +354,6 @@ __device__ __forceinline__ void prolong_point(const MGLevel<T>& F, const MGLevel
   const long long p = lin(C.geo, coarse_index(i, F.f[0]), coarse_index(j, F.f[1]),
                           coarse_index(k, F.f[2]));
   F.x[c] = F.x[c] + C.x[p];
-}
-
-template <typename T>
-__device__ __forceinline__ void prolong_point(const MGLevel<T>& F, const MGLevel<T>& C,
-                                              long long c) {
-  int i, j, k;
-  decode_lv(F.geo, c, i, j, k);
-  prolong_point(F, C, i, j, k);
 }
 
 // one thread per fine cell on a 3D grid (no index division per thread)
@@ -342,7 +407,7 @@ __global__ void k_gs_prolong(MGLevel<T> F, MGLevel<T> C, int colour) {
     xlo[d] = F.x[nb.lo[d]] + C.x[pl];
     xhi[d] = F.x[nb.hi[d]] + C.x[ph];
   }
-  F.x[c] = gs_formula(g, F.w, F.b[c], nb.blo, nb.bhi, xlo, xhi);
+  F.x[c] = gs_value(F, c, nb, xlo, xhi);
 }
 
 // The first sweep of a solve that starts from x = 0 (the mixed form's inner
@@ -364,7 +429,7 @@ __global__ void k_gs_zero(MGLevel<T> L, int colour) {
   OpNb<T> nb;
   neighbours(L, i, j, k, row + i, nb);
   const T z[3] = {T(0), T(0), T(0)};
-  L.x[row + i] = gs_formula(g, L.w, L.b[row + i], nb.blo, nb.bhi, z, z);
+  L.x[row + i] = gs_value(L, row + i, nb, z, z);
 }
 
 // The last sweep of the mixed form's inner correction with p += e folded in:
@@ -390,7 +455,7 @@ __global__ void k_gs_addp(MGLevel<float> L, int colour, double* __restrict__ p) 
     xlo[d] = L.x[nb.lo[d]];
     xhi[d] = L.x[nb.hi[d]];
   }
-  const float e = gs_formula(g, L.w, L.b[row + i], nb.blo, nb.bhi, xlo, xhi);
+  const float e = gs_value(L, row + i, nb, xlo, xhi);
   p[row + i] = p[row + i] + (double)e;
 }
 
@@ -594,7 +659,9 @@ __global__ void k_residual64(Geo g, const double* __restrict__ p, const double* 
     r32[c] = rf;
     if (e32) {
       const float z[3] = {0.f, 0.f, 0.f};
-      e32[c] = ((i + j + k) & 1) == 0 ? gs_formula(g, w32.w, rf, blo, bhi, z, z) : 0.f;
+      e32[c] = ((i + j + k) & 1) == 0 ? gs_formula(g, w32.w, w32.w[0] != 0.f ? w32.w[0] : (w32.w[1] != 0.f ? w32.w[1] : w32.w[2]), rf,
+                                                       blo, bhi, z, z)
+                                          : 0.f;
     }
     acc += r * r;
   }
@@ -696,7 +763,9 @@ void launch_ctl_store(const SolveCtl* ctl, SolveCtl* rec, int* sticky, cudaStrea
                                     cudaStream_t);                                           \
   template void launch_zero<T>(T*, long long, cudaStream_t);                                 \
   template void launch_gs<T>(const MGLevel<T>&, int, cudaStream_t, const int*, int);        \
-  template void launch_residual_restrict<T>(const MGLevel<T>&, const MGLevel<T>&, cudaStream_t, bool); \
+  template void launch_residual_restrict<T>(const MGLevel<T>&, const MGLevel<T>&, cudaStream_t, bool, \
+                                            bool);                                           \
+  template void launch_inv_diag<T>(const MGLevel<T>&, cudaStream_t);                         \
   template void launch_prolong<T>(const MGLevel<T>&, const MGLevel<T>&, cudaStream_t);       \
   template void launch_gs_prolong<T>(const MGLevel<T>&, const MGLevel<T>&, int, cudaStream_t); \
   template void launch_gs_zero<T>(const MGLevel<T>&, int, cudaStream_t);                      \

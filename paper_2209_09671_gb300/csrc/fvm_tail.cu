@@ -229,9 +229,10 @@ __device__ __forceinline__ void sweep(const View<T>& V, int col) {
   }
 }
 
-// r = b - L x over the CTA's rows
+// r = b - L x over the CTA's rows; 0 at the cells of colour 1 when the last
+// sweep was theirs (in double: see restrict_point)
 template <typename T>
-__device__ __forceinline__ void residual(const View<T>& V, T* r) {
+__device__ __forceinline__ void residual(const View<T>& V, T* r, bool half) {
   const TailLevel<T>& L = V.L;
   const T* x = V.x();
   const T* b = V.b();
@@ -242,6 +243,10 @@ __device__ __forceinline__ void residual(const View<T>& V, T* r) {
     const int q = quot(t, ip), p = t - q * L.pitch;
     const int i = p < hx ? 2 * p : 2 * (p - hx) + 1;
     if (i >= nx) continue;
+    if (half && ((i + V.tab()[2 * q + 1].y) & 1)) {
+      r[t] = T(0);
+      continue;
+    }
     const int4 ra = V.tab()[2 * q];
     const int row = q * L.pitch;
     T ym, yp, zm, zp;
@@ -739,7 +744,7 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
       sweep(V, h & 1);
       sync(l);
     }
-    residual(V, scr);
+    residual(V, scr, A.pre > 0 && sizeof(T) == sizeof(double));
     sync(l);
     restrict_rows(V, View<T>(A.L[l + 1], sm, rank), base, A.oscr, l + 1 == last, A.pre > 0);
     sync(l);
