@@ -396,7 +396,7 @@ __device__ __forceinline__ R plane_normal(const R* __restrict__ m, const R* __re
   const R gz = ((p[e] - m[e]) + (p[e - sd] - m[e - sd])) * q;
   // tangential terms in axis order, as for the z-face
   const R sq = gd * gd + gt * gt + gz * gz;
-  return gd / (sqrt(sq) + epsn);
+  return quotient(gd, root(sq) + epsn);
 }
 
 // normal on the face between plane c (below) and plane p (above)
@@ -410,7 +410,7 @@ __device__ __forceinline__ R z_normal(const R* __restrict__ c, const R* __restri
   const R gx = ((p[e + 1] - p[e - 1]) + (c[e + 1] - c[e - 1])) * q;
   const R gy = ((p[e + P1::PX] - p[e - P1::PX]) + (c[e + P1::PX] - c[e - P1::PX])) * q;
   const R sq = gd * gd + gx * gx + gy * gy;
-  return gd / (sqrt(sq) + epsn);
+  return quotient(gd, root(sq) + epsn);
 }
 
 // binomial weights of K passes of [1,2,1]/4 on an axis of n cells (identity
@@ -534,25 +534,23 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 4 : 2)
       }
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
-        // central difference of the sigma field (Eq. 5 as a cell field).  In
-        // float it is taken as dsigma/dT (T+ - T-), the same number for the
-        // linear sigma(T): the difference of two neighbouring temperatures is
-        // exact, while sigma0 + dsigma/dT (T - T0) rounded to float at
-        // sigma ~ 1.9 keeps only ~4 digits of a variation of ~1e-3
-        if (conc) {
-          // sigma(c, T) of Eq. 5: in float the exact neighbour differences
-          // again, in double the difference of the two cells' sigma values
-          if (sizeof(R) == 4) sv[d] = (ph.dsdT * (TP[d] - TM[d]) + ph.dsdc * (cP[d] - cM[d])) * i2h;
-          else sv[d] = (sigma_rc(TP[d], cP[d], ph) - sigma_rc(TM[d], cM[d], ph)) * i2h;
-        } else if (sizeof(R) == 4) {
-          sv[d] = ph.dsdT * (TP[d] - TM[d]) * i2h;
-        } else {
-          sv[d] = (sigma_r(TP[d], ph) - sigma_r(TM[d], ph)) * i2h;
-        }
+        // central difference of the sigma field (Eq. 5 as a cell field), taken
+        // as dsigma/dT (T+ - T-) (+ dsigma/dc (c+ - c-)), the same number for
+        // the linear sigma(c, T): the difference of two neighbouring
+        // temperatures is exact, while sigma0 + dsigma/dT (T - T0) rounded to
+        // float at sigma ~ 1.9 keeps only ~4 digits of a variation of ~1e-3
+        if (conc) sv[d] = (ph.dsdT * (TP[d] - TM[d]) + ph.dsdc * (cP[d] - cM[d])) * i2h;
+        else sv[d] = ph.dsdT * (TP[d] - TM[d]) * i2h;
       }
-      R gn = sqrt(gv[0] * gv[0] + gv[1] * gv[1] + gv[2] * gv[2]);
-      R tn = sqrt(tv[0] * tv[0] + tv[1] * tv[1] + tv[2] * tv[2]) + epsn;
-      R n0 = tv[0] / tn, n1 = tv[1] / tn, n2 = tv[2] / tn;
+      R gn = root(gv[0] * gv[0] + gv[1] * gv[1] + gv[2] * gv[2]);
+      R tn = root(tv[0] * tv[0] + tv[1] * tv[1] + tv[2] * tv[2]) + epsn;
+      R n0, n1, n2;
+      if (sizeof(R) == 8) {
+        tn = quotient(R(1), tn);
+        n0 = tv[0] * tn, n1 = tv[1] * tn, n2 = tv[2] * tn;
+      } else {
+        n0 = tv[0] / tn, n1 = tv[1] / tn, n2 = tv[2] / tn;
+      }
       R ns = n0 * sv[0] + n1 * sv[1] + n2 * sv[2];
       M0[c] = gn * (sv[0] - n0 * ns);
       M1[c] = gn * (sv[1] - n1 * ns);
@@ -638,9 +636,13 @@ __device__ __forceinline__ void scal_flux(const R* av, const R* tv, R U, const P
                                           R& Fa, R& FT, R& Df) {
   Fa = upwind_flux(U, av, ph.eps_a);
   FT = upwind_flux(U, tv, ph.eps_T);
-  const R lL = mixr(av[2], ph.lam), lR = mixr(av[3], ph.lam);
-  const R lf = R(2) * lL * lR / (lL + lR);
-  Df = lf * (tv[3] - tv[2]) * ph.ih;
+  const R lL = mixr(av[2], ph.lam, ph.dlam), lR = mixr(av[3], ph.lam, ph.dlam);
+  if (sizeof(R) == 8) {
+    Df = quotient((lL * lR) * ((tv[3] - tv[2]) * (R(2) * ph.ih)), lL + lR);
+  } else {
+    const R lf = R(2) * lL * lR / (lL + lR);
+    Df = lf * (tv[3] - tv[2]) * ph.ih;
+  }
 }
 
 template <typename R>
@@ -763,19 +765,34 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 4 : 2)
     __syncthreads();
     if (col) {
       const int c = (k * ny + j) * nx + i;
-      R Ra = -((S.fx[0][ty][tx + 1] - S.fx[0][ty][tx]) * ih +
-               (S.fy[0][ty + 1][tx] - S.fy[0][ty][tx]) * ih + (fz1[0] - fz0[0]) * ih);
-      R RT = -((S.fx[1][ty][tx + 1] - S.fx[1][ty][tx]) * ih +
-               (S.fy[1][ty + 1][tx] - S.fy[1][ty][tx]) * ih + (fz1[1] - fz0[1]) * ih);
-      const R Dif = (S.fx[2][ty][tx + 1] - S.fx[2][ty][tx]) * ih +
-                    (S.fy[2][ty + 1][tx] - S.fy[2][ty][tx]) * ih + (fz1[2] - fz0[2]) * ih;
       const R al = wa[3];
-      const R rcp = mixr(al, ph.rcp);
-      RT += Dif / rcp;
-      if (qamp != R(0)) {
-        const R gz = (wa[4] - wa[2]) * i2h;
-        const R gn = sqrt(gx * gx + gy * gy + gz * gz);
-        RT += qcol * gn / rcp;
+      const R rcp = mixr(al, ph.rcp, ph.drcp);
+      R Ra, RT;
+      if (sizeof(R) == 8) {
+        Ra = -(((S.fx[0][ty][tx + 1] - S.fx[0][ty][tx]) +
+                (S.fy[0][ty + 1][tx] - S.fy[0][ty][tx])) + (fz1[0] - fz0[0])) * ih;
+        RT = -(((S.fx[1][ty][tx + 1] - S.fx[1][ty][tx]) +
+                (S.fy[1][ty + 1][tx] - S.fy[1][ty][tx])) + (fz1[1] - fz0[1])) * ih;
+        R src = (((S.fx[2][ty][tx + 1] - S.fx[2][ty][tx]) +
+                  (S.fy[2][ty + 1][tx] - S.fy[2][ty][tx])) + (fz1[2] - fz0[2])) * ih;
+        if (qamp != R(0)) {
+          const R gz = (wa[4] - wa[2]) * i2h;
+          src += qcol * root(gx * gx + gy * gy + gz * gz);
+        }
+        RT += quotient(src, rcp);
+      } else {
+        Ra = -((S.fx[0][ty][tx + 1] - S.fx[0][ty][tx]) * ih +
+               (S.fy[0][ty + 1][tx] - S.fy[0][ty][tx]) * ih + (fz1[0] - fz0[0]) * ih);
+        RT = -((S.fx[1][ty][tx + 1] - S.fx[1][ty][tx]) * ih +
+               (S.fy[1][ty + 1][tx] - S.fy[1][ty][tx]) * ih + (fz1[1] - fz0[1]) * ih);
+        const R Dif = (S.fx[2][ty][tx + 1] - S.fx[2][ty][tx]) * ih +
+                      (S.fy[2][ty + 1][tx] - S.fy[2][ty][tx]) * ih + (fz1[2] - fz0[2]) * ih;
+        RT += Dif / rcp;
+        if (qamp != R(0)) {
+          const R gz = (wa[4] - wa[2]) * i2h;
+          const R gn = sqrt(gx * gx + gy * gy + gz * gz);
+          RT += qcol * gn / rcp;
+        }
       }
       const R Ea = al + dt * Ra;
       const R ET = wt[3] + dt * RT;
@@ -911,7 +928,7 @@ __global__ void __launch_bounds__(kThreads)
   stage<3, F_EVEN, 0>(S.c, X.c, g, tb);
   stage<1, F_EVEN, 0>(S.D, X.alpha, g, tb);
   __syncthreads();
-  for (int e = flat_tid(); e < Tile<1>::N; e += kThreads) S.D[e] = mixr(S.D[e], ph.diff_c);
+  for (int e = flat_tid(); e < Tile<1>::N; e += kThreads) S.D[e] = mixr(S.D[e], ph.diff_c, ph.ddiff);
   const bool in = tile_interior(g, 3);
   __syncthreads();
   const R dt = (R)dtp[0];
@@ -983,7 +1000,7 @@ struct MomZ {
   R v[3][Plane<3>::N];    // v planes (m mod 3)
   R w[3][Plane<3>::N];    // w planes (m mod 3)
   R al[4][Plane<1>::N];   // alpha (m mod 4)
-  R mu[3][Plane<1>::N];   // mu(alpha) (m mod 3)
+  R mu[3][Plane<1>::N];   // viscosity measure (m mod 3), see mz_mu
   // fluxes of the current plane, [0] advective, [1] viscous
   R c0[2][kZY][kZX + 1];    // u: centre fluxes of cells x0-1 .. x0+31
   R e0y[2][kZY + 1][kZX];   // u: low y-edges of the faces, rows y0 .. y0+8
@@ -1012,6 +1029,21 @@ __device__ __forceinline__ R cell_at(const R* __restrict__ a, const Geo& g, cons
   return ld_rule<KIND, 0>(a, g, tb, i, j, k);
 }
 
+// What the planes hold for the viscosity: mu(alpha) in float; in double the
+// clamped phase fraction, of which mu is linear (so that the mean over four
+// cells and the densities come from it in two operations)
+template <typename R>
+__device__ __forceinline__ R mz_mu(R alpha, const PhysR<R>& ph) {
+  return sizeof(R) == 8 ? clamp01(alpha) : mixr(alpha, ph.mu, ph.dmu);
+}
+
+// viscous flux 2 mu du/dx of a face pair in a cell
+template <typename R>
+__device__ __forceinline__ R mz_visc(R mu, R du, const PhysR<R>& ph) {
+  if (sizeof(R) == 8) return ((R(2) * ph.ih * ph.dmu) * mu + R(2) * ph.ih * ph.mu[0]) * du;
+  return R(2) * mu * du * ph.ih;
+}
+
 // normal flux of a component at the centre of local cell (lx, ly) along the
 // in-plane axis A: WENO5 of the six faces around it with the mean of the
 // cell's two faces as the advecting velocity; viscous 2 mu du/dx_A
@@ -1024,7 +1056,7 @@ __device__ __forceinline__ void mz_centre(const R* __restrict__ q, const R* __re
   for (int m = 0; m < 6; ++m) v[m] = q[A == 0 ? P3::at(lx + m - 2, ly) : P3::at(lx, ly + m - 2)];
   const R Uc = R(0.5) * (v[2] + v[3]);
   Fa = upwind_flux(Uc, v, ph.eps_u);
-  Fv = R(2) * mu[Plane<1>::at(lx, ly)] * (v[3] - v[2]) * ph.ih;
+  Fv = mz_visc(mu[Plane<1>::at(lx, ly)], v[3] - v[2], ph);
 }
 
 // the same along z from the column window v[0..5] (faces k-2 .. k+3 of cell k)
@@ -1033,21 +1065,26 @@ __device__ __forceinline__ void mz_centre_col(const R* v, R mu_c, const PhysR<R>
                                               R& Fv) {
   const R Uc = R(0.5) * (v[2] + v[3]);
   Fa = upwind_flux(Uc, v, ph.eps_u);
-  Fv = R(2) * mu_c * (v[3] - v[2]) * ph.ih;
+  Fv = mz_visc(mu_c, v[3] - v[2], ph);
 }
 
 // tangential flux at an edge: v[0..5] the advected component at offsets -3..2
 // across the edge (v[2] below, v[3] above), ut_lo / ut_hi the crossing
-// component on the two faces meeting there, mue the mean viscosity of the
-// four cells around the edge
+// component on the two faces meeting there, m0 .. m3 the viscosity measures of
+// the four cells around the edge
 template <typename R>
-__device__ __forceinline__ void mz_edge(const R* v, R ut_lo, R ut_hi, R mue, const PhysR<R>& ph,
-                                        R& Fa, R& Fv) {
+__device__ __forceinline__ void mz_edge(const R* v, R ut_lo, R ut_hi, R m0, R m1, R m2, R m3,
+                                        const PhysR<R>& ph, R& Fa, R& Fv) {
+  const R mue = sizeof(R) == 8
+                    ? (R(0.25) * ph.ih * ph.dmu) * ((m0 + m1) + (m2 + m3)) + ph.ih * ph.mu[0]
+                    : R(0.25) * (m0 + m1 + m2 + m3);
   const R Ue = R(0.5) * (ut_lo + ut_hi);
   Fa = upwind_flux(Ue, v, ph.eps_u);
-  const R dud_dt = (v[3] - v[2]) * ph.ih;
-  const R dut_dd = (ut_hi - ut_lo) * ph.ih;
-  Fv = mue * (dud_dt + dut_dd);
+  if (sizeof(R) == 8) {
+    Fv = mue * ((v[3] - v[2]) + (ut_hi - ut_lo));
+  } else {
+    Fv = mue * fma(ut_hi - ut_lo, ph.ih, (v[3] - v[2]) * ph.ih);
+  }
 }
 
 template <int T, typename R>
@@ -1065,9 +1102,8 @@ __device__ __forceinline__ void mz_e0y(const R* U, const R* V, const R* mu, cons
   using P1 = Plane<1>;
   R v[6];
   mz_gather<1>(U, lx, ly, v);
-  const R mue = R(0.25) * (mu[P1::at(lx, ly)] + mu[P1::at(lx - 1, ly)] + mu[P1::at(lx, ly - 1)] +
-                           mu[P1::at(lx - 1, ly - 1)]);
-  mz_edge(v, V[P3::at(lx - 1, ly)], V[P3::at(lx, ly)], mue, ph, F[0], F[1]);
+  mz_edge(v, V[P3::at(lx - 1, ly)], V[P3::at(lx, ly)], mu[P1::at(lx, ly)], mu[P1::at(lx - 1, ly)],
+          mu[P1::at(lx, ly - 1)], mu[P1::at(lx - 1, ly - 1)], ph, F[0], F[1]);
 }
 
 // v's low x-edge at face (lx, ly) of plane k
@@ -1078,9 +1114,8 @@ __device__ __forceinline__ void mz_e1x(const R* U, const R* V, const R* mu, cons
   using P1 = Plane<1>;
   R v[6];
   mz_gather<0>(V, lx, ly, v);
-  const R mue = R(0.25) * (mu[P1::at(lx, ly)] + mu[P1::at(lx, ly - 1)] + mu[P1::at(lx - 1, ly)] +
-                           mu[P1::at(lx - 1, ly - 1)]);
-  mz_edge(v, U[P3::at(lx, ly - 1)], U[P3::at(lx, ly)], mue, ph, F[0], F[1]);
+  mz_edge(v, U[P3::at(lx, ly - 1)], U[P3::at(lx, ly)], mu[P1::at(lx, ly)], mu[P1::at(lx, ly - 1)],
+          mu[P1::at(lx - 1, ly)], mu[P1::at(lx - 1, ly - 1)], ph, F[0], F[1]);
 }
 
 // w's low x-edge (T = 0) or y-edge (T = 1) at z-face (lx, ly) of height k;
@@ -1093,8 +1128,8 @@ __device__ __forceinline__ void mz_e2(const R* W, const R* Qk, const R* Qm, cons
   R v[6];
   mz_gather<T>(W, lx, ly, v);
   const int e = P1::at(lx, ly), et = T == 0 ? P1::at(lx - 1, ly) : P1::at(lx, ly - 1);
-  const R mue = R(0.25) * (muk[e] + mum[e] + muk[et] + mum[et]);
-  mz_edge(v, Qm[P3::at(lx, ly)], Qk[P3::at(lx, ly)], mue, ph, F[0], F[1]);
+  mz_edge(v, Qm[P3::at(lx, ly)], Qk[P3::at(lx, ly)], muk[e], mum[e], muk[et], mum[et], ph, F[0],
+          F[1]);
 }
 
 // u's (D = 0) or v's (D = 1) z-edge at the face column (lx, ly) between
@@ -1106,18 +1141,44 @@ __device__ __forceinline__ void mz_ez(const R* v, const R* Wu, const R* muu, con
   using P3 = Plane<3>;
   using P1 = Plane<1>;
   const int e = P1::at(lx, ly), ed = D == 0 ? P1::at(lx - 1, ly) : P1::at(lx, ly - 1);
-  const R mue = R(0.25) * (muu[e] + muu[ed] + mud[e] + mud[ed]);
   const int w1 = P3::at(lx, ly), w0 = D == 0 ? P3::at(lx - 1, ly) : P3::at(lx, ly - 1);
-  mz_edge(v, Wu[w0], Wu[w1], mue, ph, F[0], F[1]);
+  mz_edge(v, Wu[w0], Wu[w1], muu[e], muu[ed], mud[e], mud[ed], ph, F[0], F[1]);
 }
 
+// advection A = -(a0 + a1 + a2)/h and viscous force V = (v0 + v1 + v2)/h from
+// the flux differences of a control volume's three axes
+#define MZ_SUM(a0, a1, a2, v0, v1, v2)  \
+  R A, V;                               \
+  if (sizeof(R) == 8) {                 \
+    A = -(((a0) + (a1)) + (a2)) * ih;   \
+    V = (((v0) + (v1)) + (v2)) * ih;    \
+  } else {                              \
+    A = R(0) - (a0) * ih;               \
+    V = R(0) + (v0) * ih;               \
+    A -= (a1) * ih;                     \
+    V += (v1) * ih;                     \
+    A -= (a2) * ih;                     \
+    V += (v2) * ih;                     \
+  }
+
 // the forces on a D-face between cell L and cell R and the new face velocity
+// (mL, mR: the cells' viscosity measures, in double their clamped phase
+// fractions; sigma_f is then the linear sigma(c, T) of the mean T and c)
 template <int D, typename R>
 __device__ __forceinline__ void mz_update(const PhysR<R>& ph, bool conc, R A, R V, R alL, R alR,
-                                          R TL, R TR, R cL, R cR, R kL, R kR, R ML, R MR, R uf,
-                                          R dt, R& us, R& phi) {
+                                          R mL, R mR, R TL, R TR, R cL, R cR, R kL, R kR, R ML,
+                                          R MR, R uf, R dt, R& us, R& phi) {
   const R ih = ph.ih;
-  const R rho_f = R(0.5) * (mixr(alL, ph.rho) + mixr(alR, ph.rho));
+  if (sizeof(R) == 8) {
+    const R rho_f = (R(0.5) * ph.drho) * (mL + mR) + ph.rho[0];
+    R sig_f = ph.dsdT * (R(0.5) * (TL + TR) - ph.T0) + ph.sigma0;
+    if (conc) sig_f += ph.dsdc * (R(0.5) * (cL + cR) - ph.c0);
+    const R fn = (sig_f * (R(-0.5) * ih)) * ((kL + kR) * (alR - alL));
+    phi = (V + fn) + R(0.5) * (ML + MR);   // before 1/rho_f (the adjoint's density term)
+    us = uf + dt * (A + quotient(phi, rho_f) + ph.g[D]);
+    return;
+  }
+  const R rho_f = R(0.5) * (mixr(alL, ph.rho, ph.drho) + mixr(alR, ph.rho, ph.drho));
   const R sig_f = conc ? R(0.5) * (sigma_rc(TL, cL, ph) + sigma_rc(TR, cR, ph))
                        : R(0.5) * (sigma_r(TL, ph) + sigma_r(TR, ph));
   const R kap_f = R(0.5) * (kL + kR);
@@ -1125,7 +1186,7 @@ __device__ __forceinline__ void mz_update(const PhysR<R>& ph, bool conc, R A, R 
   const R fn = -sig_f * kap_f * jump;
   const R fM = R(0.5) * (ML + MR);
   us = uf + dt * (A + (V + fn + fM) / rho_f + ph.g[D]);
-  phi = V + fn + fM;   // the force sum before 1/rho_f (the adjoint's density term)
+  phi = V + fn + fM;
 }
 
 template <typename R>
@@ -1159,7 +1220,7 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 3 : 2)
   for (int m = z0 - 1; m <= z0 + 1; ++m) stage_plane<1, F_EVEN>(S.al[mod4(m)], X.alpha, g, tb, in, m);
   __syncthreads();
   for (int m = z0 - 1; m <= z0; ++m)
-    for (int e = tx + kZX * ty; e < P1::N; e += kZT) S.mu[mod3(m)][e] = mixr(S.al[mod4(m)][e], ph.mu);
+    for (int e = tx + kZX * ty; e < P1::N; e += kZT) S.mu[mod3(m)][e] = mz_mu(S.al[mod4(m)][e], ph);
   __syncthreads();
   // column windows: after the warm-up cu[0..5] = u at heights k-2 .. k+3
   R cu[7], cv[7], cw[7];
@@ -1205,11 +1266,11 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 3 : 2)
         nw = col_vel<2>(X.u[2], g, i, j, k + 4);
       }
     }
-    // mu of plane k + 1 (alpha k + 1 arrived with the previous step's copies)
+    // the viscosity measure of plane k + 1 (alpha k + 1 arrived with the previous step's copies)
     {
       const R* __restrict__ a1 = S.al[mod4(k + 1)];
       R* __restrict__ m1 = S.mu[mod3(k + 1)];
-      for (int e = tx + kZX * ty; e < P1::N; e += kZT) m1[e] = mixr(a1[e], ph.mu);
+      for (int e = tx + kZX * ty; e < P1::N; e += kZT) m1[e] = mz_mu(a1[e], ph);
     }
     __syncthreads();
     const R* __restrict__ Uk = S.u[mod3(k)];
@@ -1300,6 +1361,7 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 3 : 2)
       const R* __restrict__ ak = S.al[mod4(k)];
       const R* __restrict__ am = S.al[mod4(k - 1)];
       const int e1 = P1::at(tx, ty), e3 = P3::at(tx, ty);
+      const R mR = mk[e1];
       const R alR = ak[e1], TR = X.T[c], kR = kappa[c], cR = conc ? X.c[c] : R(0);
       R us, phv;
       // u on the x-face (i, j, k)
@@ -1307,18 +1369,15 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 3 : 2)
         us0[c] = R(0);
         if (ph0) ph0[c] = R(0);
       } else {
-        R A = R(0) - (S.c0[0][ty][tx + 1] - S.c0[0][ty][tx]) * ih;
-        R V = R(0) + (S.c0[1][ty][tx + 1] - S.c0[1][ty][tx]) * ih;
-        A -= (S.e0y[0][ty + 1][tx] - S.e0y[0][ty][tx]) * ih;
-        V += (S.e0y[1][ty + 1][tx] - S.e0y[1][ty][tx]) * ih;
-        A -= (ez0h[0] - ez0[0]) * ih;
-        V += (ez0h[1] - ez0[1]) * ih;
+        MZ_SUM(S.c0[0][ty][tx + 1] - S.c0[0][ty][tx], S.e0y[0][ty + 1][tx] - S.e0y[0][ty][tx],
+               ez0h[0] - ez0[0], S.c0[1][ty][tx + 1] - S.c0[1][ty][tx],
+               S.e0y[1][ty + 1][tx] - S.e0y[1][ty][tx], ez0h[1] - ez0[1])
         const bool d = i >= 1;
         const R TL = d ? X.T[c - 1] : ld_T(X.T, g, tb, i - 1, j, k);
         const R kL = d ? kappa[c - 1] : ld_even(kappa, g, i - 1, j, k);
         const R cL = conc ? (d ? X.c[c - 1] : ld_even(X.c, g, i - 1, j, k)) : R(0);
         const R ML = d ? M0[c - 1] : ld_even(M0, g, i - 1, j, k);
-        mz_update<0>(ph, conc, A, V, ak[e1 - 1], alR, TL, TR, cL, cR, kL, kR, ML, M0[c], Uk[e3],
+        mz_update<0>(ph, conc, A, V, ak[e1 - 1], alR, mk[e1 - 1], mR, TL, TR, cL, cR, kL, kR, ML, M0[c], Uk[e3],
                      dt, us, phv);
         us0[c] = us;
         if (ph0) ph0[c] = phv;
@@ -1328,18 +1387,15 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 3 : 2)
         us1[c] = R(0);
         if (ph1) ph1[c] = R(0);
       } else {
-        R A = R(0) - (S.c1[0][ty + 1][tx] - S.c1[0][ty][tx]) * ih;
-        R V = R(0) + (S.c1[1][ty + 1][tx] - S.c1[1][ty][tx]) * ih;
-        A -= (S.e1x[0][ty][tx + 1] - S.e1x[0][ty][tx]) * ih;
-        V += (S.e1x[1][ty][tx + 1] - S.e1x[1][ty][tx]) * ih;
-        A -= (ez1h[0] - ez1[0]) * ih;
-        V += (ez1h[1] - ez1[1]) * ih;
+        MZ_SUM(S.c1[0][ty + 1][tx] - S.c1[0][ty][tx], S.e1x[0][ty][tx + 1] - S.e1x[0][ty][tx],
+               ez1h[0] - ez1[0], S.c1[1][ty + 1][tx] - S.c1[1][ty][tx],
+               S.e1x[1][ty][tx + 1] - S.e1x[1][ty][tx], ez1h[1] - ez1[1])
         const bool d = j >= 1;
         const R TL = d ? X.T[c - nx] : ld_T(X.T, g, tb, i, j - 1, k);
         const R kL = d ? kappa[c - nx] : ld_even(kappa, g, i, j - 1, k);
         const R cL = conc ? (d ? X.c[c - nx] : ld_even(X.c, g, i, j - 1, k)) : R(0);
         const R ML = d ? M1[c - nx] : ld_even(M1, g, i, j - 1, k);
-        mz_update<1>(ph, conc, A, V, ak[e1 - P1::PX], alR, TL, TR, cL, cR, kL, kR, ML, M1[c],
+        mz_update<1>(ph, conc, A, V, ak[e1 - P1::PX], alR, mk[e1 - P1::PX], mR, TL, TR, cL, cR, kL, kR, ML, M1[c],
                      Vk[e3], dt, us, phv);
         us1[c] = us;
         if (ph1) ph1[c] = phv;
@@ -1350,13 +1406,10 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 3 : 2)
         us2[c] = R(0);
         if (ph2) ph2[c] = R(0);
       } else {
-        R A = R(0) - (cc2h[0] - cc2[0]) * ih;
-        R V = R(0) + (cc2h[1] - cc2[1]) * ih;
-        A -= (S.e2x[0][ty][tx + 1] - S.e2x[0][ty][tx]) * ih;
-        V += (S.e2x[1][ty][tx + 1] - S.e2x[1][ty][tx]) * ih;
-        A -= (S.e2y[0][ty + 1][tx] - S.e2y[0][ty][tx]) * ih;
-        V += (S.e2y[1][ty + 1][tx] - S.e2y[1][ty][tx]) * ih;
-        mz_update<2>(ph, conc, A, V, am[e1], alR, TL2, TR, cL2, cR, kL2, kR, ML2, M2R, Wk[e3], dt,
+        MZ_SUM(cc2h[0] - cc2[0], S.e2x[0][ty][tx + 1] - S.e2x[0][ty][tx],
+               S.e2y[0][ty + 1][tx] - S.e2y[0][ty][tx], cc2h[1] - cc2[1],
+               S.e2x[1][ty][tx + 1] - S.e2x[1][ty][tx], S.e2y[1][ty + 1][tx] - S.e2y[1][ty][tx])
+        mz_update<2>(ph, conc, A, V, am[e1], alR, mm[e1], mR, TL2, TR, cL2, cR, kL2, kR, ML2, M2R, Wk[e3], dt,
                      us, phv);
         us2[c] = us;
         if (ph2) ph2[c] = phv;
