@@ -182,6 +182,8 @@ struct fvm_ctx {
   void* beta0[3];        // fine beta (double in F64, float in MIXED)
   float* e32;            // MIXED: inner correction
   float* r32;            // MIXED: inner right-hand side
+  double* rd;            // MIXED: the residual that is updated (null: formed from p each time)
+  float* y;              // MIXED: the first sweep beside it
   // hierarchy
   int nlev;
   LevelShape shp[kMaxLevels];
@@ -237,6 +239,7 @@ struct fvm_ctx {
 namespace {
 
 constexpr int kProfSlots = 4096;
+constexpr long long kUpdateCells = 1 << 19;   // see residual_updated()
 constexpr int kRecords = 4;   // solve records: the three stages of a step, a lone solve
 
 void prof_fold(fvm_ctx* c) {
@@ -349,6 +352,9 @@ size_t plan_workspace(const fvm_params& p, fvm_ctx* c) {
     c->b = (double*)(w + o_b);
     c->e32 = mixed ? (float*)(w + o_e) : nullptr;
     c->r32 = mixed ? (float*)(w + o_r) : nullptr;
+    // the solves leave as and tmp (beside each other: N doubles) and M free
+    c->rd = mixed && N >= kUpdateCells ? (double*)c->as : nullptr;
+    c->y = mixed ? (float*)c->M[0] : nullptr;
     c->nlev = nl;
     for (int l = 0; l < nl; ++l) c->shp[l] = lv[l];
     for (int l = 1; l < nl; ++l) {
@@ -463,16 +469,19 @@ template <typename T>
 struct SweepFold {
   const MGLevel<T>* corr = nullptr;   // first sweep: the coarse correction of this level (prolongation)
   bool zero = false;                  // first sweep: x starts at 0 (zeroes the other colour)
-  bool skip_first = false;            // first sweep: already taken (by k_residual64)
+  bool skip_first = false;            // first sweep: already taken (by the residual pass)
+  const T* xin = nullptr;             // second sweep: the first one's values are here (its colour only)
+  bool keep = false;                  // last sweep with addp: store x as well
   const int* gate = nullptr;          // first sweep: skipped on the device once *gate >= gate_min
   int gate_min = 0;
   double* addp = nullptr;             // last sweep: p += x (the mixed form's float level 0)
 };
 
-inline void addp_sweep(fvm_ctx* c, int kg, const MGLevel<float>& L, int colour, double* p) {
-  TIMED(c, kg, 1, launch_gs_addp(L, colour, p, c->stream));
+inline void addp_sweep(fvm_ctx* c, int kg, const MGLevel<float>& L, int colour, double* p,
+                       bool keep) {
+  TIMED(c, kg, 1, launch_gs_addp(L, colour, p, keep, c->stream));
 }
-inline void addp_sweep(fvm_ctx*, int, const MGLevel<double>&, int, double*) {}
+inline void addp_sweep(fvm_ctx*, int, const MGLevel<double>&, int, double*, bool) {}
 
 // `iters` Gauss-Seidel iterations on level l: a sweep of colour `first`,
 // then one of the other colour.  The first sweep can apply the coarse
@@ -492,9 +501,11 @@ void smooth(fvm_ctx* c, MGLevel<T>& L, int l, int iters, int first,
     else if (t == 0 && f.zero)
       TIMED(c, kg, 1, launch_gs_zero<T>(L, colour, c->stream));
     else if (t == last && f.addp)
-      addp_sweep(c, kg, L, colour, f.addp);
+      addp_sweep(c, kg, L, colour, f.addp, f.keep);
     else if (t == 0 && f.gate)
       TIMED(c, kg, 1, launch_gs<T>(L, colour, c->stream, f.gate, f.gate_min));
+    else if (t == 1 && f.xin)
+      TIMED(c, kg, 1, launch_gs<T>(L, colour, c->stream, nullptr, 0, f.xin));
     else
       TIMED(c, kg, 1, launch_gs<T>(L, colour, c->stream));
   }
@@ -557,7 +568,8 @@ void coarsen_betas(fvm_ctx* c, MGLevel<T>* Ls) {
 // first sweep already taken (by k_residual64 in the mixed form, or skipped
 // because it would repeat the previous cycle's last sweep), or with that skip
 // decided on the device (FP64 solve graph: from the second cycle on).
-enum { kStartAsIs = 0, kStartZero = 1, kStartFirstSwept = 2, kStartGated = 3 };
+// kStartFirstAside: the first sweep was taken into c->y (colour 0 only).
+enum { kStartAsIs = 0, kStartZero = 1, kStartFirstSwept = 2, kStartGated = 3, kStartFirstAside = 4 };
 
 // a cycle's first finest-level sweep repeats the previous cycle's last one
 // (same colour, same right-hand side, the other colour unchanged) when both
@@ -572,14 +584,25 @@ bool residual_takes_first_sweep(const fvm_ctx* c) {
   return c->prm.mg_pre > 0 && c->nlev > 1 && c->prm.mx_inner_cycles > 0;
 }
 
+// the mixed form updates its double residual (k_residual_update) on grids of at
+// least kUpdateCells cells when there is room for it (c->rd); its first sweep then
+// goes to c->y, which needs a second sweep on that level to read it
+bool residual_updated(const fvm_ctx* c) { return c->rd != nullptr; }
+bool first_sweep_aside(const fvm_ctx* c) {
+  return residual_updated(c) && residual_takes_first_sweep(c) && c->prm.mg_pre > 1;
+}
+
 // the residual r = b - L p (double, stored as float) of the mixed form, with
 // the next inner solve's first sweep when residual_takes_first_sweep()
-void mixed_residual(fvm_ctx* c, double* p, const double* b, float* const* be) {
-  const bool f = residual_takes_first_sweep(c);
+void mixed_residual(fvm_ctx* c, double* p, const double* b, float* const* be,
+                    const int* gate = nullptr) {
+  float* first = nullptr;
+  if (residual_updated(c)) first = first_sweep_aside(c) ? c->y : nullptr;
+  else if (residual_takes_first_sweep(c)) first = c->e32;
   const float w32[3] = {(float)c->g.w[0], (float)c->g.w[1], (float)c->g.w[2]};
   TIMED(c, FVM_K_RESIDUAL64, 2,
-        launch_residual64(c->g, p, b, be, c->r32, c->partial, c->scal + 1, c->stream,
-                          f ? c->e32 : nullptr, w32));
+        launch_residual64(c->g, p, b, be, c->r32, c->partial, c->scal + 1, c->stream, first, w32,
+                          c->rd, gate));
 }
 
 // start: how level l's x starts (kStart*); addp: add level 0's x to p at the
@@ -606,7 +629,8 @@ void vcycle(fvm_ctx* c, MGLevel<T>* Ls, int l, double coarse_rtol, int start = k
   } else {
     SweepFold<T> fpre;
     fpre.zero = fold_zero;
-    fpre.skip_first = start == kStartFirstSwept;
+    fpre.skip_first = start == kStartFirstSwept || start == kStartFirstAside;
+    if (start == kStartFirstAside) fpre.xin = (const T*)c->y;
     if (start == kStartGated) {
       // the controller counts the cycle being run: 1 in the first
       fpre.gate = &c->ctl->iters;
@@ -625,6 +649,7 @@ void vcycle(fvm_ctx* c, MGLevel<T>* Ls, int l, double coarse_rtol, int start = k
       SweepFold<T> fpost;
       fpost.corr = &Ls[l + 1];
       fpost.addp = fold_add ? addp : nullptr;
+      fpost.keep = addp && residual_updated(c);
       smooth<T>(c, Ls[l], l, post, 1, fpost);
     } else {
       TIMED(c, l == 0 ? FVM_K_PROLONG_FINE : FVM_K_PROLONG_COARSE, 1,
@@ -706,7 +731,8 @@ void refine_once(fvm_ctx* c, MGLevel<float>* Ls, const float* alpha, double* p, 
   // of the first cycle (or that sweep was taken by the residual kernel), the
   // addition on the last sweep of the last one
   const int m = c->prm.mx_inner_cycles;
-  const int start0 = residual_takes_first_sweep(c) ? kStartFirstSwept : kStartZero;
+  int start0 = residual_takes_first_sweep(c) ? kStartFirstSwept : kStartZero;
+  if (residual_updated(c)) start0 = first_sweep_aside(c) ? kStartFirstAside : kStartZero;
   // a cycle after the first begins with a colour-0 sweep right after the
   // previous cycle's last one, also of colour 0, on the same right-hand side
   // with the other colour unchanged: it would write the same values again,
@@ -714,7 +740,12 @@ void refine_once(fvm_ctx* c, MGLevel<float>* Ls, const float* alpha, double* p, 
   const int startq = first_sweep_repeats(c) ? kStartFirstSwept : kStartAsIs;
   for (int q = 0; q < m; ++q)
     vcycle<float>(c, Ls, 0, crtol, q == 0 ? start0 : startq, q == m - 1 ? p : nullptr);
-  mixed_residual(c, p, b, be);
+  if (residual_updated(c))
+    TIMED(c, FVM_K_RESIDUAL64, 2,
+          launch_residual_update(Ls[0], c->rd, first_sweep_aside(c) ? c->y : nullptr, c->partial,
+                                 c->scal + 1, c->stream));
+  else
+    mixed_residual(c, p, b, be);
 }
 
 fvm_status solve_mixed(fvm_ctx* c, const float* alpha, double* p, double* b, int* cycles_out,
@@ -743,24 +774,27 @@ fvm_status solve_mixed(fvm_ctx* c, const float* alpha, double* p, double* b, int
   int outer = 0;
   double rel = 0.0;
   mixed_residual(c, p, b, be);
+  bool updated = false;   // the residual is an updated one
   for (;;) {
-    if (fixed > 0) {
-      if (outer == fixed) {
-        double r2;
-        st = read_scalar(c, c->scal + 1, &r2);
-        if (st) return st;
-        rel = sqrt(r2) / bn;
-        break;
-      }
-    } else {
-      double r2;
+    double r2;
+    if (fixed == 0 || outer == fixed) {
       st = read_scalar(c, c->scal + 1, &r2);
       if (st) return st;
       rel = sqrt(r2) / bn;
-      if (!isfinite(rel)) return set_err(c, FVM_EUNSTABLE, "non-finite pressure residual");
-      if (rel <= c->prm.mg_rtol || outer >= c->prm.mg_max_cycles) break;
+      const bool stop = fixed > 0 || !isfinite(rel) || rel <= c->prm.mg_rtol ||
+                        outer >= c->prm.mg_max_cycles;
+      if (stop && updated) {
+        // an updated residual that would stop the solve is formed from p again
+        mixed_residual(c, p, b, be);
+        updated = false;
+        continue;
+      }
+      if (fixed == 0 && !isfinite(rel))
+        return set_err(c, FVM_EUNSTABLE, "non-finite pressure residual");
+      if (stop) break;
     }
     refine_once(c, Ls, alpha, p, b, be, crtol);
+    updated = residual_updated(c);
     ++outer;
   }
   TIMED(c, FVM_K_MISC, 2, launch_sum_field<double>(p, N, false, c->partial, c->scal + 2, s));
@@ -816,6 +850,12 @@ void graph_body(fvm_ctx* c, double* p, cudaGraphConditionalHandle h) {
     hierarchy<float>(c, c->e32, c->r32, be, Ls);
     const double crtol = c->prm.coarse_rtol > 1e-6 ? c->prm.coarse_rtol : 1e-6;
     refine_once(c, Ls, nullptr, p, c->b, be, crtol);
+    if (residual_updated(c)) {
+      TIMED(c, FVM_K_MISC, 1,
+            launch_ctl_check(c->ctl, c->scal + 0, c->scal + 1, c->prm.mg_rtol,
+                             c->prm.mg_max_cycles, fixed, s));
+      mixed_residual(c, p, c->b, be, &c->ctl->verify);
+    }
   } else {
     MGLevel<double> Ls[kMaxLevels];
     double* be[3] = {(double*)c->beta0[0], (double*)c->beta0[1], (double*)c->beta0[2]};

@@ -130,7 +130,8 @@ void launch_diagnostics(const Geo& g, const Phys& ph, Fields<R> X, const double*
 // ----- reductions and multigrid (fvm_mg.cu) ----------------------------------
 // Deterministic two-pass sums: per-block partial sums in `partial`, then one
 // block adds them in a fixed order into *out.
-void launch_sum_partials(const double* partial, int nparts, double* out, cudaStream_t s);
+void launch_sum_partials(const double* partial, int nparts, double* out, cudaStream_t s,
+                         const int* gate = nullptr);
 template <typename T>
 void launch_sum_field(const T* a, long long n, bool squares, double* partial, double* out,
                       cudaStream_t s);
@@ -139,9 +140,10 @@ template <typename T>
 void launch_zero(T* a, long long n, cudaStream_t s);
 
 // gate (optional): the sweep does nothing once *gate >= gate_min
+// xin (optional): the array the neighbours are read from instead of L.x
 template <typename T>
 void launch_gs(const MGLevel<T>& L, int colour, cudaStream_t s, const int* gate = nullptr,
-               int gate_min = 0);
+               int gate_min = 0, const T* xin = nullptr);
 
 
 // half: the last sweep was of colour 1, whose cells' residuals are taken as 0
@@ -161,8 +163,9 @@ void launch_gs_prolong(const MGLevel<T>& F, const MGLevel<T>& C, int colour, cud
 template <typename T>
 void launch_gs_zero(const MGLevel<T>& L, int colour, cudaStream_t s);
 // a float sweep of `colour` that adds the new values of its cells and the
-// values of the other colour to the double p (p += x after the sweep)
-void launch_gs_addp(const MGLevel<float>& L, int colour, double* p, cudaStream_t s);
+// values of the other colour to the double p (p += x after the sweep); store:
+// the new values are written to x as well
+void launch_gs_addp(const MGLevel<float>& L, int colour, double* p, bool store, cudaStream_t s);
 template <typename T>
 void launch_beta_coarsen(const MGLevel<T>& F, const MGLevel<T>& C, cudaStream_t s);
 // The coarse tail of a V-cycle (fvm_tail.cu): the levels from the first one
@@ -231,10 +234,17 @@ void launch_coarse_cg(const MGLevel<T>& L, double* r, double* d, double* Ad, dou
 // ||b - L x||^2 into *out (double), x, b, beta in precision T
 template <typename T>
 void launch_residual_norm2(const MGLevel<T>& L, double* partial, double* out, cudaStream_t s);
-// Mixed form: r = b - L p in double with float beta; writes r32 and ||r||^2
+// Mixed form: r = b - L p in double with float beta; writes r32, with rd the
+// double r too, and ||r||^2.  e32, w32: also the first sweep of the next
+// inner solve.  gate (optional): nothing is done unless *gate.
 void launch_residual64(const Geo& g, const double* p, const double* b, float* const* beta,
                        float* r32, double* partial, double* out, cudaStream_t s,
-                       float* e32 = nullptr, const float* w32 = nullptr);
+                       float* e32 = nullptr, const float* w32 = nullptr, double* rd = nullptr,
+                       const int* gate = nullptr);
+// rd -= L e (L.x) and the same outputs: r32 (L.b), ||r||^2, and with y the next
+// inner solve's first sweep (its colour 0 only)
+void launch_residual_update(const MGLevel<float>& L, double* rd, float* y, double* partial,
+                            double* out, cudaStream_t s);
 void launch_add_correction(long long n, double* p, const float* e, cudaStream_t s);
 
 // ----- device-side control of the pressure solve (fvm_mg.cu) -----------------
@@ -246,7 +256,7 @@ struct SolveCtl {
   int iters;      // cycles (F64) or refinements (MIXED) done
   int status;     // 0, FVM_ENOCONV or FVM_EUNSTABLE
   int zero;       // 1: ||b|| = 0, the solution is set to 0
-  int pad;
+  int verify;     // 1: the updated residual would stop the solve; form it from p
   double rel;     // last relative residual
 };
 void launch_ctl_reset(SolveCtl* ctl, cudaStream_t s);
@@ -255,6 +265,9 @@ void launch_ctl_reset(SolveCtl* ctl, cudaStream_t s);
 void launch_ctl_step(cudaGraphConditionalHandle h, SolveCtl* ctl, const double* bn2,
                      const double* r2, double rtol, int maxit, int fixed,
                      unsigned long long* runs_total, cudaStream_t s);
+// verify = whether the updated residual r2 would stop the solve after this cycle
+void launch_ctl_check(SolveCtl* ctl, const double* bn2, const double* r2, double rtol, int maxit,
+                      int fixed, cudaStream_t s);
 void launch_zero_if_rhs_zero(const SolveCtl* ctl, double* p, long long n, cudaStream_t s);
 // copy the controller into a per-stage record and raise the sticky status
 void launch_ctl_store(const SolveCtl* ctl, SolveCtl* rec, int* sticky, cudaStream_t s);

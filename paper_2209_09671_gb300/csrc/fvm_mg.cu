@@ -64,7 +64,8 @@ __global__ void k_sum_field(const T* __restrict__ a, long long n, int squares,
 }
 
 __global__ void k_sum_partials(const double* __restrict__ partial, int nparts,
-                               double* __restrict__ out) {
+                               double* __restrict__ out, const int* __restrict__ gate) {
+  if (gate && !*gate) return;
   __shared__ double sh[33];
   double acc = 0.0;
   for (int q = threadIdx.x; q < nparts; q += blockDim.x) acc += partial[q];
@@ -72,8 +73,9 @@ __global__ void k_sum_partials(const double* __restrict__ partial, int nparts,
   if (threadIdx.x == 0) *out = s;
 }
 
-void launch_sum_partials(const double* partial, int nparts, double* out, cudaStream_t s) {
-  k_sum_partials<<<1, 1024, 0, s>>>(partial, nparts, out);
+void launch_sum_partials(const double* partial, int nparts, double* out, cudaStream_t s,
+                         const int* gate) {
+  k_sum_partials<<<1, 1024, 0, s>>>(partial, nparts, out, gate);
 }
 
 template <typename T>
@@ -247,9 +249,10 @@ void launch_inv_diag(const MGLevel<T>& L, cudaStream_t s) {
   k_inv_diag<T><<<gs, bs, 0, s>>>(L);
 }
 
-// Gauss-Seidel update of one cell (its colour's neighbours are fixed)
+// Gauss-Seidel update of one cell (its colour's neighbours are fixed), which
+// are read from x
 template <typename T>
-__device__ __forceinline__ void gs_point(const MGLevel<T>& L, int i, int j, int k) {
+__device__ __forceinline__ void gs_point(const MGLevel<T>& L, int i, int j, int k, const T* x) {
   const Geo& g = L.geo;
   const int c = (k * g.n[1] + j) * g.n[0] + i;
   OpNb<T> nb;
@@ -257,8 +260,8 @@ __device__ __forceinline__ void gs_point(const MGLevel<T>& L, int i, int j, int 
   T xlo[3], xhi[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    xlo[d] = L.x[nb.lo[d]];
-    xhi[d] = L.x[nb.hi[d]];
+    xlo[d] = x[nb.lo[d]];
+    xhi[d] = x[nb.hi[d]];
   }
   L.x[c] = gs_value(L, c, nb, xlo, xhi);
 }
@@ -267,7 +270,8 @@ __device__ __forceinline__ void gs_point(const MGLevel<T>& L, int i, int j, int 
 // solve graph skips the first sweep of every cycle after the first, which
 // would repeat the previous cycle's last sweep)
 template <typename T>
-__global__ void k_gs(MGLevel<T> L, int colour, const int* __restrict__ gate, int gate_min) {
+__global__ void k_gs(MGLevel<T> L, int colour, const int* __restrict__ gate, int gate_min,
+                     const T* xin) {
   if (gate && *gate >= gate_min) return;
   const Geo& g = L.geo;
   const int i2 = blockIdx.x * blockDim.x + threadIdx.x;
@@ -276,15 +280,16 @@ __global__ void k_gs(MGLevel<T> L, int colour, const int* __restrict__ gate, int
   if (j >= g.n[1] || k >= g.n[2]) return;
   const int i = 2 * i2 + ((colour + j + k) & 1);
   if (i >= g.n[0]) return;
-  gs_point(L, i, j, k);
+  gs_point(L, i, j, k, xin ? xin : L.x);
 }
 
 template <typename T>
-void launch_gs(const MGLevel<T>& L, int colour, cudaStream_t s, const int* gate, int gate_min) {
+void launch_gs(const MGLevel<T>& L, int colour, cudaStream_t s, const int* gate, int gate_min,
+               const T* xin) {
   const int hx = (L.geo.n[0] + 1) / 2;
   dim3 bs(32, 4, 2);
   dim3 gs((hx + 31) / 32, (L.geo.n[1] + 3) / 4, (L.geo.n[2] + 1) / 2);
-  k_gs<T><<<gs, bs, 0, s>>>(L, colour, gate, gate_min);
+  k_gs<T><<<gs, bs, 0, s>>>(L, colour, gate, gate_min, xin);
 }
 
 // coarse b = mean over children of (b - L x) on the fine level; coarse x = 0.
@@ -435,9 +440,9 @@ __global__ void k_gs_zero(MGLevel<T> L, int colour) {
 // The last sweep of the mixed form's inner correction with p += e folded in:
 // the thread adds the new value of its cell and the final value of the other
 // colour's cell beside it (not written in this sweep) to the double p.  The
-// correction e itself is not stored again; the next refinement starts it
-// from 0.
-__global__ void k_gs_addp(MGLevel<float> L, int colour, double* __restrict__ p) {
+// correction e itself is stored only when the residual is updated with it
+// (k_residual_update); the next refinement starts it from 0.
+__global__ void k_gs_addp(MGLevel<float> L, int colour, double* __restrict__ p, int store) {
   const Geo& g = L.geo;
   const int i2 = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -456,6 +461,7 @@ __global__ void k_gs_addp(MGLevel<float> L, int colour, double* __restrict__ p) 
     xhi[d] = L.x[nb.hi[d]];
   }
   const float e = gs_value(L, row + i, nb, xlo, xhi);
+  if (store) L.x[row + i] = e;
   p[row + i] = p[row + i] + (double)e;
 }
 
@@ -467,11 +473,11 @@ void launch_gs_zero(const MGLevel<T>& L, int colour, cudaStream_t s) {
   k_gs_zero<T><<<gs, bs, 0, s>>>(L, colour);
 }
 
-void launch_gs_addp(const MGLevel<float>& L, int colour, double* p, cudaStream_t s) {
+void launch_gs_addp(const MGLevel<float>& L, int colour, double* p, bool store, cudaStream_t s) {
   const int hx = (L.geo.n[0] + 1) / 2;
   dim3 bs(32, 4, 2);
   dim3 gs((hx + 31) / 32, (L.geo.n[1] + 3) / 4, (L.geo.n[2] + 1) / 2);
-  k_gs_addp<<<gs, bs, 0, s>>>(L, colour, p);
+  k_gs_addp<<<gs, bs, 0, s>>>(L, colour, p, store ? 1 : 0);
 }
 
 template <typename T>
@@ -627,7 +633,9 @@ __device__ __forceinline__ double beta_to_double(float f) {
 __global__ void k_residual64(Geo g, const double* __restrict__ p, const double* __restrict__ b,
                              const float* __restrict__ b0, const float* __restrict__ b1,
                              const float* __restrict__ b2, float* __restrict__ r32,
-                             double* __restrict__ partial, float* __restrict__ e32, W3 w32) {
+                             double* __restrict__ partial, float* __restrict__ e32, W3 w32,
+                             double* __restrict__ rd, const int* __restrict__ gate) {
+  if (gate && !*gate) return;
   __shared__ double sh[33];
   const float* be[3] = {b0, b1, b2};
   const int st[3] = {1, g.n[0], g.n[0] * g.n[1]};
@@ -657,6 +665,7 @@ __global__ void k_residual64(Geo g, const double* __restrict__ p, const double* 
     const double r = fma(-wu, lsum, b[c]);
     const float rf = (float)r;
     r32[c] = rf;
+    if (rd) rd[c] = r;
     if (e32) {
       const float z[3] = {0.f, 0.f, 0.f};
       e32[c] = ((i + j + k) & 1) == 0 ? gs_formula(g, w32.w, w32.w[0] != 0.f ? w32.w[0] : (w32.w[1] != 0.f ? w32.w[1] : w32.w[2]), rf,
@@ -671,12 +680,133 @@ __global__ void k_residual64(Geo g, const double* __restrict__ p, const double* 
 
 void launch_residual64(const Geo& g, const double* p, const double* b, float* const* beta,
                        float* r32, double* partial, double* out, cudaStream_t s, float* e32,
-                       const float* w32) {
+                       const float* w32, double* rd, const int* gate) {
   W3 w = {{0.f, 0.f, 0.f}};
   if (w32)
     for (int d = 0; d < 3; ++d) w.w[d] = w32[d];
-  k_residual64<<<kRedBlocks, 256, 0, s>>>(g, p, b, beta[0], beta[1], beta[2], r32, partial, e32, w);
-  launch_sum_partials(partial, kRedBlocks, out, s);
+  k_residual64<<<kRedBlocks, 256, 0, s>>>(g, p, b, beta[0], beta[1], beta[2], r32, partial, e32, w,
+                                          rd, gate);
+  launch_sum_partials(partial, kRedBlocks, out, s, gate);
+}
+
+// ---------------------------------------------------------------------------
+// The residual of the next refinement from the one before: after p += e,
+// r -= L e.  The correction e and beta are float, so the differences of e
+// and their products with beta are formed exactly as pairs of floats (Knuth's
+// two-sum, the fused product error) and summed as such: 48 bits in float
+// arithmetic, which the GPU does 64 times as fast as double.  Formed from p
+// (k_residual64, 14 FP64 operations a cell) the pass is bound by the FP64
+// pipe: 0.56 ms at 256^3 against 0.29 ms here.  Its error, 2^-48 beta |de| of a
+// face, is that of rounding p itself (2^-53 beta |p|) once e varies over 32
+// cells and more, and it does not grow: the solve forms the residual from p
+// again before it stops, and goes on from that one if it is above the
+// tolerance.  The rule (fvm_api.cu) takes this pass from 2^19 cells; below,
+// the two launches more of a refinement cost what it saves.
+struct FloatPair {
+  float h, l;
+};
+
+__device__ __forceinline__ FloatPair face_product(float beta, float a, float b) {
+  const float s = __fsub_rn(a, b);
+  const float t = __fsub_rn(s, a);
+  const float err = __fsub_rn(__fsub_rn(a, __fsub_rn(s, t)), __fadd_rn(b, t));
+  FloatPair p;
+  p.h = __fmul_rn(beta, s);
+  p.l = __fmaf_rn(beta, err, __fmaf_rn(beta, s, -p.h));
+  return p;
+}
+
+__device__ __forceinline__ void pair_add(FloatPair& s, float h, float l) {
+  const float t = __fadd_rn(s.h, h);
+  const float z = __fsub_rn(t, s.h);
+  const float e = __fadd_rn(__fsub_rn(s.h, __fsub_rn(t, z)), __fsub_rn(h, z));
+  s.h = t;
+  s.l = __fadd_rn(s.l, __fadd_rn(e, l));
+}
+
+// float -> double with integer operations (as beta_to_double; an infinity or a
+// NaN takes the conversion instruction)
+__device__ __forceinline__ double pair_to_double(float f) {
+  if ((__float_as_uint(f) & 0x7fffffffu) >= 0x7f800000u) return (double)f;
+  return beta_to_double(f);
+}
+
+// A thread owns a column of cells and walks planes k0 .. k1-1 upward; the
+// product of a z-face serves the cells on both of its sides.
+__global__ void __launch_bounds__(256)
+    k_residual_update(MGLevel<float> L, double* __restrict__ rd, float* __restrict__ y,
+                      double* __restrict__ partial, int tx, int ty, int chunks, int kz) {
+  __shared__ double sh[33];
+  const Geo& g = L.geo;
+  const int nx = g.n[0], ny = g.n[1], nz = g.n[2], nxy = nx * ny;
+  const float* __restrict__ e = L.x;
+  const float *__restrict__ b0 = L.beta[0], *__restrict__ b1 = L.beta[1],
+              *__restrict__ b2 = L.beta[2];
+  const double w = (double)g.w[nx > 1 ? 0 : (ny > 1 ? 1 : 2)];
+  double acc = 0.0;
+  for (int t = blockIdx.x; t < tx * ty * chunks; t += gridDim.x) {
+    const int q = t / tx, i = (t - q * tx) * 32 + (threadIdx.x & 31);
+    const int ch = q / ty, j = (q - ch * ty) * 8 + (threadIdx.x >> 5);
+    if (i >= nx || j >= ny) continue;
+    const int k0 = ch * kz, k1 = min(k0 + kz, nz);
+    const int col = j * nx + i;
+    const int xm = i == 0 ? nx - 1 : -1, xp = i == nx - 1 ? 1 - nx : 1;
+    const int ym = j == 0 ? (ny - 1) * nx : -nx, yp = j == ny - 1 ? (1 - ny) * nx : nx;
+    const bool wx = i == nx - 1 && g.bc[0] == WALL, wy = j == ny - 1 && g.bc[1] == WALL;
+    int c = k0 * nxy + col;
+    float ec = e[c];
+    float bz = b2[c];
+    FloatPair zl = face_product(bz, ec, e[k0 == 0 ? (nz - 1) * nxy + col : c - nxy]);
+    for (int k = k0; k < k1; ++k) {
+      const int cn = k == nz - 1 ? col : c + nxy;
+      const float en = e[cn], bzl = bz;
+      bz = (k == nz - 1 && g.bc[2] == WALL) ? 0.f : b2[cn];
+      const float xl = b0[c], xh = wx ? 0.f : b0[c + xp];
+      const float yl = b1[c], yh = wy ? 0.f : b1[c + yp];
+      FloatPair s = face_product(xl, ec, e[c + xm]);
+      FloatPair f = face_product(xh, ec, e[c + xp]);
+      pair_add(s, f.h, f.l);
+      f = face_product(yl, ec, e[c + ym]);
+      pair_add(s, f.h, f.l);
+      f = face_product(yh, ec, e[c + yp]);
+      pair_add(s, f.h, f.l);
+      pair_add(s, zl.h, zl.l);
+      f = face_product(bz, ec, en);
+      pair_add(s, f.h, f.l);
+      zl.h = -f.h;
+      zl.l = -f.l;
+      const double r = fma(-w, pair_to_double(s.l), fma(-w, pair_to_double(s.h), rd[c]));
+      rd[c] = r;
+      const float rf = (float)r;
+      L.b[c] = rf;
+      if (y && ((i + j + k) & 1) == 0) {
+        // the next inner solve's first sweep: colour 0 from 0
+        const float lo[3] = {xl, yl, bzl}, hi[3] = {xh, yh, bz}, z[3] = {0.f, 0.f, 0.f};
+        y[c] = gs_formula(g, L.w, L.wu, rf, lo, hi, z, z);
+      }
+      acc = fma(r, r, acc);
+      ec = en;
+      c = cn;
+    }
+  }
+  const double s = block_sum_all(acc, sh);
+  if (threadIdx.x == 0) partial[blockIdx.x] = s;
+}
+
+void launch_residual_update(const MGLevel<float>& L, double* rd, float* y, double* partial,
+                            double* out, cudaStream_t s) {
+  // about kRedBlocks blocks, each a 32 x 8 tile of columns and a run of at
+  // least 16 planes
+  const int tx = (L.geo.n[0] + 31) / 32, ty = (L.geo.n[1] + 7) / 8, nz = L.geo.n[2];
+  const long long tiles = (long long)tx * ty;
+  int chunks = (int)(tiles >= kRedBlocks ? 1 : kRedBlocks / tiles);
+  int kz = (nz + chunks - 1) / chunks;
+  if (kz < 16) kz = nz < 16 ? nz : 16;
+  chunks = (nz + kz - 1) / kz;
+  const long long work = tiles * chunks;
+  const int blocks = (int)(work < kRedBlocks ? work : kRedBlocks);
+  k_residual_update<<<blocks, 256, 0, s>>>(L, rd, y, partial, tx, ty, chunks, kz);
+  launch_sum_partials(partial, blocks, out, s);
 }
 
 __global__ void k_add_correction(long long n, double* __restrict__ p, const float* __restrict__ e) {
@@ -694,6 +824,7 @@ __global__ void k_ctl_reset(SolveCtl* ctl) {
   ctl->iters = 0;
   ctl->status = 0;
   ctl->zero = 0;
+  ctl->verify = 0;
   ctl->rel = 0.0;
 }
 
@@ -737,6 +868,19 @@ void launch_ctl_step(cudaGraphConditionalHandle h, SolveCtl* ctl, const double* 
   k_ctl_step<<<1, 1, 0, s>>>(h, ctl, bn2, r2, rtol, maxit, fixed, runs_total);
 }
 
+__global__ void k_ctl_check(SolveCtl* ctl, const double* bn2p, const double* r2p, double rtol,
+                            int maxit, int fixed) {
+  const double rel = sqrt(*r2p) / sqrt(*bn2p);
+  const bool go = isfinite(rel) && (fixed > 0 ? ctl->iters < fixed
+                                              : (rel > rtol && ctl->iters < maxit));
+  ctl->verify = go ? 0 : 1;
+}
+
+void launch_ctl_check(SolveCtl* ctl, const double* bn2, const double* r2, double rtol, int maxit,
+                      int fixed, cudaStream_t s) {
+  k_ctl_check<<<1, 1, 0, s>>>(ctl, bn2, r2, rtol, maxit, fixed);
+}
+
 __global__ void k_zero_if_rhs_zero(const SolveCtl* __restrict__ ctl, double* __restrict__ p,
                                    long long n) {
   if (!ctl->zero) return;
@@ -762,7 +906,7 @@ void launch_ctl_store(const SolveCtl* ctl, SolveCtl* rec, int* sticky, cudaStrea
   template void launch_sum_field<T>(const T*, long long, bool, double*, double*,             \
                                     cudaStream_t);                                           \
   template void launch_zero<T>(T*, long long, cudaStream_t);                                 \
-  template void launch_gs<T>(const MGLevel<T>&, int, cudaStream_t, const int*, int);        \
+  template void launch_gs<T>(const MGLevel<T>&, int, cudaStream_t, const int*, int, const T*); \
   template void launch_residual_restrict<T>(const MGLevel<T>&, const MGLevel<T>&, cudaStream_t, bool, \
                                             bool);                                           \
   template void launch_inv_diag<T>(const MGLevel<T>&, cudaStream_t);                         \
