@@ -80,8 +80,8 @@ Geo make_geo(const fvm_params& p, const LevelShape& s) {
 }
 
 // the coarse tail (fvm_tail.cu) of a hierarchy: its first level, the finest
-// one below level 0 (or level 0 when there is no other) from which all
-// levels fit, -1 when not even the coarsest does; the bytes of its packed
+// one below level 0 (level 0 itself on a small double grid, or when there is no
+// other) from which all levels fit, -1 when not even the coarsest does; the bytes of its packed
 // coefficients and of the two matrices of the coarsest level's float inverse
 struct TailPlan {
   int first;
@@ -101,7 +101,9 @@ TailPlan plan_tail_of(const fvm_params& p, const LevelShape* lv, int nl, bool in
   inverse = inverse && nc > 32 && nc <= kTailInvMax && p.coarse_maxit >= nc;
   TailArgs<T> A;
   size_t smem = 0, pack = 0;
-  for (int l = nl > 1 ? 1 : 0; l < nl; ++l)
+  // a small double grid is solved in the tail as a whole
+  const bool whole = nl == 1 || (sizeof(T) == 8 && Ls[0].geo.N <= kTailTopCells);
+  for (int l = whole ? 0 : 1; l < nl; ++l)
     if (tail_layout<T>(Ls + l, nl - l, inverse, A, &smem, &pack))
       return {l, inverse, pack, (size_t)A.np * A.np * 2 * sizeof(float) + (inverse ? 256 : 0)};
   return {-1, false, 0, 0};
@@ -536,6 +538,13 @@ size_t tail_args(fvm_ctx* c, const MGLevel<T>* Ls, double rtol, TailArgs<T>& A) 
   A.maxit = c->prm.coarse_maxit;
   A.pre = coarse_pre(c);
   A.post = coarse_post(c);
+  A.pre0 = c->tail.first == 0 ? c->prm.mg_pre : A.pre;
+  A.post0 = c->tail.first == 0 ? c->prm.mg_post : A.post;
+  A.ctl = nullptr;
+  A.bn2 = nullptr;
+  A.tol = c->prm.mg_rtol;
+  A.maxcycles = c->prm.mg_max_cycles;
+  A.fixed = c->prm.mg_fixed_cycles;
   // at most 32 coarsest cells are solved by a packed inverse, unless the caller
   // cuts the conjugate gradients short
   const long long nc = Ls[c->nlev - 1].geo.N;
@@ -660,6 +669,30 @@ void vcycle(fvm_ctx* c, MGLevel<T>* Ls, int l, double coarse_rtol, int start = k
     TIMED(c, FVM_K_ADD_CORRECTION, 1, launch_add_correction(Ls[0].geo.N, addp, (const float*)Ls[0].x, s));
 }
 
+// status of a device-side record, as the host loop would have returned it
+fvm_status record_status(fvm_ctx* c, const SolveCtl& r) {
+  if (r.status == FVM_EUNSTABLE)
+    return set_err(c, FVM_EUNSTABLE, "non-finite projection right-hand side or residual");
+  if (r.status == FVM_ENOCONV)
+    return set_err(c, FVM_ENOCONV, "pressure solve reached mg_max_cycles above mg_rtol");
+  return FVM_OK;
+}
+
+// a double grid small enough that the tail holds every level is solved by one
+// launch, stopping test included
+bool solve_is_tail(const fvm_ctx* c) { return !c->mixed && c->nlev > 1 && c->tail.first == 0; }
+
+// ||b||^2 and the cycles of such a solve (the controller then holds the result)
+void tail_solve(fvm_ctx* c, MGLevel<double>* Ls) {
+  TIMED(c, FVM_K_MISC, 2,
+        launch_sum_field<double>(Ls[0].b, c->g.N, true, c->partial, c->scal + 0, c->stream));
+  TailArgs<double> A;
+  const size_t smem = tail_args<double>(c, Ls, c->prm.coarse_rtol, A);
+  A.ctl = c->ctl;
+  A.bn2 = c->scal + 0;
+  TIMED(c, FVM_K_COARSE_TAIL, 1, launch_tail<double>(A, smem, c->stream));
+}
+
 // F64: L p = b (b mean-free, double), beta0 already computed
 fvm_status solve_f64(fvm_ctx* c, double* p, double* b, int* cycles_out, double* rel_out,
                      bool want_rel) {
@@ -669,6 +702,20 @@ fvm_status solve_f64(fvm_ctx* c, double* p, double* b, int* cycles_out, double* 
   hierarchy<double>(c, p, b, be, Ls);
   coarsen_betas<double>(c, Ls);
   const long long N = c->g.N;
+  if (solve_is_tail(c)) {
+    tail_solve(c, Ls);
+    TIMED(c, FVM_K_MISC, 1, launch_zero_if_rhs_zero(c->ctl, p, N, s));
+    TIMED(c, FVM_K_MISC, 2, launch_sum_field<double>(p, N, false, c->partial, c->scal + 2, s));
+    TIMED(c, FVM_K_MISC, 1, launch_sub_mean(p, N, c->scal + 2, s));
+    SolveCtl r;
+    cudaError_t e = cudaMemcpyAsync(&r, c->ctl, sizeof(r), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return set_err(c, FVM_ECUDA, cudaGetErrorString(e));
+    *cycles_out = r.iters;
+    *rel_out = r.rel;
+    fvm_status st = cuda_check(c, "f64 pressure solve");
+    return st ? st : record_status(c, r);
+  }
   double bn2;
   TIMED(c, FVM_K_MISC, 2, launch_sum_field<double>(b, N, true, c->partial, c->scal + 0, s));
   fvm_status st = read_scalar(c, c->scal + 0, &bn2);
@@ -832,6 +879,10 @@ void graph_prologue(fvm_ctx* c, double* p, cudaGraphConditionalHandle h) {
     double* be[3] = {(double*)c->beta0[0], (double*)c->beta0[1], (double*)c->beta0[2]};
     hierarchy<double>(c, p, c->b, be, Ls);
     coarsen_betas<double>(c, Ls);
+    if (solve_is_tail(c)) {
+      tail_solve(c, Ls);
+      return;
+    }
     TIMED(c, FVM_K_MISC, 1, launch_ctl_reset(c->ctl, s));
     TIMED(c, FVM_K_MISC, 2, launch_sum_field<double>(c->b, N, true, c->partial, c->scal + 0, s));
     TIMED(c, FVM_K_RESNORM, 2, launch_residual_norm2<double>(Ls[0], c->partial, c->scal + 1, s));
@@ -895,11 +946,14 @@ cudaGraphExec_t solve_graph(fvm_ctx* c, double* p, long* nk_fixed) {
   size_t nleaves = 0;
   const long n0 = c->nlaunch;
   long n_body = 0;
+  const bool whole = solve_is_tail(c);   // one launch: nothing to loop over
   bool ok = cudaGraphCreate(&g, 0) == cudaSuccess &&
-            cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault) == cudaSuccess &&
+            (whole || cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault) ==
+                          cudaSuccess) &&
             cudaStreamBeginCaptureToGraph(s, g, nullptr, nullptr, 0, mode) == cudaSuccess;
   if (ok) {
     graph_prologue(c, p, h);
+    if (whole) graph_epilogue(c, p);
     cudaStreamCaptureStatus cs;
     const cudaGraphNode_t* deps = nullptr;
     size_t nd = 0;
@@ -910,7 +964,7 @@ cudaGraphExec_t solve_graph(fvm_ctx* c, double* p, long* nk_fixed) {
     nleaves = nd;
     if (cudaStreamEndCapture(s, &tmp) != cudaSuccess) ok = false;
   }
-  if (ok) {
+  if (ok && !whole) {
     // zeroed storage: the parameter union has no default constructor
     alignas(cudaGraphNodeParams) unsigned char prm_raw[sizeof(cudaGraphNodeParams)];
     memset(prm_raw, 0, sizeof(prm_raw));
@@ -931,7 +985,7 @@ cudaGraphExec_t solve_graph(fvm_ctx* c, double* p, long* nk_fixed) {
       }
     }
   }
-  if (ok) {
+  if (ok && !whole) {
     ok = cudaStreamBeginCaptureToGraph(s, g, &cond, nullptr, 1, mode) == cudaSuccess;
     if (ok) {
       graph_epilogue(c, p);
@@ -985,15 +1039,6 @@ fvm_status solve(fvm_ctx* c, const void* alpha, double* p, int slot, int* cyc, d
   }
   if (c->mixed) return solve_mixed(c, (const float*)alpha, p, c->b, cyc, rel, want_rel);
   return solve_f64(c, p, c->b, cyc, rel, want_rel);
-}
-
-// status of a device-side record, as the host loop would have returned it
-fvm_status record_status(fvm_ctx* c, const SolveCtl& r) {
-  if (r.status == FVM_EUNSTABLE)
-    return set_err(c, FVM_EUNSTABLE, "non-finite projection right-hand side or residual");
-  if (r.status == FVM_ENOCONV)
-    return set_err(c, FVM_ENOCONV, "pressure solve reached mg_max_cycles above mg_rtol");
-  return FVM_OK;
 }
 
 template <typename R>
@@ -1756,6 +1801,7 @@ size_t plan_noalloc(const fvm_params& p, fvm_ctx* c, char* base) {
   if (tail.pack + kAlign > room) tail.pack = 0;
   const size_t o_pack = pl.take(tail.pack);
   const size_t o_inv = pl.take(tail.inv);
+  const size_t o_ctl = tail.first == 0 ? pl.take(sizeof(SolveCtl)) : 0;   // (small grids only)
   // likewise the reciprocal diagonals, finest level first
   const int above = tail.first < 0 ? nl - 1 : tail.first;
   size_t o_linv[kMaxLevels];
@@ -1766,6 +1812,7 @@ size_t plan_noalloc(const fvm_params& p, fvm_ctx* c, char* base) {
   if (c) {
     for (int l = 0; l < above; ++l) c->linv[l] = o_linv[l] ? base + o_linv[l] : nullptr;
     c->tail = tail;
+    c->ctl = tail.first == 0 ? (SolveCtl*)(base + o_ctl) : nullptr;
     c->pack = tail.pack ? base + o_pack : nullptr;
     c->inv = tail.inv ? base + o_inv : nullptr;
     c->b = (double*)(base + o_b);

@@ -168,12 +168,22 @@ void launch_gs_zero(const MGLevel<T>& L, int colour, cudaStream_t s);
 void launch_gs_addp(const MGLevel<float>& L, int colour, double* p, bool store, cudaStream_t s);
 template <typename T>
 void launch_beta_coarsen(const MGLevel<T>& F, const MGLevel<T>& C, cudaStream_t s);
+// state of a pressure solve's stopping test on the device
+struct SolveCtl {
+  int iters;      // cycles (F64) or refinements (MIXED) done
+  int status;     // 0, FVM_ENOCONV or FVM_EUNSTABLE
+  int zero;       // 1: ||b|| = 0, the solution is set to 0
+  int verify;     // 1: the updated residual would stop the solve; form it from p
+  double rel;     // last relative residual
+};
+
 // The coarse tail of a V-cycle (fvm_tail.cu): the levels from the first one
 // that fits down to the coarsest, in one launch of one cluster of kTailCTAs
 // CTAs.
 constexpr int kTailCTAs = 16;
 constexpr int kTailLevels = 16;
 constexpr int kTailMaxCells = 32768;        // of the tail's first level
+constexpr int kTailTopCells = 16384;        // of a double grid solved in the tail as a whole
 constexpr int kTailSmem = 220 * 1024;       // shared memory of a CTA
 constexpr int kTailCells32 = 512, kTailCells64 = 256;   // cells a CTA should have (float, double)
 constexpr int kTailCgCells = 64, kTailCgSingle = 400;    // the same for the coarsest level's CG
@@ -193,6 +203,9 @@ struct TailLevel {
   T* x;
   size_t opack;                // byte offset of the level's blocks in the packed coefficients
 };
+// With ctl the launch is a whole solve of L[0] (the finest level, x its start):
+// cycles until ||b - L x|| <= tol ||b||, b's squared norm in *bn2; otherwise
+// it is one cycle from x = 0.
 template <typename T>
 struct TailArgs {
   int nl;                      // levels, the last one the coarsest
@@ -201,9 +214,14 @@ struct TailArgs {
   int np;                      // order of the float inverse (a multiple of 64; 0: none)
   const float* G;              // the inverse of the coarsest operator / *gscale (null: CG)
   const double* gscale;
+  SolveCtl* ctl;
+  const double* bn2;
+  double tol;
+  int maxcycles, fixed;
   const void* pack;            // coefficients of launch_tail_pack (null: formed from beta)
   double rtol;
   int maxit, pre, post;
+  int pre0, post0;             // sweeps of the first level
   bool direct;                 // the coarsest level by its packed inverse instead of CG
 };
 // lay out levels Ls[0 .. nl-1]; false when they do not fit.  smem: bytes per
@@ -252,13 +270,6 @@ void launch_add_correction(long long n, double* p, const float* e, cudaStream_t 
 // a conditional WHILE node: after every cycle (refinement) the controller
 // kernel forms ||b - L p|| / ||b|| from the two reduction slots and sets the
 // node's condition, so the host never waits for a residual.
-struct SolveCtl {
-  int iters;      // cycles (F64) or refinements (MIXED) done
-  int status;     // 0, FVM_ENOCONV or FVM_EUNSTABLE
-  int zero;       // 1: ||b|| = 0, the solution is set to 0
-  int verify;     // 1: the updated residual would stop the solve; form it from p
-  double rel;     // last relative residual
-};
 void launch_ctl_reset(SolveCtl* ctl, cudaStream_t s);
 // bn2 = ||b||^2 and r2 = ||b - L p||^2 (device); fixed > 0: exactly `fixed`
 // cycles; runs_total counts the cycles of every solve (launch bookkeeping)

@@ -654,6 +654,78 @@ __device__ void coarsest_direct(const View<T>& V) {
   if (lane < N) V.x()[c] = (T)(s0 + s1);
 }
 
+// The whole solve of a grid whose finest level is in the tail: cycles until
+// ||b - L x|| <= rtol ||b|| (or the fixed count, or the cap), with the stopping
+// rule of k_ctl_step.  Warp 0 of every CTA works it out from the same sums.
+template <typename T, typename F>
+__device__ __forceinline__ void solve_loop(const View<T>& V, const TailArgs<T>& A, Reduce& red,
+                                           F cycle) {
+  const TailLevel<T>& L = V.L;
+  const int hx = L.hx, nx = L.n[0], cap = L.cap;
+  const float ip = 1.0f / (float)L.pitch;
+  int iters = 0, status = 0, zero = 0;
+  double rel = 0.0;
+  const double bn2 = *A.bn2;
+  for (;;) {
+    const T* x = V.x();
+    const T* b = V.b();
+    const T* a = V.template a<T>();
+    double acc = 0.0;
+    for (int t = threadIdx.x; t < V.nrows * L.pitch; t += kTailThreads) {
+      const int q = quot(t, ip), p = t - q * L.pitch;
+      const int i = p < hx ? 2 * p : 2 * (p - hx) + 1;
+      if (i >= nx) continue;
+      const int4 ra = V.tab()[2 * q];
+      const int row = q * L.pitch;
+      T ym, yp, zm, zp;
+      const unsigned o = p * (unsigned)sizeof(T);
+      ld_cl(ra.x + o, ym);
+      ld_cl(ra.y + o, yp);
+      ld_cl(ra.z + o, zm);
+      ld_cl(ra.w + o, zp);
+      const T xc = x[t];
+      const T xm = x[row + row_pos(i == 0 ? nx - 1 : i - 1, hx)];
+      const T xp = x[row + row_pos(i == nx - 1 ? 0 : i + 1, hx)];
+      const T ox = a[t] * (xc - xm) + a[cap + t] * (xc - xp);
+      const T oy = a[2 * cap + t] * (xc - ym) + a[3 * cap + t] * (xc - yp);
+      const T oz = L.n[2] > 1 ? a[4 * cap + t] * (xc - zm) + a[5 * cap + t] * (xc - zp) : T(0);
+      const double r = (double)(b[t] - ((ox + oy) + oz));
+      acc = fma(r, r, acc);
+    }
+    red.nact = L.nact;
+    red.used = min(V.nrows * L.pitch, kTailThreads);
+    const double go = red.run(acc, [&](double r2) {
+      if (!isfinite(bn2)) {
+        status = FVM_EUNSTABLE;
+        return 0.0;
+      }
+      if (bn2 == 0.0) {
+        zero = 1;
+        return 0.0;
+      }
+      rel = sqrt(r2) / sqrt(bn2);
+      if (!isfinite(rel)) {
+        status = FVM_EUNSTABLE;
+        return 0.0;
+      }
+      if (A.fixed > 0) return iters < A.fixed ? 1.0 : 0.0;
+      if (rel <= A.tol) return 0.0;
+      if (iters < A.maxcycles) return 1.0;
+      status = FVM_ENOCONV;
+      return 0.0;
+    });
+    if (go == 0.0) break;
+    cycle(iters > 0 && A.pre0 > 0 && A.post0 > 0);
+    ++iters;
+  }
+  if (V.rank == 0 && threadIdx.x == 0) {
+    A.ctl->iters = iters;
+    A.ctl->status = status;
+    A.ctl->zero = zero;
+    A.ctl->rel = rel;
+  }
+}
+
 // row tables: addresses of the rows beside each own row (the array a sweep or
 // the conjugate gradients read there), the parent row, the row's parity
 template <typename T>
@@ -710,13 +782,18 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
   red.slots = red.vals + 2 * kTailThreads;
   red.out = red.slots + 4 * kTailCTAs;
   red.base_slots = base + A.ored + 2 * kTailThreads * 8;
-  red.nact = A.L[last].nact;
+  red.nact = red.used = 0;
   red.rank = rank;
   red.phase = 0;
-  red.used = min(View<T>(A.L[last], sm, rank).nrows * A.L[last].pitch, kTailThreads);
   __syncthreads();
+  int single = 0;   // first level that CTA 0 holds alone
+  while (single <= last && A.L[single].nact > 1) ++single;
+  auto sync = [&](int l) {
+    if (l < single) cluster_sync();
+    else __syncthreads();
+  };
   {
-    // the top level's right-hand side; x starts at 0
+    // the top level's right-hand side; x starts at 0, or from the caller's
     const View<T> V(A.L[0], sm, rank);
     const TailLevel<T>& L = V.L;
     const float ip = 1.0f / (float)L.pitch;
@@ -724,46 +801,55 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
       const int q = quot(t, ip), p = t - q * L.pitch;
       const int i = p < L.hx ? 2 * p : 2 * (p - L.hx) + 1;
       if (i >= L.n[0]) continue;
-      const T b = __ldg(L.b + (rank * L.rpc + q) * L.n[0] + i);
+      const int c = (rank * L.rpc + q) * L.n[0] + i;
+      const T b = __ldg(L.b + c);
       V.b()[t] = b;
-      if (last > 0) V.x()[t] = first_x(V, t, i, V.tab()[2 * q + 1].y, b, A.pre > 0);
+      if (A.ctl) V.x()[t] = L.x[c];
+      else if (last > 0) V.x()[t] = first_x(V, t, i, V.tab()[2 * q + 1].y, b, A.pre > 0);
     }
   }
   cluster_sync();
-  int single = 0;   // first level that CTA 0 holds alone
-  while (single <= last && A.L[single].nact > 1) ++single;
-  auto sync = [&](int l) {
-    if (l < single) cluster_sync();
-    else __syncthreads();
-  };
   T* scr = reinterpret_cast<T*>(sm + A.oscr);
-  for (int l = 0; l < last; ++l) {
-    if (l >= single && rank) break;
-    const View<T> V(A.L[l], sm, rank);
-    for (int h = 1; h < 2 * A.pre; ++h) {   // the first half-sweep came with b
-      sweep(V, h & 1);
+  // one V-cycle; swept: the top level's first half-sweep is taken (it came with
+  // b, or would repeat the previous cycle's last one)
+  auto cycle = [&](bool swept) {
+    for (int l = 0; l < last; ++l) {
+      if (l >= single && rank) break;
+      const View<T> V(A.L[l], sm, rank);
+      const int pre = l == 0 ? A.pre0 : A.pre;
+      for (int h = l > 0 || swept ? 1 : 0; h < 2 * pre; ++h) {
+        sweep(V, h & 1);
+        sync(l);
+      }
+      residual(V, scr, pre > 0 && sizeof(T) == sizeof(double));
+      sync(l);
+      restrict_rows(V, View<T>(A.L[l + 1], sm, rank), base, A.oscr, l + 1 == last, A.pre > 0);
       sync(l);
     }
-    residual(V, scr, A.pre > 0 && sizeof(T) == sizeof(double));
-    sync(l);
-    restrict_rows(V, View<T>(A.L[l + 1], sm, rank), base, A.oscr, l + 1 == last, A.pre > 0);
-    sync(l);
-  }
-  if (last < single || rank == 0) {
-    const View<T> V(A.L[last], sm, rank);
-    if (A.direct) coarsest_direct(V);
-    else if (!A.G || !coarsest_refine(V, A, red)) coarsest_cg(V, A, red);
-  }
-  for (int l = last - 1; l >= 0; --l) {
-    if (l >= single && rank) continue;
-    const View<T> V(A.L[l], sm, rank);
-    sync(l);
-    prolong_rows(V, A.L[l + 1]);
-    sync(l);
-    for (int h = 0; h < 2 * A.post; ++h) {
-      sweep(V, 1 - (h & 1));
-      sync(l);
+    if (last < single || rank == 0) {
+      const View<T> V(A.L[last], sm, rank);
+      red.nact = V.L.nact;
+      red.used = min(V.nrows * V.L.pitch, kTailThreads);
+      if (A.direct) coarsest_direct(V);
+      else if (!A.G || !coarsest_refine(V, A, red)) coarsest_cg(V, A, red);
     }
+    for (int l = last - 1; l >= 0; --l) {
+      if (l >= single && rank) continue;
+      const View<T> V(A.L[l], sm, rank);
+      sync(l);
+      prolong_rows(V, A.L[l + 1]);
+      sync(l);
+      const int post = l == 0 ? A.post0 : A.post;
+      for (int h = 0; h < 2 * post; ++h) {
+        sweep(V, 1 - (h & 1));
+        sync(l);
+      }
+    }
+  };
+  if (!A.ctl) {
+    cycle(A.pre0 > 0);
+  } else if (single > 0 || rank == 0) {
+    solve_loop(View<T>(A.L[0], sm, rank), A, red, cycle);
   }
   if (last == 0) __syncthreads();
   {

@@ -107,3 +107,29 @@ def test_noalloc_without_room_for_the_coefficients():
     assert got["vcycles"][0] == info["vcycles"][0]
     assert got["rel_residual"][0] <= 1e-10
     assert rel_l2(dp.cpu().numpy(), ref) <= 1e-6
+
+
+@pytest.mark.parametrize("nx", [128, 132])
+def test_largest_grid_solved_in_one_launch_and_the_next(nx):
+    """16384 double cells are solved by one launch, 16896 level by level."""
+    P = need_gpu()
+    p, alpha, rhs = _problem(nx, 128, 1, (W, W, P_), mg_fixed_cycles=3)
+    ref, _, rel = O.poisson_solve(alpha, rhs, np.zeros(p.shape), p)
+    got, info = _solve(P, p, alpha, rhs)
+    assert info["vcycles"][0] == 3
+    assert info["rel_residual"][0] == pytest.approx(rel, rel=1e-6)
+    assert rel_l2(got, ref.numpy()) <= 1e-11
+
+
+def test_one_launch_solve_of_zero_and_of_non_finite_right_hand_sides():
+    P = need_gpu()
+    p, alpha, rhs = _problem(16, 16, 8, (W, P_, W))
+    got, info = _solve(P, p, alpha, 0.0 * rhs)
+    assert info["status"] == 0 and info["vcycles"][0] == 0 and not got.any()
+    s = P.Solver(p)
+    rhs[1, 2, 3] = np.inf
+    dp = torch.zeros(p.shape, dtype=torch.float64, device="cuda")
+    info = s.fvm_poisson_solve(torch.tensor(alpha, device="cuda"), torch.tensor(rhs, device="cuda"),
+                               dp, raise_on_error=False)
+    assert info["status"] == 5
+    s.close()
