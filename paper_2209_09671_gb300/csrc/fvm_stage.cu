@@ -215,9 +215,29 @@ struct Plane {
   static __device__ __forceinline__ int at(int lx, int ly) { return (ly + H) * PX + lx + H; }
 };
 
-static inline dim3 zmarch_grid(const Geo& g, int kz) {
-  return dim3((unsigned)((g.n[0] + kZX - 1) / kZX), (unsigned)((g.n[1] + kZY - 1) / kZY),
-              (unsigned)((g.n[2] + kz - 1) / kz));
+// Planes per CTA of a z-marching kernel.  A run pays its warm-up (up to 6
+// planes) once, but short runs are what fills the GPU on a small grid: the
+// launch gets about `target` CTAs, in runs of 4 to `cap` planes.  Measured over
+// 64^3 to 256^3: float 512 CTAs and runs up to 24 (128x128x64: interface 199 us in
+// runs of 32 -> 98 in runs of 8, scalars 133 -> 95 and momentum 230 -> 185 from
+// runs of 16; 88x72x40: 254 -> 64, 174 -> 90, 166 -> 71; 256^3: scalars and momentum 1036 ->
+// 993, 1827 -> 1734 in runs of 24; the interface, whose warm-up is longest, up to
+// 32); double 1024 CTAs, 256 for the interface
+// (96x96x48: 573 -> 272, 515 -> 377, 956 -> 672).  Tiles of two rows of columns
+// instead of eight were slower everywhere but on 64 x 64 x 1.
+struct ZRuns {
+  int kz;
+  dim3 grid;
+};
+static ZRuns zmarch_runs(const Geo& g, int target, int cap) {
+  ZRuns r;
+  const long long tx = (g.n[0] + kZX - 1) / kZX, ty = (g.n[1] + kZY - 1) / kZY;
+  long long kz = (tx * ty * g.n[2] + target / 2) / target;
+  kz = kz < 4 ? 4 : (kz > cap ? cap : kz);
+  const int runs = (int)((g.n[2] + kz - 1) / kz);
+  r.kz = (g.n[2] + runs - 1) / runs;   // of even length
+  r.grid = dim3((unsigned)tx, (unsigned)ty, (unsigned)((g.n[2] + r.kz - 1) / r.kz));
+  return r;
 }
 
 // the CTA's columns and their x-y reach H stay inside the domain
@@ -330,8 +350,6 @@ __device__ __forceinline__ void plane_async(R* __restrict__ s, const R* __restri
 // 2K+1 taps ([1,4,6,4,1]/16 for K = 2), and the passes along different axes
 // commute, so the smoothing is applied as one 5-tap pass per axis: x and y
 // on each staged plane, z across a ring of x-y-smoothed planes.
-constexpr int kZKI = 32;   // planes per CTA
-
 template <typename R>
 struct IfaceZ {
   R ar[6][Plane<3>::N];      // alpha, ring of planes (m mod 6)
@@ -429,7 +447,7 @@ template <typename R>
 __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 4 : 2)
     k_interface(Geo g, PhysR<R> ph, TBC tb, int passes, const R* __restrict__ alpha,
                 const R* __restrict__ T, const R* __restrict__ conc, R* __restrict__ kappa,
-                R* __restrict__ M0, R* __restrict__ M1, R* __restrict__ M2) {
+                R* __restrict__ M0, R* __restrict__ M1, R* __restrict__ M2, int kz) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   IfaceZ<R>& S = *reinterpret_cast<IfaceZ<R>*>(smem_raw);
   using P1 = Plane<1>;
@@ -437,8 +455,8 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 4 : 2)
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int i = blockIdx.x * kZX + tx, j = blockIdx.y * kZY + ty;
-  const int z0 = blockIdx.z * kZKI;
-  const int z1 = min(z0 + kZKI, nz);
+  const int z0 = blockIdx.z * kz;
+  const int z1 = min(z0 + kz, nz);
   const bool in = zcols_interior(g, 3);
   const bool col = i < nx && j < ny;
   const R ih = ph.ih, i2h = R(0.5) * ph.ih, epsn = ph.eps_n;
@@ -565,8 +583,9 @@ void launch_interface(const Geo& g, const Phys& ph, const TBC& tb, int passes, c
                       const R* T, const R* c, R* kappa, R* M0, R* M1, R* M2, cudaStream_t s) {
   const int smem = (int)sizeof(IfaceZ<R>);
   cudaFuncSetAttribute(k_interface<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  k_interface<R><<<zmarch_grid(g, kZKI), dim3(kZX, kZY), smem, s>>>(
-      g, make_physr<R>(ph, g), tb, passes, alpha, T, c, kappa, M0, M1, M2);
+  const ZRuns z = zmarch_runs(g, sizeof(R) == 4 ? 512 : 256, 32);
+  k_interface<R><<<z.grid, dim3(kZX, kZY), smem, s>>>(g, make_physr<R>(ph, g), tb, passes, alpha,
+                                                      T, c, kappa, M0, M1, M2, z.kz);
 }
 
 // ---------------------------------------------------------------------------
@@ -608,8 +627,6 @@ __device__ __forceinline__ R fct_flux(const FctRatios<R>& f, const Geo& g, bool 
 // y-face flux is evaluated once per plane: each thread takes the low face of
 // its cell, one warp the high y-faces of the tile's last row, another the
 // high x-faces of its last column.
-constexpr int kZKS = 16;   // planes per CTA
-
 // one cell of column (i, j) at height k (any k: ghost planes go through the
 // boundary rules)
 template <int KIND, typename R>
@@ -678,14 +695,14 @@ template <typename R>
 __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 4 : 2)
     k_scalars(Geo g, PhysR<R> ph, TBC tb, Fields<R> X, Fields<R> Sn, Fields<R> Y,
               const double* __restrict__ dtp, R a, R b, R xc, R yc, R qamp, R ir2,
-              FctRatios<R> fct) {
+              FctRatios<R> fct, int kz) {
   __shared__ ScalZ<R> S;
   using P = Plane<3>;
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int i = blockIdx.x * kZX + tx, j = blockIdx.y * kZY + ty;
-  const int z0 = blockIdx.z * kZKS;
-  const int z1 = min(z0 + kZKS, nz);
+  const int z0 = blockIdx.z * kz;
+  const int z1 = min(z0 + kz, nz);
   const bool in = zcols_interior(g, 3);
   const bool col = i < nx && j < ny;
   const R dt = (R)dtp[0];
@@ -819,9 +836,10 @@ void launch_scalars(const Geo& g, const Phys& ph, const TBC& tb, Fields<R> X, Fi
   double r2 = ph.q_radius * ph.q_radius;
   double qamp = ph.q_power != 0.0 ? 2.0 * ph.q_power / (M_PI * r2) : 0.0;
   double ir2 = ph.q_power != 0.0 ? 1.0 / r2 : 0.0;
-  k_scalars<R><<<zmarch_grid(g, kZKS), dim3(kZX, kZY), 0, s>>>(
+  const ZRuns z = zmarch_runs(g, sizeof(R) == 4 ? 512 : 1024, sizeof(R) == 4 ? 24 : 16);
+  k_scalars<R><<<z.grid, dim3(kZX, kZY), 0, s>>>(
       g, make_physr<R>(ph, g), tb, X, Sn, Y, dt, (R)a, (R)b, (R)xc, (R)ph.q_y0, (R)qamp, (R)ir2,
-      FctRatios<R>{fct_p, fct_m});
+      FctRatios<R>{fct_p, fct_m}, z.kz);
 }
 
 // limiter ratios of the bounded alpha transport for one stage: per cell the
@@ -992,8 +1010,6 @@ void launch_concentration(const Geo& g, const Phys& ph, Fields<R> X, Fields<R> S
 // through the z-facing sides of a control volume are carried from one plane
 // to the next.  Every flux is evaluated once: each thread takes those of its
 // own faces, four warps the ones on the tile's high (or low) side.
-constexpr int kZKM = 16;   // planes per CTA
-
 template <typename R>
 struct MomZ {
   R u[3][Plane<3>::N];    // u planes (m mod 3)
@@ -1195,7 +1211,7 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 3 : 2)
                const R* __restrict__ M0, const R* __restrict__ M1, const R* __restrict__ M2,
                R* __restrict__ us0, R* __restrict__ us1, R* __restrict__ us2,
                const double* __restrict__ dtp, R* __restrict__ ph0, R* __restrict__ ph1,
-               R* __restrict__ ph2) {
+               R* __restrict__ ph2, int kz) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   MomZ<R>& S = *reinterpret_cast<MomZ<R>*>(smem_raw);
   using P1 = Plane<1>;
@@ -1204,8 +1220,8 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 3 : 2)
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int i = blockIdx.x * kZX + tx, j = blockIdx.y * kZY + ty;
   const int x0 = blockIdx.x * kZX, y0 = blockIdx.y * kZY;
-  const int z0 = blockIdx.z * kZKM;
-  const int z1 = min(z0 + kZKM, nz);
+  const int z0 = blockIdx.z * kz;
+  const int z1 = min(z0 + kz, nz);
   const bool in = zcols_interior(g, 3);
   const bool col = i < nx && j < ny;
   const bool conc = X.c != nullptr;
@@ -1443,9 +1459,10 @@ void launch_momentum(const Geo& g, const Phys& ph, const TBC& tb, Fields<R> X, c
                      const double* dt, cudaStream_t s, R* const* phi) {
   const int smem = (int)sizeof(MomZ<R>);
   cudaFuncSetAttribute(k_momentum<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  k_momentum<R><<<zmarch_grid(g, kZKM), dim3(kZX, kZY), smem, s>>>(
+  const ZRuns z = zmarch_runs(g, sizeof(R) == 4 ? 512 : 1024, sizeof(R) == 4 ? 24 : 16);
+  k_momentum<R><<<z.grid, dim3(kZX, kZY), smem, s>>>(
       g, make_physr<R>(ph, g), tb, X, kappa, M0, M1, M2, us0, us1, us2, dt,
-      phi ? phi[0] : nullptr, phi ? phi[1] : nullptr, phi ? phi[2] : nullptr);
+      phi ? phi[0] : nullptr, phi ? phi[1] : nullptr, phi ? phi[2] : nullptr, z.kz);
 }
 
 // ---------------------------------------------------------------------------
