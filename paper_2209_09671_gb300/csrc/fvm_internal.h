@@ -79,6 +79,34 @@ constexpr int kMaxLevels = 24;
 constexpr int kBX = 32, kBY = 4, kBZ = 4;
 constexpr int kRedBlocks = 1024;   // partial-sum slots of the two-pass reductions
 
+// ----- launches that overlap their predecessor's end --------------------------
+// A kernel launched with overlap_launch() may be scheduled while the kernel
+// before it on the stream still runs; it calls dependency_wait() before it
+// touches memory, which returns once that kernel has completed and its writes
+// are visible, and so keeps the stream's order (of kernels before that one as
+// well: each waits for its own predecessor).
+template <typename... P, typename... A>
+inline void overlap_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                           A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#ifdef __CUDACC__
+// wait for the predecessor, and let the successor be scheduled
+__device__ __forceinline__ void dependency_wait() {
+  asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+}
+#endif
+
 // ----- stage launchers (fvm_stage.cu) --------------------------------------
 template <typename R>
 void launch_smooth(const Geo& g, const R* in, R* out, cudaStream_t s);

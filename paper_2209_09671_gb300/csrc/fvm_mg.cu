@@ -52,6 +52,7 @@ __device__ double block_sum_all(double v, double* sh) {
 template <typename T>
 __global__ void k_sum_field(const T* __restrict__ a, long long n, int squares,
                             double* __restrict__ partial) {
+  dependency_wait();
   __shared__ double sh[33];
   double acc = 0.0;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
@@ -65,6 +66,7 @@ __global__ void k_sum_field(const T* __restrict__ a, long long n, int squares,
 
 __global__ void k_sum_partials(const double* __restrict__ partial, int nparts,
                                double* __restrict__ out, const int* __restrict__ gate) {
+  dependency_wait();
   if (gate && !*gate) return;
   __shared__ double sh[33];
   double acc = 0.0;
@@ -75,19 +77,20 @@ __global__ void k_sum_partials(const double* __restrict__ partial, int nparts,
 
 void launch_sum_partials(const double* partial, int nparts, double* out, cudaStream_t s,
                          const int* gate) {
-  k_sum_partials<<<1, 1024, 0, s>>>(partial, nparts, out, gate);
+  overlap_launch(k_sum_partials, 1, 1024, 0, s, partial, nparts, out, gate);
 }
 
 template <typename T>
 void launch_sum_field(const T* a, long long n, bool squares, double* partial, double* out,
                       cudaStream_t s) {
-  k_sum_field<T><<<kRedBlocks, 256, 0, s>>>(a, n, squares ? 1 : 0, partial);
+  overlap_launch(k_sum_field<T>, kRedBlocks, 256, 0, s, a, n, squares ? 1 : 0, partial);
   launch_sum_partials(partial, kRedBlocks, out, s);
 }
 
 // a -= sum / n, with the mean formed once per block (one double division per
 // block instead of per element)
 __global__ void k_sub_mean(double* __restrict__ a, long long n, const double* __restrict__ sum) {
+  dependency_wait();
   __shared__ double mean;
   if (threadIdx.x == 0) mean = (*sum) / (double)n;
   __syncthreads();
@@ -97,18 +100,19 @@ __global__ void k_sub_mean(double* __restrict__ a, long long n, const double* __
 }
 
 void launch_sub_mean(double* a, long long n, const double* sum, cudaStream_t s) {
-  k_sub_mean<<<grid1d(n, 256), 256, 0, s>>>(a, n, sum);
+  overlap_launch(k_sub_mean, grid1d(n, 256), 256, 0, s, a, n, sum);
 }
 
 template <typename T>
 __global__ void k_zero(T* __restrict__ a, long long n) {
+  dependency_wait();
   long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c < n) a[c] = T(0);
 }
 
 template <typename T>
 void launch_zero(T* a, long long n, cudaStream_t s) {
-  k_zero<T><<<grid1d(n, 256), 256, 0, s>>>(a, n);
+  overlap_launch(k_zero<T>, grid1d(n, 256), 256, 0, s, a, n);
 }
 
 // ---------------------------------------------------------------------------
@@ -227,6 +231,7 @@ __device__ __forceinline__ T gs_value(const MGLevel<T>& L, int c, const OpNb<T>&
 
 template <typename T>
 __global__ void k_inv_diag(MGLevel<T> L) {
+  dependency_wait();
   const Geo& g = L.geo;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -246,7 +251,7 @@ template <typename T>
 void launch_inv_diag(const MGLevel<T>& L, cudaStream_t s) {
   const dim3 bs(32, 4, 2);
   const dim3 gs((L.geo.n[0] + 31) / 32, (L.geo.n[1] + 3) / 4, (L.geo.n[2] + 1) / 2);
-  k_inv_diag<T><<<gs, bs, 0, s>>>(L);
+  overlap_launch(k_inv_diag<T>, gs, bs, 0, s, L);
 }
 
 // Gauss-Seidel update of one cell (its colour's neighbours are fixed), which
@@ -272,6 +277,7 @@ __device__ __forceinline__ void gs_point(const MGLevel<T>& L, int i, int j, int 
 template <typename T>
 __global__ void k_gs(MGLevel<T> L, int colour, const int* __restrict__ gate, int gate_min,
                      const T* xin) {
+  dependency_wait();
   if (gate && *gate >= gate_min) return;
   const Geo& g = L.geo;
   const int i2 = blockIdx.x * blockDim.x + threadIdx.x;
@@ -289,7 +295,7 @@ void launch_gs(const MGLevel<T>& L, int colour, cudaStream_t s, const int* gate,
   const int hx = (L.geo.n[0] + 1) / 2;
   dim3 bs(32, 4, 2);
   dim3 gs((hx + 31) / 32, (L.geo.n[1] + 3) / 4, (L.geo.n[2] + 1) / 2);
-  k_gs<T><<<gs, bs, 0, s>>>(L, colour, gate, gate_min, xin);
+  overlap_launch(k_gs<T>, gs, bs, 0, s, L, colour, gate, gate_min, xin);
 }
 
 // coarse b = mean over children of (b - L x) on the fine level; coarse x = 0.
@@ -324,6 +330,7 @@ __device__ __forceinline__ void restrict_point(const MGLevel<T>& F, const MGLeve
 // one thread per coarse cell on a 3D grid (no index division per thread)
 template <typename T>
 __global__ void k_residual_restrict(MGLevel<T> F, MGLevel<T> C, int sweep, int half) {
+  dependency_wait();
   const int I = blockIdx.x * blockDim.x + threadIdx.x;
   const int J = blockIdx.y * blockDim.y + threadIdx.y;
   const int K = blockIdx.z * blockDim.z + threadIdx.z;
@@ -346,7 +353,7 @@ void launch_residual_restrict(const MGLevel<T>& F, const MGLevel<T>& C, cudaStre
                               bool half) {
   const dim3 bs(32, 4, 2);
   const dim3 gs((C.geo.n[0] + 31) / 32, (C.geo.n[1] + 3) / 4, (C.geo.n[2] + 1) / 2);
-  k_residual_restrict<T><<<gs, bs, 0, s>>>(F, C, sweep ? 1 : 0, half ? 1 : 0);
+  overlap_launch(k_residual_restrict<T>, gs, bs, 0, s, F, C, sweep ? 1 : 0, half ? 1 : 0);
 }
 
 // the coarsening factor of an axis is 1 or 2
@@ -364,6 +371,7 @@ __device__ __forceinline__ void prolong_point(const MGLevel<T>& F, const MGLevel
 // one thread per fine cell on a 3D grid (no index division per thread)
 template <typename T>
 __global__ void k_prolong(MGLevel<T> F, MGLevel<T> C) {
+  dependency_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z * blockDim.z + threadIdx.z;
@@ -375,7 +383,7 @@ template <typename T>
 void launch_prolong(const MGLevel<T>& F, const MGLevel<T>& C, cudaStream_t s) {
   const dim3 bs(32, 4, 2);
   const dim3 gs((F.geo.n[0] + 31) / 32, (F.geo.n[1] + 3) / 4, (F.geo.n[2] + 1) / 2);
-  k_prolong<T><<<gs, bs, 0, s>>>(F, C);
+  overlap_launch(k_prolong<T>, gs, bs, 0, s, F, C);
 }
 
 // The first colour sweep after the coarse correction with the
@@ -387,6 +395,7 @@ void launch_prolong(const MGLevel<T>& F, const MGLevel<T>& C, cudaStream_t s) {
 // launches would, bit for bit, without the prolongation's pass over x.
 template <typename T>
 __global__ void k_gs_prolong(MGLevel<T> F, MGLevel<T> C, int colour) {
+  dependency_wait();
   const Geo& g = F.geo;
   const int i2 = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -422,6 +431,7 @@ __global__ void k_gs_prolong(MGLevel<T> F, MGLevel<T> C, int colour) {
 // replaces zeroing x in a pass of its own.
 template <typename T>
 __global__ void k_gs_zero(MGLevel<T> L, int colour) {
+  dependency_wait();
   const Geo& g = L.geo;
   const int i2 = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -443,6 +453,7 @@ __global__ void k_gs_zero(MGLevel<T> L, int colour) {
 // correction e itself is stored only when the residual is updated with it
 // (k_residual_update); the next refinement starts it from 0.
 __global__ void k_gs_addp(MGLevel<float> L, int colour, double* __restrict__ p, int store) {
+  dependency_wait();
   const Geo& g = L.geo;
   const int i2 = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -470,14 +481,14 @@ void launch_gs_zero(const MGLevel<T>& L, int colour, cudaStream_t s) {
   const int hx = (L.geo.n[0] + 1) / 2;
   dim3 bs(32, 4, 2);
   dim3 gs((hx + 31) / 32, (L.geo.n[1] + 3) / 4, (L.geo.n[2] + 1) / 2);
-  k_gs_zero<T><<<gs, bs, 0, s>>>(L, colour);
+  overlap_launch(k_gs_zero<T>, gs, bs, 0, s, L, colour);
 }
 
 void launch_gs_addp(const MGLevel<float>& L, int colour, double* p, bool store, cudaStream_t s) {
   const int hx = (L.geo.n[0] + 1) / 2;
   dim3 bs(32, 4, 2);
   dim3 gs((hx + 31) / 32, (L.geo.n[1] + 3) / 4, (L.geo.n[2] + 1) / 2);
-  k_gs_addp<<<gs, bs, 0, s>>>(L, colour, p, store ? 1 : 0);
+  overlap_launch(k_gs_addp, gs, bs, 0, s, L, colour, p, store ? 1 : 0);
 }
 
 template <typename T>
@@ -485,11 +496,12 @@ void launch_gs_prolong(const MGLevel<T>& F, const MGLevel<T>& C, int colour, cud
   const int hx = (F.geo.n[0] + 1) / 2;
   dim3 bs(32, 4, 2);
   dim3 gs((hx + 31) / 32, (F.geo.n[1] + 3) / 4, (F.geo.n[2] + 1) / 2);
-  k_gs_prolong<T><<<gs, bs, 0, s>>>(F, C, colour);
+  overlap_launch(k_gs_prolong<T>, gs, bs, 0, s, F, C, colour);
 }
 
 template <typename T>
 __global__ void k_beta_coarsen(MGLevel<T> F, MGLevel<T> C) {
+  dependency_wait();
   long long cc = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (cc >= C.geo.N) return;
   int I, J, K;
@@ -510,7 +522,7 @@ __global__ void k_beta_coarsen(MGLevel<T> F, MGLevel<T> C) {
 
 template <typename T>
 void launch_beta_coarsen(const MGLevel<T>& F, const MGLevel<T>& C, cudaStream_t s) {
-  k_beta_coarsen<T><<<grid1d(C.geo.N, 128), 128, 0, s>>>(F, C);
+  overlap_launch(k_beta_coarsen<T>, grid1d(C.geo.N, 128), 128, 0, s, F, C);
 }
 
 // ---------------------------------------------------------------------------
@@ -593,6 +605,7 @@ void launch_coarse_cg(const MGLevel<T>& L, double* r, double* d, double* Ad, dou
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void k_residual_norm2(MGLevel<T> L, double* __restrict__ partial) {
+  dependency_wait();
   __shared__ double sh[33];
   double acc = 0.0;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < L.geo.N;
@@ -610,7 +623,7 @@ __global__ void k_residual_norm2(MGLevel<T> L, double* __restrict__ partial) {
 
 template <typename T>
 void launch_residual_norm2(const MGLevel<T>& L, double* partial, double* out, cudaStream_t s) {
-  k_residual_norm2<T><<<kRedBlocks, 256, 0, s>>>(L, partial);
+  overlap_launch(k_residual_norm2<T>, kRedBlocks, 256, 0, s, L, partial);
   launch_sum_partials(partial, kRedBlocks, out, s);
 }
 
@@ -635,6 +648,7 @@ __global__ void k_residual64(Geo g, const double* __restrict__ p, const double* 
                              const float* __restrict__ b2, float* __restrict__ r32,
                              double* __restrict__ partial, float* __restrict__ e32, W3 w32,
                              double* __restrict__ rd, const int* __restrict__ gate) {
+  dependency_wait();
   if (gate && !*gate) return;
   __shared__ double sh[33];
   const float* be[3] = {b0, b1, b2};
@@ -684,7 +698,7 @@ void launch_residual64(const Geo& g, const double* p, const double* b, float* co
   W3 w = {{0.f, 0.f, 0.f}};
   if (w32)
     for (int d = 0; d < 3; ++d) w.w[d] = w32[d];
-  k_residual64<<<kRedBlocks, 256, 0, s>>>(g, p, b, beta[0], beta[1], beta[2], r32, partial, e32, w,
+  overlap_launch(k_residual64, kRedBlocks, 256, 0, s, g, p, b, beta[0], beta[1], beta[2], r32, partial, e32, w,
                                           rd, gate);
   launch_sum_partials(partial, kRedBlocks, out, s, gate);
 }
@@ -736,6 +750,7 @@ __device__ __forceinline__ double pair_to_double(float f) {
 __global__ void __launch_bounds__(256)
     k_residual_update(MGLevel<float> L, double* __restrict__ rd, float* __restrict__ y,
                       double* __restrict__ partial, int tx, int ty, int chunks, int kz) {
+  dependency_wait();
   __shared__ double sh[33];
   const Geo& g = L.geo;
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2], nxy = nx * ny;
@@ -805,22 +820,24 @@ void launch_residual_update(const MGLevel<float>& L, double* rd, float* y, doubl
   chunks = (nz + kz - 1) / kz;
   const long long work = tiles * chunks;
   const int blocks = (int)(work < kRedBlocks ? work : kRedBlocks);
-  k_residual_update<<<blocks, 256, 0, s>>>(L, rd, y, partial, tx, ty, chunks, kz);
+  overlap_launch(k_residual_update, blocks, 256, 0, s, L, rd, y, partial, tx, ty, chunks, kz);
   launch_sum_partials(partial, blocks, out, s);
 }
 
 __global__ void k_add_correction(long long n, double* __restrict__ p, const float* __restrict__ e) {
+  dependency_wait();
   long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c < n) p[c] = p[c] + (double)e[c];
 }
 
 void launch_add_correction(long long n, double* p, const float* e, cudaStream_t s) {
-  k_add_correction<<<grid1d(n, 256), 256, 0, s>>>(n, p, e);
+  overlap_launch(k_add_correction, grid1d(n, 256), 256, 0, s, n, p, e);
 }
 
 // ---------------------------------------------------------------------------
 // device-side control of the pressure solve (one thread each)
 __global__ void k_ctl_reset(SolveCtl* ctl) {
+  dependency_wait();
   ctl->iters = 0;
   ctl->status = 0;
   ctl->zero = 0;
@@ -828,7 +845,7 @@ __global__ void k_ctl_reset(SolveCtl* ctl) {
   ctl->rel = 0.0;
 }
 
-void launch_ctl_reset(SolveCtl* ctl, cudaStream_t s) { k_ctl_reset<<<1, 1, 0, s>>>(ctl); }
+void launch_ctl_reset(SolveCtl* ctl, cudaStream_t s) { overlap_launch(k_ctl_reset, 1, 1, 0, s, ctl); }
 
 // the stopping rule of the host loop, on the device: stop on a non-finite
 // norm (EUNSTABLE), a zero right-hand side, after `fixed` cycles, at
@@ -836,6 +853,7 @@ void launch_ctl_reset(SolveCtl* ctl, cudaStream_t s) { k_ctl_reset<<<1, 1, 0, s>
 __global__ void k_ctl_step(cudaGraphConditionalHandle h, SolveCtl* ctl, const double* bn2p,
                            const double* r2p, double rtol, int maxit, int fixed,
                            unsigned long long* runs_total) {
+  dependency_wait();
   const double bn2 = *bn2p;
   unsigned go = 0;
   if (!isfinite(bn2)) {
@@ -865,11 +883,12 @@ __global__ void k_ctl_step(cudaGraphConditionalHandle h, SolveCtl* ctl, const do
 void launch_ctl_step(cudaGraphConditionalHandle h, SolveCtl* ctl, const double* bn2,
                      const double* r2, double rtol, int maxit, int fixed,
                      unsigned long long* runs_total, cudaStream_t s) {
-  k_ctl_step<<<1, 1, 0, s>>>(h, ctl, bn2, r2, rtol, maxit, fixed, runs_total);
+  overlap_launch(k_ctl_step, 1, 1, 0, s, h, ctl, bn2, r2, rtol, maxit, fixed, runs_total);
 }
 
 __global__ void k_ctl_check(SolveCtl* ctl, const double* bn2p, const double* r2p, double rtol,
                             int maxit, int fixed) {
+  dependency_wait();
   const double rel = sqrt(*r2p) / sqrt(*bn2p);
   const bool go = isfinite(rel) && (fixed > 0 ? ctl->iters < fixed
                                               : (rel > rtol && ctl->iters < maxit));
@@ -878,11 +897,12 @@ __global__ void k_ctl_check(SolveCtl* ctl, const double* bn2p, const double* r2p
 
 void launch_ctl_check(SolveCtl* ctl, const double* bn2, const double* r2, double rtol, int maxit,
                       int fixed, cudaStream_t s) {
-  k_ctl_check<<<1, 1, 0, s>>>(ctl, bn2, r2, rtol, maxit, fixed);
+  overlap_launch(k_ctl_check, 1, 1, 0, s, ctl, bn2, r2, rtol, maxit, fixed);
 }
 
 __global__ void k_zero_if_rhs_zero(const SolveCtl* __restrict__ ctl, double* __restrict__ p,
                                    long long n) {
+  dependency_wait();
   if (!ctl->zero) return;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
        c += (long long)gridDim.x * blockDim.x)
@@ -890,16 +910,17 @@ __global__ void k_zero_if_rhs_zero(const SolveCtl* __restrict__ ctl, double* __r
 }
 
 void launch_zero_if_rhs_zero(const SolveCtl* ctl, double* p, long long n, cudaStream_t s) {
-  k_zero_if_rhs_zero<<<kRedBlocks, 256, 0, s>>>(ctl, p, n);
+  overlap_launch(k_zero_if_rhs_zero, kRedBlocks, 256, 0, s, ctl, p, n);
 }
 
 __global__ void k_ctl_store(const SolveCtl* ctl, SolveCtl* rec, int* sticky) {
+  dependency_wait();
   *rec = *ctl;
   if (ctl->status) atomicMax(sticky, ctl->status);
 }
 
 void launch_ctl_store(const SolveCtl* ctl, SolveCtl* rec, int* sticky, cudaStream_t s) {
-  k_ctl_store<<<1, 1, 0, s>>>(ctl, rec, sticky);
+  overlap_launch(k_ctl_store, 1, 1, 0, s, ctl, rec, sticky);
 }
 
 #define FVM_MG_INST(T)                                                                       \

@@ -760,6 +760,7 @@ __device__ void fill_table(const TailArgs<T>& A, int l, char* sm, unsigned base,
 template <typename T>
 __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ TailArgs<T> A) {
   extern __shared__ __align__(16) char sm[];
+  dependency_wait();
   const int rank = (int)cluster_rank();
   const unsigned base = smem_u32(sm);
   const int last = A.nl - 1;
@@ -866,6 +867,7 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
 // the coefficient blocks of every level and CTA, once per solve
 template <typename T>
 __global__ void k_tail_pack(const __grid_constant__ TailArgs<T> A) {
+  dependency_wait();
   const int l = blockIdx.y, rank = blockIdx.x;
   const TailLevel<T>& L = A.L[l];
   if (rank >= L.nact) return;
@@ -890,6 +892,7 @@ __global__ void k_tail_pack(const __grid_constant__ TailArgs<T> A) {
 template <typename T>
 __global__ void k_inv_init(const __grid_constant__ TailLevel<T> L, float* __restrict__ W, int np,
                            double* __restrict__ gscale) {
+  dependency_wait();
   __shared__ float part[8];
   const int nx = L.n[0], N = L.rows * nx;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -936,6 +939,7 @@ __global__ void k_inv_init(const __grid_constant__ TailLevel<T> L, float* __rest
 // subtracts A[tile, pivots] X
 __global__ void __launch_bounds__(256) k_inv_step(const float* __restrict__ A,
                                                   float* __restrict__ B, int np, int b) {
+  dependency_wait();
   __shared__ float D[2][32][33];
   __shared__ __align__(16) float Ct[32][68], R[32][64], X[32][64];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -1019,9 +1023,9 @@ template <typename T>
 void launch_tail_inverse(const TailArgs<T>& A, float* W0, float* W1, double* gscale,
                          cudaStream_t s) {
   const int nb = inverse_blocks(A), nt = A.np / 64;
-  k_inv_init<T><<<A.np / 8, 256, 0, s>>>(A.L[A.nl - 1], W0, A.np, gscale);
+  overlap_launch(k_inv_init<T>, A.np / 8, 256, 0, s, A.L[A.nl - 1], W0, A.np, gscale);
   for (int b = 0; b < nb; ++b)
-    k_inv_step<<<dim3(nt, nt), 256, 0, s>>>(b & 1 ? W1 : W0, b & 1 ? W0 : W1, A.np, b);
+    overlap_launch(k_inv_step, dim3(nt, nt), 256, 0, s, b & 1 ? W1 : W0, b & 1 ? W0 : W1, A.np, b);
 }
 
 // Layout of a tail that starts at level Ls[0] with nl levels; false when it
@@ -1096,7 +1100,7 @@ bool tail_layout(const MGLevel<T>* Ls, int nl, bool inverse, TailArgs<T>& A, siz
 
 template <typename T>
 void launch_tail_pack(const TailArgs<T>& A, cudaStream_t s) {
-  k_tail_pack<T><<<dim3(kTailCTAs, A.nl, 2), 256, 0, s>>>(A);
+  overlap_launch(k_tail_pack<T>, dim3(kTailCTAs, A.nl, 2), 256, 0, s, A);
 }
 
 template <typename T>
@@ -1108,13 +1112,15 @@ void launch_tail(const TailArgs<T>& A, size_t smem, cudaStream_t s) {
   cfg.blockDim = dim3(kTailThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = kTailCTAs;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   cudaLaunchKernelEx(&cfg, k_tail<T>, A);
 }
 
