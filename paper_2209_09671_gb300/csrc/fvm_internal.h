@@ -84,7 +84,10 @@ constexpr int kRedBlocks = 1024;   // partial-sum slots of the two-pass reductio
 // before it on the stream still runs; it calls dependency_wait() before it
 // touches memory, which returns once that kernel has completed and its writes
 // are visible, and so keeps the stream's order (of kernels before that one as
-// well: each waits for its own predecessor).
+// well: each waits for its own predecessor).  Such a kernel reads what earlier
+// ones wrote with plain loads only: a pointer to const __restrict__ or __ldg
+// allows the read-only path, whose data must not change while the kernel runs,
+// and it is running before its predecessor has finished.
 template <typename... P, typename... A>
 inline void overlap_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                            A... args) {

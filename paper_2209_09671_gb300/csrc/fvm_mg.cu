@@ -50,8 +50,8 @@ __device__ double block_sum_all(double v, double* sh) {
 
 // ---------------------------------------------------------------------------
 template <typename T>
-__global__ void k_sum_field(const T* __restrict__ a, long long n, int squares,
-                            double* __restrict__ partial) {
+__global__ void k_sum_field(const T* a, long long n, int squares,
+                            double* partial) {
   dependency_wait();
   __shared__ double sh[33];
   double acc = 0.0;
@@ -64,8 +64,8 @@ __global__ void k_sum_field(const T* __restrict__ a, long long n, int squares,
   if (threadIdx.x == 0) partial[blockIdx.x] = s;
 }
 
-__global__ void k_sum_partials(const double* __restrict__ partial, int nparts,
-                               double* __restrict__ out, const int* __restrict__ gate) {
+__global__ void k_sum_partials(const double* partial, int nparts,
+                               double* out, const int* gate) {
   dependency_wait();
   if (gate && !*gate) return;
   __shared__ double sh[33];
@@ -89,7 +89,7 @@ void launch_sum_field(const T* a, long long n, bool squares, double* partial, do
 
 // a -= sum / n, with the mean formed once per block (one double division per
 // block instead of per element)
-__global__ void k_sub_mean(double* __restrict__ a, long long n, const double* __restrict__ sum) {
+__global__ void k_sub_mean(double* a, long long n, const double* sum) {
   dependency_wait();
   __shared__ double mean;
   if (threadIdx.x == 0) mean = (*sum) / (double)n;
@@ -104,7 +104,7 @@ void launch_sub_mean(double* a, long long n, const double* sum, cudaStream_t s) 
 }
 
 template <typename T>
-__global__ void k_zero(T* __restrict__ a, long long n) {
+__global__ void k_zero(T* a, long long n) {
   dependency_wait();
   long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c < n) a[c] = T(0);
@@ -142,7 +142,7 @@ __device__ __forceinline__ void neighbours(const MGLevel<T>& L, int i, int j, in
 }
 
 template <typename T, typename X>
-__device__ __forceinline__ X apply_L_at(const MGLevel<T>& L, const X* __restrict__ x, int c,
+__device__ __forceinline__ X apply_L_at(const MGLevel<T>& L, const X* x, int c,
                                         const OpNb<T>& nb) {
   const Geo& g = L.geo;
   X xc = x[c];
@@ -275,7 +275,7 @@ __device__ __forceinline__ void gs_point(const MGLevel<T>& L, int i, int j, int 
 // solve graph skips the first sweep of every cycle after the first, which
 // would repeat the previous cycle's last sweep)
 template <typename T>
-__global__ void k_gs(MGLevel<T> L, int colour, const int* __restrict__ gate, int gate_min,
+__global__ void k_gs(MGLevel<T> L, int colour, const int* gate, int gate_min,
                      const T* xin) {
   dependency_wait();
   if (gate && *gate >= gate_min) return;
@@ -452,7 +452,7 @@ __global__ void k_gs_zero(MGLevel<T> L, int colour) {
 // colour's cell beside it (not written in this sweep) to the double p.  The
 // correction e itself is stored only when the residual is updated with it
 // (k_residual_update); the next refinement starts it from 0.
-__global__ void k_gs_addp(MGLevel<float> L, int colour, double* __restrict__ p, int store) {
+__global__ void k_gs_addp(MGLevel<float> L, int colour, double* p, int store) {
   dependency_wait();
   const Geo& g = L.geo;
   const int i2 = blockIdx.x * blockDim.x + threadIdx.x;
@@ -530,8 +530,8 @@ void launch_beta_coarsen(const MGLevel<T>& F, const MGLevel<T>& C, cudaStream_t 
 // x0 = 0, stop at ||r|| <= rtol ||b|| or on breakdown, mean-free result.
 // The vectors are double in both precisions.
 template <typename T>
-__device__ void coarse_cg_block(const MGLevel<T>& L, double* __restrict__ r,
-                                double* __restrict__ dd, double* __restrict__ Ad, double rtol,
+__device__ void coarse_cg_block(const MGLevel<T>& L, double* r,
+                                double* dd, double* Ad, double rtol,
                                 int maxit, double* sh) {
   const Geo& g = L.geo;
   const int N = (int)g.N;
@@ -588,9 +588,9 @@ __device__ void coarse_cg_block(const MGLevel<T>& L, double* __restrict__ r,
 }
 
 template <typename T>
-__global__ void __launch_bounds__(1024) k_coarse_cg(MGLevel<T> L, double* __restrict__ r,
-                                                    double* __restrict__ dd,
-                                                    double* __restrict__ Ad, double rtol,
+__global__ void __launch_bounds__(1024) k_coarse_cg(MGLevel<T> L, double* r,
+                                                    double* dd,
+                                                    double* Ad, double rtol,
                                                     int maxit) {
   __shared__ double sh[33];
   coarse_cg_block(L, r, dd, Ad, rtol, maxit, sh);
@@ -604,7 +604,7 @@ void launch_coarse_cg(const MGLevel<T>& L, double* r, double* d, double* Ad, dou
 
 // ---------------------------------------------------------------------------
 template <typename T>
-__global__ void k_residual_norm2(MGLevel<T> L, double* __restrict__ partial) {
+__global__ void k_residual_norm2(MGLevel<T> L, double* partial) {
   dependency_wait();
   __shared__ double sh[33];
   double acc = 0.0;
@@ -643,11 +643,11 @@ __device__ __forceinline__ double beta_to_double(float f) {
 // from e = 0, the other colour 0) is taken here, from the float residual just
 // stored, with the same arithmetic as k_gs_zero: the inner solve then starts
 // at its second sweep.  w32: the finest level's float 1/h^2 per axis.
-__global__ void k_residual64(Geo g, const double* __restrict__ p, const double* __restrict__ b,
-                             const float* __restrict__ b0, const float* __restrict__ b1,
-                             const float* __restrict__ b2, float* __restrict__ r32,
-                             double* __restrict__ partial, float* __restrict__ e32, W3 w32,
-                             double* __restrict__ rd, const int* __restrict__ gate) {
+__global__ void k_residual64(Geo g, const double* p, const double* b,
+                             const float* b0, const float* b1,
+                             const float* b2, float* r32,
+                             double* partial, float* e32, W3 w32,
+                             double* rd, const int* gate) {
   dependency_wait();
   if (gate && !*gate) return;
   __shared__ double sh[33];
@@ -748,15 +748,15 @@ __device__ __forceinline__ double pair_to_double(float f) {
 // A thread owns a column of cells and walks planes k0 .. k1-1 upward; the
 // product of a z-face serves the cells on both of its sides.
 __global__ void __launch_bounds__(256)
-    k_residual_update(MGLevel<float> L, double* __restrict__ rd, float* __restrict__ y,
-                      double* __restrict__ partial, int tx, int ty, int chunks, int kz) {
+    k_residual_update(MGLevel<float> L, double* rd, float* y,
+                      double* partial, int tx, int ty, int chunks, int kz) {
   dependency_wait();
   __shared__ double sh[33];
   const Geo& g = L.geo;
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2], nxy = nx * ny;
-  const float* __restrict__ e = L.x;
-  const float *__restrict__ b0 = L.beta[0], *__restrict__ b1 = L.beta[1],
-              *__restrict__ b2 = L.beta[2];
+  const float* e = L.x;
+  const float *b0 = L.beta[0], *b1 = L.beta[1],
+              *b2 = L.beta[2];
   const double w = (double)g.w[nx > 1 ? 0 : (ny > 1 ? 1 : 2)];
   double acc = 0.0;
   for (int t = blockIdx.x; t < tx * ty * chunks; t += gridDim.x) {
@@ -824,7 +824,7 @@ void launch_residual_update(const MGLevel<float>& L, double* rd, float* y, doubl
   launch_sum_partials(partial, blocks, out, s);
 }
 
-__global__ void k_add_correction(long long n, double* __restrict__ p, const float* __restrict__ e) {
+__global__ void k_add_correction(long long n, double* p, const float* e) {
   dependency_wait();
   long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c < n) p[c] = p[c] + (double)e[c];
@@ -900,7 +900,7 @@ void launch_ctl_check(SolveCtl* ctl, const double* bn2, const double* r2, double
   overlap_launch(k_ctl_check, 1, 1, 0, s, ctl, bn2, r2, rtol, maxit, fixed);
 }
 
-__global__ void k_zero_if_rhs_zero(const SolveCtl* __restrict__ ctl, double* __restrict__ p,
+__global__ void k_zero_if_rhs_zero(const SolveCtl* ctl, double* p,
                                    long long n) {
   dependency_wait();
   if (!ctl->zero) return;

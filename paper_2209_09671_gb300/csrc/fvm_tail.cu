@@ -139,7 +139,7 @@ __device__ void fill_coefs(const TailLevel<T>& L, bool coarsest, void* dst, int 
 // diagonal: Gauss-Jordan without pivoting (the matrix is symmetric and positive
 // definite: L has the constants as its only null vectors), by one block
 template <typename T>
-__device__ void coarsest_inverse(const TailLevel<T>& L, double* __restrict__ G) {
+__device__ void coarsest_inverse(const TailLevel<T>& L, double* G) {
   __shared__ double M[32][33];
   __shared__ double diag[32];
   const int N = L.rows * L.n[0], nx = L.n[0], ny = L.n[1];
@@ -540,7 +540,7 @@ __device__ bool coarsest_refine(const View<T>& V, const TailArgs<T>& A, Reduce& 
     if (threadIdx.x == 0) {
       const int e = (int)((__double2hiint(rr) >> 20) & 0x7ff) - 1023;
       bmean[1] = __hiloint2double((1023 - (e >> 1)) << 20, 0);
-      bmean[2] = 1.0 / (bmean[1] * __ldg(A.gscale));
+      bmean[2] = 1.0 / (bmean[1] * (*A.gscale));
     }
     __syncthreads();
     const double scale = bmean[1], back = bmean[2];
@@ -568,8 +568,8 @@ __device__ bool coarsest_refine(const View<T>& V, const TailArgs<T>& A, Reduce& 
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
           if (r0 + m >= own) continue;
-          const float4 g = __ldg(reinterpret_cast<const float4*>(
-                                     A.G + (size_t)(V.rank * chunk + r0 + m) * np) + c);
+          const float4 g = reinterpret_cast<const float4*>(
+              A.G + (size_t)(V.rank * chunk + r0 + m) * np)[c];
           s[m] += g.x * v.x + g.y * v.y + g.z * v.z + g.w * v.w;
         }
       }
@@ -772,7 +772,7 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
     if (A.pack) {
       const int4* src = reinterpret_cast<const int4*>((const char*)A.pack + L.opack + (size_t)rank * bytes);
       int4* dst = reinterpret_cast<int4*>(sm + L.oa);
-      for (int t = threadIdx.x; t < bytes / 16; t += kTailThreads) dst[t] = __ldg(src + t);
+      for (int t = threadIdx.x; t < bytes / 16; t += kTailThreads) dst[t] = src[t];
     } else {
       fill_coefs(L, l == last, sm + L.oa, rank, threadIdx.x, kTailThreads);
     }
@@ -803,7 +803,7 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(const __grid_constant__ T
       const int i = p < L.hx ? 2 * p : 2 * (p - L.hx) + 1;
       if (i >= L.n[0]) continue;
       const int c = (rank * L.rpc + q) * L.n[0] + i;
-      const T b = __ldg(L.b + c);
+      const T b = L.b[c];
       V.b()[t] = b;
       if (A.ctl) V.x()[t] = L.x[c];
       else if (last > 0) V.x()[t] = first_x(V, t, i, V.tab()[2 * q + 1].y, b, A.pre > 0);
@@ -890,9 +890,8 @@ __global__ void k_tail_pack(const __grid_constant__ TailArgs<T> A) {
 // 32 x 32 tiles, whose CTAs are more and each repeat the pivot block's
 // inverse, took 17 us per block for 625 cells, 32 us for 990.
 template <typename T>
-__global__ void k_inv_init(const __grid_constant__ TailLevel<T> L, float* __restrict__ W, int np,
-                           double* __restrict__ gscale) {
-  dependency_wait();
+__global__ void k_inv_init(const __grid_constant__ TailLevel<T> L, float* W, int np,
+                           double* gscale) {
   __shared__ float part[8];
   const int nx = L.n[0], N = L.rows * nx;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -939,7 +938,6 @@ __global__ void k_inv_init(const __grid_constant__ TailLevel<T> L, float* __rest
 // subtracts A[tile, pivots] X
 __global__ void __launch_bounds__(256) k_inv_step(const float* __restrict__ A,
                                                   float* __restrict__ B, int np, int b) {
-  dependency_wait();
   __shared__ float D[2][32][33];
   __shared__ __align__(16) float Ct[32][68], R[32][64], X[32][64];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -1023,9 +1021,9 @@ template <typename T>
 void launch_tail_inverse(const TailArgs<T>& A, float* W0, float* W1, double* gscale,
                          cudaStream_t s) {
   const int nb = inverse_blocks(A), nt = A.np / 64;
-  overlap_launch(k_inv_init<T>, A.np / 8, 256, 0, s, A.L[A.nl - 1], W0, A.np, gscale);
+  k_inv_init<T><<<A.np / 8, 256, 0, s>>>(A.L[A.nl - 1], W0, A.np, gscale);
   for (int b = 0; b < nb; ++b)
-    overlap_launch(k_inv_step, dim3(nt, nt), 256, 0, s, b & 1 ? W1 : W0, b & 1 ? W0 : W1, A.np, b);
+    k_inv_step<<<dim3(nt, nt), 256, 0, s>>>(b & 1 ? W1 : W0, b & 1 ? W0 : W1, A.np, b);
 }
 
 // Layout of a tail that starts at level Ls[0] with nl levels; false when it
