@@ -285,6 +285,13 @@ __global__ void k_gs(MGLevel<T> L, int colour, const int* gate, int gate_min,
   const int k = blockIdx.z * blockDim.z + threadIdx.z;
   if (j >= g.n[1] || k >= g.n[2]) return;
   const int i = 2 * i2 + ((colour + j + k) & 1);
+  if (xin) {
+    // the other colour's first-sweep values move to x: on an axis with walls and
+    // an odd number of cells the wrapped neighbour of a wall cell (times beta = 0)
+    // has the cell's own colour, so the next sweep reads them there
+    const int io = i ^ 1, row = (k * g.n[1] + j) * g.n[0];
+    if (io < g.n[0]) L.x[row + io] = xin[row + io];
+  }
   if (i >= g.n[0]) return;
   gs_point(L, i, j, k, xin ? xin : L.x);
 }

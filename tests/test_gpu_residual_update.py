@@ -20,7 +20,7 @@ def _solve(P, p, alpha, rhs, host_loop=False):
     if host_loop:
         s.fvm_profile(True)
     dp = torch.zeros(p.shape, dtype=torch.float64, device="cuda")
-    info = s.fvm_poisson_solve(torch.tensor(alpha, device="cuda"), torch.tensor(rhs, device="cuda"), dp)
+    info = s.fvm_poisson_solve(torch.as_tensor(alpha, device="cuda"), torch.tensor(rhs, device="cuda"), dp)
     s.close()
     return dp.cpu(), info
 
@@ -67,3 +67,24 @@ def test_reported_residual_is_that_of_the_pressure(nx, ny, nz, bc, kw):
     host, hinfo = _solve(P, p, alpha, rhs, host_loop=True)
     assert hinfo["vcycles"][0] == info["vcycles"][0]
     assert torch.equal(host, got)
+
+
+def test_a_failed_solve_leaves_nothing_behind():
+    """A solve whose residual overflows float, then one on the same context: the
+    bits of a fresh context, also where an axis has walls and an odd number of
+    cells (a wall cell's wrapped neighbour then has the cell's own colour)."""
+    P = need_gpu()
+    p = cases.Params(nx=100, ny=76, nz=71, h=0.01, bc=(W, W, W), rho=(1.0, 2.0),
+                     precision=cases.MIXED, mg_max_cycles=30)
+    alpha = torch.tensor((cases.uniform(5, p.shape, 0, 1) > 0.5).astype(np.float32), device="cuda")
+    rhs = cases.uniform(31, p.shape, -1, 1)
+    fresh, info = _solve(P, p, alpha, rhs)
+    assert info["status"] == 0
+    s = P.Solver(p)
+    dp = torch.zeros(p.shape, dtype=torch.float64, device="cuda")
+    bad = s.fvm_poisson_solve(alpha, torch.tensor(rhs * 1e60, device="cuda"), dp, raise_on_error=False)
+    assert bad["status"] != 0
+    dp.zero_()
+    s.fvm_poisson_solve(alpha, torch.tensor(rhs, device="cuda"), dp)
+    s.close()
+    assert torch.equal(dp.cpu(), fresh)
