@@ -1073,8 +1073,9 @@ fvm_status stage(fvm_ctx* c, Fields<R> X, Fields<R> Sn, Fields<R> Y, double* p, 
     TIMED(c, FVM_K_SCALARS, 1, launch_concentration<R>(g, c->ph, X, Sn, Y, c->dt_dev, ca, cb, s));
   TIMED(c, FVM_K_MOMENTUM, 1, launch_momentum<R>(g, c->ph, c->tb, X, (R*)c->kappa, M[0], M[1], M[2],
                                               us[0], us[1], us[2], c->dt_dev, s));
-  TIMED(c, FVM_K_DIV_RHS, 1, launch_div_rhs<R>(g, us, c->dt_dev, c->b, c->partial, s));
-  TIMED(c, FVM_K_MISC, 1, launch_sum_partials(c->partial, kRedBlocks, c->scal + 3, s));
+  int parts = 0;
+  TIMED(c, FVM_K_DIV_RHS, 1, parts = launch_div_rhs<R>(g, us, c->dt_dev, c->b, c->partial, s));
+  TIMED(c, FVM_K_MISC, 1, launch_sum_partials(c->partial, parts, c->scal + 3, s));
   TIMED(c, FVM_K_MISC, 1, launch_sub_mean(c->b, g.N, c->scal + 3, s));
   fvm_status st;
   if (c->mixed) {
@@ -1491,8 +1492,10 @@ fvm_status adjoint_stage(fvm_ctx* c, const double* const* X, double xc, double* 
   double* lus[3] = {(double*)c->us[0], (double*)c->us[1], (double*)c->us[2]};
   TIMED(c, FVM_K_ADJOINT, 1, launch_zero_wall_faces(g, aEu, s));
   TIMED(c, FVM_K_ADJOINT, 1, launch_face_mul(g, be, aEu, wbeta, s));
-  TIMED(c, FVM_K_DIV_RHS, 1, launch_div_rhs<double>(g, wbeta, c->dt_dev, c->b, c->partial, s));
-  TIMED(c, FVM_K_MISC, 1, launch_sum_partials(c->partial, kRedBlocks, c->scal + 3, s));
+  int parts = 0;
+  TIMED(c, FVM_K_DIV_RHS, 1,
+        parts = launch_div_rhs<double>(g, wbeta, c->dt_dev, c->b, c->partial, s));
+  TIMED(c, FVM_K_MISC, 1, launch_sum_partials(c->partial, parts, c->scal + 3, s));
   TIMED(c, FVM_K_MISC, 1, launch_sub_mean(c->b, N, c->scal + 3, s));
   TIMED(c, FVM_K_MISC, 1, launch_zero<double>(c->ap, N, s));
   fvm_status st = solve_f64(c, c->ap, c->b, cyc, rel, true);

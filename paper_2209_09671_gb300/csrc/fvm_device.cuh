@@ -138,6 +138,21 @@ __device__ __forceinline__ double quotient(double n, double d) {
 }
 __device__ __forceinline__ float quotient(float n, float d) { return n / d; }
 
+// float -> double, exact, with integer operations for normal numbers and zero:
+// the conversion instruction takes the FP64 pipe for as long as two
+// additions.  It is kept for subnormal numbers, infinities and NaN, as volatile
+// assembly so that the compiler does not issue it for every value and select.
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f), mag = u & 0x7fffffffu;
+  double d = __hiloint2double((int)((u & 0x80000000u) | ((mag >> 3) + 0x38000000u)), (int)(u << 29));
+  if (mag - 0x00800000u >= 0x7f000000u) {
+    d = 0.0;
+    if (mag != 0u) asm volatile("cvt.f64.f32 %0, %1;" : "=d"(d) : "f"(f));
+  }
+  return d;
+}
+
 // sqrt(a) for a >= 0 to about a unit in the last place: the approximate
 // reciprocal root y and one Newton step on a y, with the rounding error of
 // that product (5 FP64 operations instead of about 15).  Below 2^-960 (a

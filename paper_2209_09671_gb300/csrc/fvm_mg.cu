@@ -717,7 +717,7 @@ void launch_residual64(const Geo& g, const double* p, const double* b, float* co
 // two-sum, the fused product error) and summed as such: 48 bits in float
 // arithmetic, which the GPU does 64 times as fast as double.  Formed from p
 // (k_residual64, 14 FP64 operations a cell) the pass is bound by the FP64
-// pipe: 0.56 ms at 256^3 against 0.29 ms here.  Its error, 2^-48 beta |de| of a
+// pipe: 0.56 ms at 256^3 against 0.19 ms here.  Its error, 2^-48 beta |de| of a
 // face, is that of rounding p itself (2^-53 beta |p|) once e varies over 32
 // cells and more, and it does not grow: the solve forms the residual from p
 // again before it stops, and goes on from that one if it is above the
@@ -745,16 +745,9 @@ __device__ __forceinline__ void pair_add(FloatPair& s, float h, float l) {
   s.l = __fadd_rn(s.l, __fadd_rn(e, l));
 }
 
-// float -> double with integer operations (as beta_to_double; an infinity or a
-// NaN takes the conversion instruction)
-__device__ __forceinline__ double pair_to_double(float f) {
-  if ((__float_as_uint(f) & 0x7fffffffu) >= 0x7f800000u) return (double)f;
-  return beta_to_double(f);
-}
-
 // A thread owns a column of cells and walks planes k0 .. k1-1 upward; the
 // product of a z-face serves the cells on both of its sides.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 6)
     k_residual_update(MGLevel<float> L, double* rd, float* y,
                       double* partial, int tx, int ty, int chunks, int kz) {
   dependency_wait();
@@ -797,7 +790,7 @@ __global__ void __launch_bounds__(256)
       pair_add(s, f.h, f.l);
       zl.h = -f.h;
       zl.l = -f.l;
-      const double r = fma(-w, pair_to_double(s.l), fma(-w, pair_to_double(s.h), rd[c]));
+      const double r = fma(-w, widen(s.l), fma(-w, widen(s.h), rd[c]));
       rd[c] = r;
       const float rf = (float)r;
       L.b[c] = rf;
@@ -817,18 +810,10 @@ __global__ void __launch_bounds__(256)
 
 void launch_residual_update(const MGLevel<float>& L, double* rd, float* y, double* partial,
                             double* out, cudaStream_t s) {
-  // about kRedBlocks blocks, each a 32 x 8 tile of columns and a run of at
-  // least 16 planes
-  const int tx = (L.geo.n[0] + 31) / 32, ty = (L.geo.n[1] + 7) / 8, nz = L.geo.n[2];
-  const long long tiles = (long long)tx * ty;
-  int chunks = (int)(tiles >= kRedBlocks ? 1 : kRedBlocks / tiles);
-  int kz = (nz + chunks - 1) / chunks;
-  if (kz < 16) kz = nz < 16 ? nz : 16;
-  chunks = (nz + kz - 1) / kz;
-  const long long work = tiles * chunks;
-  const int blocks = (int)(work < kRedBlocks ? work : kRedBlocks);
-  overlap_launch(k_residual_update, blocks, 256, 0, s, L, rd, y, partial, tx, ty, chunks, kz);
-  launch_sum_partials(partial, blocks, out, s);
+  const ColumnRuns r = column_runs(L.geo);
+  overlap_launch(k_residual_update, r.blocks, 256, 0, s, L, rd, y, partial, r.tx, r.ty, r.chunks,
+                 r.kz);
+  launch_sum_partials(partial, r.blocks, out, s);
 }
 
 __global__ void k_add_correction(long long n, double* p, const float* e) {

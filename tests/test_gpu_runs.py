@@ -32,3 +32,33 @@ def test_predictor_equals_oracle(nx, ny, nz, precision):
     for k in ("alpha", "T"):
         assert rel_l2(got[k].double().cpu().numpy(), ref[k].numpy()) <= tol["alpha"], k
     solver.close()
+
+
+@pytest.mark.parametrize("nx,ny,nz", [(40, 20, 7), (160, 96, 44), (200, 120, 107)])
+@pytest.mark.parametrize("precision", [cases.F64, cases.MIXED])
+def test_projected_velocity_is_divergence_free(nx, ny, nz, precision):
+    """From rest each stage's divergence is -dt times its solve's residual, at
+    most the solve's tolerance times |D u*|, plus roundings of the velocities; a
+    right-hand side wrong in one plane or column leaves |D u*| there.  Factors: 2
+    for the stages after the first, 6 faces a cell and 4 roundings a face."""
+    P = need_gpu()
+    p = _physics_case(nx, ny, nz, (1, 0, 1), 2).replace(precision=precision, mg_fixed_cycles=0)
+    s = cases.random_smooth_state(p, amp_u=0.0)
+    dt = 1e-3
+    solver = P.Solver(p)
+    d = P.to_device(s, precision == cases.MIXED)
+    star = solver.fvm_stage_predict(d, 3, dt)
+
+    def div(f):
+        u, v, w = (f[k].double().cpu() for k in ("u", "v", "w"))
+        return sum((a.roll(-1, 2 - q) - a) / p.h for q, a in enumerate((u, v, w)))
+
+    before = div(star)
+    solver.fvm_step(d, 3, dt)
+    torch.cuda.synchronize()
+    umax = max(float(star[k].abs().max()) for k in ("u", "v", "w"))
+    eps = 2.0 ** (-53 if precision == cases.F64 else -24)
+    bound = 2 * p.mg_rtol * float(before.norm()) + 24 * eps * umax / p.h * before.numel() ** 0.5
+    assert float(div(d).norm()) <= bound
+    assert bound < 1e-2 * float(before.norm())
+    solver.close()
