@@ -153,6 +153,27 @@ __device__ __forceinline__ double widen(float f) {
   return d;
 }
 
+// double -> R, rounded to nearest even; to float with integer operations where
+// the result is a normal number or zero (the same reason)
+template <typename R>
+__device__ __forceinline__ R narrow(double d);
+template <>
+__device__ __forceinline__ double narrow<double>(double d) { return d; }
+template <>
+__device__ __forceinline__ float narrow<float>(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const unsigned sign = hi & 0x80000000u, mag = hi & 0x7fffffffu;
+  unsigned r = sign | ((mag - 0x38000000u) << 3) | (lo >> 29);
+  const unsigned rest = lo << 3;
+  if (rest > 0x80000000u || (rest == 0x80000000u && (r & 1u))) ++r;
+  float f = __uint_as_float(r);
+  if (mag - 0x38100000u >= 0x0fe00000u) {   // not 2^-126 <= |d| < 2^128
+    f = __uint_as_float(sign);
+    if ((mag | lo) != 0u) asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(f) : "d"(d));
+  }
+  return f;
+}
+
 // sqrt(a) for a >= 0 to about a unit in the last place: the approximate
 // reciprocal root y and one Newton step on a y, with the rounding error of
 // that product (5 FP64 operations instead of about 15).  Below 2^-960 (a
