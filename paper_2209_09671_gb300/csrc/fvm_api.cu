@@ -485,11 +485,21 @@ inline void addp_sweep(fvm_ctx* c, int kg, const MGLevel<float>& L, int colour, 
 }
 inline void addp_sweep(fvm_ctx*, int, const MGLevel<double>&, int, double*, bool) {}
 
+inline void pair_sweep(fvm_ctx* c, int kg, MGLevel<float>& L, const MGLevel<float>* C, int colour,
+                       double* p, bool keep) {
+  TIMED(c, kg, 1, launch_gs_pair(L, C, colour, p, keep, c->stream));
+  float* x = L.x;
+  L.x = L.x2;
+  L.x2 = x;
+}
+inline void pair_sweep(fvm_ctx*, int, MGLevel<double>&, const MGLevel<double>*, int, double*, bool) {}
+
 // `iters` Gauss-Seidel iterations on level l: a sweep of colour `first`,
 // then one of the other colour.  The first sweep can apply the coarse
 // correction (k_gs_prolong) or start from x = 0 (k_gs_zero), the last one can
 // add x to p (k_gs_addp): each replaces a pass of its own over x, with the
 // same numbers.
+// On a level with a second array an even number of sweeps left is taken in pairs.
 template <typename T>
 void smooth(fvm_ctx* c, MGLevel<T>& L, int l, int iters, int first,
             const SweepFold<T>& f = SweepFold<T>()) {
@@ -498,6 +508,13 @@ void smooth(fvm_ctx* c, MGLevel<T>& L, int l, int iters, int first,
   for (int t = 0; t <= last; ++t) {
     const int colour = (t & 1) == 0 ? first : 1 - first;
     if (t == 0 && f.skip_first) continue;
+    const bool alone = (last - t) % 2 == 0 || (t == 0 && (f.zero || f.gate));
+    if (L.x2 && !alone) {
+      pair_sweep(c, kg, L, t == 0 ? f.corr : nullptr, colour, t + 1 == last ? f.addp : nullptr,
+                 f.keep);
+      ++t;
+      continue;
+    }
     if (t == 0 && f.corr)
       TIMED(c, kg, 1, launch_gs_prolong<T>(L, *f.corr, colour, c->stream));
     else if (t == 0 && f.zero)
@@ -785,6 +802,20 @@ void refine_once(fvm_ctx* c, MGLevel<float>* Ls, const float* alpha, double* p, 
   // with the other colour unchanged: it would write the same values again,
   // so it is skipped (when both smoothing steps sweep on the finest level)
   const int startq = first_sweep_repeats(c) ? kStartFirstSwept : kStartAsIs;
+  if (residual_updated(c) && c->nlev > 1 && pairs_fit(c->g, c->shp[0].f[0])) {
+    // the finest level's sweeps in pairs between e32 and y; the correction has to
+    // end in e32, since the update reads it while it leaves the next first sweep
+    // in y, so an odd number of swaps starts in y
+    const int pre = c->prm.mg_pre, post = c->prm.mg_post;
+    const int swaps = m * post + (pre > 0 ? m * (pre - 1) : 0) +
+                      (startq == kStartAsIs ? (m - 1) * (pre > 0 ? 1 : 0) : 0);
+    Ls[0].x2 = c->y;
+    if (swaps % 2) {
+      Ls[0].x = c->y;
+      Ls[0].x2 = c->e32;
+      if (start0 == kStartFirstAside) start0 = kStartFirstSwept;
+    }
+  }
   for (int q = 0; q < m; ++q)
     vcycle<float>(c, Ls, 0, crtol, q == 0 ? start0 : startq, q == m - 1 ? p : nullptr);
   if (residual_updated(c))

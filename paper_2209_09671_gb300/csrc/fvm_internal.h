@@ -66,6 +66,7 @@ template <typename T>
 struct MGLevel {
   Geo geo;
   T* x;
+  T* x2 = nullptr;   // the sweeps go in pairs from x to here and swap the two (null: in place)
   T* b;
   T* beta[3];
   T w[3];            // 1 / hd^2 in the level's precision (0: no coupling)
@@ -223,6 +224,12 @@ void launch_gs_zero(const MGLevel<T>& L, int colour, cudaStream_t s);
 // a float sweep of `colour` that adds the new values of its cells and the
 // values of the other colour to the double p (p += x after the sweep); store:
 // the new values are written to x as well
+// Sweeps of colours `first` and 1 - first in one pass from L.x to L.x2 (see
+// k_gs_pair); C: apply the coarse correction first; p: add the result to it, and
+// store x2 only with `keep`.  pairs_fit: the grids it takes.
+bool pairs_fit(const Geo& g, int fx);
+void launch_gs_pair(const MGLevel<float>& L, const MGLevel<float>* C, int first, double* p,
+                    bool keep, cudaStream_t s);
 void launch_gs_addp(const MGLevel<float>& L, int colour, double* p, bool store, cudaStream_t s);
 template <typename T>
 void launch_beta_coarsen(const MGLevel<T>& F, const MGLevel<T>& C, cudaStream_t s);

@@ -498,6 +498,290 @@ __global__ void k_gs_addp(MGLevel<float> L, int colour, double* p, int store) {
   p[row + i] = p[row + i] + (double)e;
 }
 
+// ---------------------------------------------------------------------------
+// Two sweeps in one pass, float: colour a = `first` from x, then colour b from
+// the new values, both colours stored to x2.  A colour sweep reads every line of
+// x, b and the three betas and writes x: 24 bytes a cell.  A pair in one pass moves
+// 24 bytes and a halo, about 33, instead of 48.
+//
+// A thread owns two neighbouring cells of a row (one of each colour) and walks
+// planes upward: the a-cell of plane k from old values, then the b-cell of plane
+// k - 1 from new ones.  Values along z stay in registers, those along x come from
+// the neighbouring lanes, those along y from global memory (old values) or shared
+// memory (new ones).  The outermost lanes, rows and planes of a CTA compute
+// a-cells only, for the b-cells beside them: x2 is another array because other
+// CTAs still read the old values there.  Every value is that of gs_formula on the
+// same operands as in the sweeps one by one, so the results are theirs bit for bit.
+//
+// A plane's loads are issued a plane ahead into registers and kPairAhead planes
+// ahead into L2; what is left is bound by instructions (about 150 per plane and
+// warp).  Rings of planes in shared memory filled by 8-byte asynchronous copies
+// (bound by L1) or by a bulk copy per row (about 12 cycles each) took half as long
+// again.  256^3: a pair 140 us as two sweeps, about 120 here; 512 x 512 x 256: 515 and
+// 430.  Below kPairCells, where most of a level stays in L2 and the planes in a
+// row count, the sweeps one by one are as fast or faster: melt pool step at
+// 256 x 256 x 128 29.3 ms both ways, 192^3 29.2 both, 160^3 18.5 against 18.8 with
+// pairs, 128^3 9.6 against 10.3; above, 224 x 224 x 192 36.0 against 35.1, 256^3 46.7
+// against 45.5, 512 x 512 x 256 220.6 against 206.7.
+constexpr long long kPairCells = 1 << 23;
+constexpr int kPairRows = 14;      // rows of a CTA, two of them halo
+constexpr int kPairCTAs = 2;       // CTAs per SM
+constexpr int kPairAhead = 3;
+
+struct PairTiles {
+  int px, py, kz;                  // cell pairs, rows and planes of a CTA
+};
+
+template <int S>
+__device__ __forceinline__ float pick(float2 v) {
+  return S ? v.y : v.x;
+}
+
+// gs_formula for one weight on three coupled axes
+__device__ __forceinline__ float pair_formula(float wu, float b, const float* lo, const float* hi,
+                                              const float* xlo, const float* xhi) {
+  float sum = 0.f, den = 0.f;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    sum += lo[d] * xlo[d];
+    sum += hi[d] * xhi[d];
+  }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) den += lo[d] + hi[d];
+  den *= wu;
+  return (b + sum * wu) / den;
+}
+
+__device__ __forceinline__ void prefetch_l2(const float* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
+// a barrier that the rows reach from different copies of the loop
+__device__ __forceinline__ void pair_barrier() { asm volatile("bar.sync 0;" ::: "memory"); }
+
+// what a plane's step reads, fetched one step ahead
+struct PairLoad {
+  float2 xn, b, bx, yl, yh, zh;  // (xn, zh: of the plane above)
+  float ylo, yhi;                // the a-cell's neighbours in the rows beside
+  float cn, clo, chi;            // the coarse corrections of xn, ylo and yhi, added when
+                                 // they are used
+};
+
+// what a thread carries from plane to plane
+struct PairWalk {
+  float2 xp, xc, zl;             // old values of planes k - 1 and k; betas below plane k
+  float a1, a2;                  // the a-cells of planes k - 1 and k - 2
+  float pb, plo[3], phi[3];      // right-hand side and betas of plane k - 1's b-cell
+};
+
+// One thread's planes.  Neighbours wrap on walls as on periodic axes: the beta of
+// a wall's face is stored as 0 (on the low side of the first cells, where the last
+// cells find it by wrapping), and the values it multiplies are finite.
+template <bool PROLONG, bool ADDP>
+struct PairStep {
+  const MGLevel<float>& L;
+  const float* xc;               // the coarse correction
+  double* p;
+  float (*sh)[kPairRows][32];
+  int lane, r, cx;               // cx: the pair's parent in a coarse plane
+  int dlo, dhi, clo, chi;        // to the rows beside, to their parents
+  bool keep;
+
+  __device__ __forceinline__ float2 old(int o, int co) const {
+    float2 v = *reinterpret_cast<const float2*>(L.x + o);
+    if (PROLONG) {
+      const float q = xc[co + cx];
+      v.x = v.x + q;
+      v.y = v.y + q;
+    }
+    return v;
+  }
+
+  // the loads of a plane at offset o below one at on (parents at co, cn), whose
+  // a-cell is component s
+  __device__ __forceinline__ PairLoad load(int o, int on, int co, int cn, int s) const {
+    PairLoad f;
+    f.xn = *reinterpret_cast<const float2*>(L.x + on);
+    f.b = *reinterpret_cast<const float2*>(L.b + o);
+    f.bx = *reinterpret_cast<const float2*>(L.beta[0] + o);
+    f.yl = *reinterpret_cast<const float2*>(L.beta[1] + o);
+    f.yh = *reinterpret_cast<const float2*>(L.beta[1] + o + dhi);
+    f.zh = *reinterpret_cast<const float2*>(L.beta[2] + on);
+    f.ylo = L.x[o + dlo + s];
+    f.yhi = L.x[o + dhi + s];
+    if (PROLONG) {
+      f.cn = xc[cn + cx];
+      f.clo = xc[co + clo + cx];
+      f.chi = xc[co + chi + cx];
+    }
+    return f;
+  }
+
+  __device__ __forceinline__ void prefetch(int o) const {
+    prefetch_l2(L.x + o);
+    prefetch_l2(L.b + o);
+    prefetch_l2(L.beta[0] + o);
+    prefetch_l2(L.beta[1] + o);
+    prefetch_l2(L.beta[2] + o);
+  }
+
+  // plane k, whose a-cell is component S of the pair; store: plane k - 1, at offset
+  // op, is complete
+  template <int S>
+  __device__ __forceinline__ void run(PairWalk& w, PairLoad f, bool store, int op) const {
+    if (PROLONG) {
+      f.xn = make_float2(f.xn.x + f.cn, f.xn.y + f.cn);
+      f.ylo = f.ylo + f.clo;
+      f.yhi = f.yhi + f.chi;
+    }
+    const float bxr = __shfl_down_sync(0xffffffffu, f.bx.x, 1);
+    // the cells beside the a-cell: one is the pair's, one the next lane's
+    const float side = S ? __shfl_down_sync(0xffffffffu, w.xc.x, 1)
+                         : __shfl_up_sync(0xffffffffu, w.xc.y, 1);
+    const float as = S ? __shfl_down_sync(0xffffffffu, w.a1, 1)
+                       : __shfl_up_sync(0xffffffffu, w.a1, 1);
+    float a;
+    {
+      const float lo[3] = {pick<S>(f.bx), pick<S>(f.yl), pick<S>(w.zl)};
+      const float hi[3] = {S ? bxr : f.bx.y, pick<S>(f.yh), pick<S>(f.zh)};
+      const float vlo[3] = {S ? w.xc.x : side, f.ylo, pick<S>(w.xp)};
+      const float vhi[3] = {S ? side : w.xc.y, f.yhi, pick<S>(f.xn)};
+      a = pair_formula(L.wu, pick<S>(f.b), lo, hi, vlo, vhi);
+    }
+    sh[S][r][lane] = a;
+    // the b-cell of plane k - 1: component S as well; the rows beside it hold that
+    // plane's a-cells in component S too
+    if (store) {
+      const float vlo[3] = {S ? w.a1 : as, sh[S][r - 1][lane], w.a2};
+      const float vhi[3] = {S ? as : w.a1, sh[S][r + 1][lane], a};
+      const float v = pair_formula(L.wu, w.pb, w.plo, w.phi, vlo, vhi);
+      const float2 e = S ? make_float2(w.a1, v) : make_float2(v, w.a1);
+      if (!ADDP || keep) *reinterpret_cast<float2*>(L.x2 + op) = e;
+      if (ADDP) {
+        p[op] = p[op] + (double)e.x;
+        p[op + 1] = p[op + 1] + (double)e.y;
+      }
+    }
+    w.pb = pick<1 - S>(f.b);
+    w.plo[0] = pick<1 - S>(f.bx);
+    w.phi[0] = S ? f.bx.y : bxr;
+    w.plo[1] = pick<1 - S>(f.yl);
+    w.phi[1] = pick<1 - S>(f.yh);
+    w.plo[2] = pick<1 - S>(w.zl);
+    w.phi[2] = pick<1 - S>(f.zh);
+    w.a2 = w.a1;
+    w.a1 = a;
+    w.xp = w.xc;
+    w.xc = f.xn;
+    w.zl = f.zh;
+  }
+
+  // planes k0 - 1 .. k1 (plane k1 for its a-cells only) from the a-cell S of plane
+  // k0 - 1 on, two at a time so that what was fetched stays where it is
+  template <int S>
+  __device__ __forceinline__ void march(int k0, int k1, int col, int nz, int nxy, int cnxy,
+                                        bool out) const {
+    const int n = nz * nxy;
+    const auto up = [&](int o) { return o + nxy >= n ? o + nxy - n : o + nxy; };
+    const auto parent = [&](int k) {
+      return PROLONG ? coarse_index(k < 0 ? k + nz : (k >= nz ? k - nz : k), L.f[2]) * cnxy : 0;
+    };
+    int om = (k0 - 2 < 0 ? k0 - 2 + nz : k0 - 2) * nxy + col;
+    const int o = up(om);
+    int on = up(o), ahead = on;          // planes k + 1 and k + kPairAhead
+    for (int q = 1; q < kPairAhead; ++q) ahead = up(ahead);
+    PairWalk w = {};
+    w.xp = old(om, parent(k0 - 2));
+    w.xc = old(o, parent(k0 - 1));
+    w.zl = *reinterpret_cast<const float2*>(L.beta[2] + o);
+    PairLoad f = load(o, on, parent(k0 - 1), parent(k0), S), h = f;
+    int op = (k0 - 2) * nxy + col;       // plane k - 1
+    for (int k = k0 - 1;; k += 2) {
+      if (k + kPairAhead <= k1) prefetch(ahead);
+      if (k < k1) h = load(on, up(on), parent(k + 1), parent(k + 2), 1 - S);
+      run<S>(w, f, out && k > k0, op);
+      pair_barrier();
+      if (k >= k1) break;
+      on = up(on);
+      ahead = up(ahead);
+      op += nxy;
+      if (k + 1 + kPairAhead <= k1) prefetch(ahead);
+      if (k + 1 < k1) f = load(on, up(on), parent(k + 2), parent(k + 3), S);
+      run<1 - S>(w, h, out && k + 1 > k0, op);
+      pair_barrier();
+      if (k + 1 >= k1) break;
+      on = up(on);
+      ahead = up(ahead);
+      op += nxy;
+    }
+  }
+};
+
+template <bool PROLONG, bool ADDP>
+__global__ void __launch_bounds__(32 * kPairRows, kPairCTAs)
+    k_gs_pair(MGLevel<float> L, MGLevel<float> C, int first, double* p, int keep, PairTiles t) {
+  dependency_wait();
+  __shared__ float sh[2][kPairRows][32];   // the a-cells of planes k and k - 1, by component
+  const Geo& g = L.geo;
+  const int nx = g.n[0], ny = g.n[1], nz = g.n[2], nxy = nx * ny, hx = nx >> 1;
+  const int lane = threadIdx.x & 31, r = threadIdx.x >> 5;
+  // this thread's pair and row, wrapped; lanes past the halo repeat its last one,
+  // rows past it only keep the barriers
+  int i2 = blockIdx.x * t.px - 1 + min(lane, t.px + 1);
+  int j = blockIdx.y * t.py - 1 + r;
+  const bool out = lane >= 1 && lane <= t.px && i2 < hx && r >= 1 && r <= t.py && j < ny;
+  i2 = i2 < 0 ? hx - 1 : (i2 >= hx ? 0 : i2);
+  const int par = j + first;
+  j = j < 0 ? ny - 1 : (j >= ny ? 0 : j);
+  const int jlo = j == 0 ? ny - 1 : j - 1, jhi = j == ny - 1 ? 0 : j + 1;
+  const int col = j * nx + 2 * i2;
+  const int cnx = C.geo.n[0], cnxy = cnx * C.geo.n[1];
+  const int cj = coarse_index(j, L.f[1]);
+  const PairStep<PROLONG, ADDP> st = {
+      L, C.x, p, sh, lane, r, i2 + cj * cnx, (jlo - j) * nx, (jhi - j) * nx,
+      (coarse_index(jlo, L.f[1]) - cj) * cnx, (coarse_index(jhi, L.f[1]) - cj) * cnx, keep != 0};
+  const int k0 = blockIdx.z * t.kz, k1 = min(k0 + t.kz, nz);
+  if (r > t.py + 1) {
+    for (int k = k0 - 1; k <= k1; ++k) pair_barrier();
+  } else if ((par + k0 - 1) & 1) {
+    st.template march<1>(k0, k1, col, nz, nxy, cnxy, out);
+  } else {
+    st.template march<0>(k0, k1, col, nz, nxy, cnxy, out);
+  }
+}
+
+bool pairs_fit(const Geo& g, int fx) {
+  return g.N >= kPairCells && g.n[0] >= 4 && fx == 2 && g.n[1] >= 4 && g.n[2] >= 4;
+}
+
+void launch_gs_pair(const MGLevel<float>& L, const MGLevel<float>* C, int first, double* p,
+                    bool keep, cudaStream_t s) {
+  // even shares of at most 30 pairs and kPairRows - 2 rows; as many runs of planes
+  // as make the number of rounds (two CTAs per SM at a time) times the planes of a
+  // run, halo included, least
+  const int hx = L.geo.n[0] / 2, ny = L.geo.n[1], nz = L.geo.n[2];
+  const int tx = (hx + 29) / 30, ty = (ny + kPairRows - 3) / (kPairRows - 2);
+  PairTiles t;
+  t.px = (hx + tx - 1) / tx;
+  t.py = (ny + ty - 1) / ty;
+  const long long tiles = (long long)tx * ty;
+  long long best = 0;
+  t.kz = nz;
+  for (int runs = 1; 4 * runs <= nz; ++runs) {
+    const int kz = (nz + runs - 1) / runs;
+    const long long cost = (tiles * ((nz + kz - 1) / kz) + kPairCTAs * 152 - 1) / (kPairCTAs * 152) * (kz + 3);
+    if (runs == 1 || cost < best) {
+      best = cost;
+      t.kz = kz;
+    }
+  }
+  const dim3 gs(tx, ty, (nz + t.kz - 1) / t.kz);
+  void (*k)(MGLevel<float>, MGLevel<float>, int, double*, int, PairTiles) =
+      C ? (p ? k_gs_pair<true, true> : k_gs_pair<true, false>)
+        : (p ? k_gs_pair<false, true> : k_gs_pair<false, false>);
+  overlap_launch(k, gs, dim3(32 * kPairRows), 0, s, L, C ? *C : L, first, p, keep ? 1 : 0, t);
+}
+
 template <typename T>
 void launch_gs_zero(const MGLevel<T>& L, int colour, cudaStream_t s) {
   const int hx = (L.geo.n[0] + 1) / 2;
@@ -809,10 +1093,10 @@ __global__ void __launch_bounds__(256, 6)
       rd[c] = r;
       const float rf = (float)r;
       L.b[c] = rf;
-      if (y && ((i + j + k) & 1) == 0) {
+      if (y) {
         // the next inner solve's first sweep: colour 0 from 0
         const float lo[3] = {xl, yl, bzl}, hi[3] = {xh, yh, bz}, z[3] = {0.f, 0.f, 0.f};
-        y[c] = gs_formula(g, L.w, L.wu, rf, lo, hi, z, z);
+        y[c] = ((i + j + k) & 1) == 0 ? gs_formula(g, L.w, L.wu, rf, lo, hi, z, z) : 0.f;
       }
       acc = fma(r, r, acc);
       ec = en;
