@@ -672,7 +672,7 @@ struct ScalZ {
 
 // x- or y-face (D = 0, 1) fluxes of the staged plane through the low face of
 // local cell (lx, ly), global cell (i, j, k)
-template <int D, typename R>
+template <int D, bool FCT, typename R>
 __device__ __forceinline__ void plane_face(const R* __restrict__ sa, const R* __restrict__ sT,
                                            const PhysR<R>& ph, const Geo& g,
                                            const Fields<R>& X, const FctRatios<R>& fct, bool in,
@@ -688,10 +688,13 @@ __device__ __forceinline__ void plane_face(const R* __restrict__ sa, const R* __
   }
   const R U = face_u<D>(X.u[D], g, in, i, j, k);
   scal_flux(av, tv, U, ph, Fa, FT, Df);
-  if (fct.Rp) Fa = fct_flux<D>(fct, g, in, i, j, k, U, av[2], av[3], Fa);
+  if (FCT) Fa = fct_flux<D>(fct, g, in, i, j, k, U, av[2], av[3], Fa);
 }
 
-template <typename R>
+// The warps wait for instructions when the loop body is long: with the tile's far
+// faces in second turns of the same code and the flux correction (FCT) in a kernel of
+// its own, 256^3 float 1001 -> 856 us, 128^3 double 1670 -> 1570 us.
+template <bool FCT, typename R>
 __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 4 : 2)
     k_scalars(Geo g, PhysR<R> ph, TBC tb, Fields<R> X, Fields<R> Sn, Fields<R> Y,
               const double* __restrict__ dtp, R a, R b, R xc, R yc, R qamp, R ir2,
@@ -726,7 +729,7 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 4 : 2)
     }
     const R U = face_u<2>(X.u[2], g, false, i, j, z0);
     scal_flux(wa, wt, U, ph, fz0[0], fz0[1], fz0[2]);
-    if (fct.Rp) fz0[0] = fct_flux<2>(fct, g, z0 >= 1, i, j, z0, U, wa[2], wa[3], fz0[0]);
+    if (FCT) fz0[0] = fct_flux<2>(fct, g, z0 >= 1, i, j, z0, U, wa[2], wa[3], fz0[0]);
   }
   // the next plane and the next column values, loaded one step ahead
   plane_async<3, F_EVEN>(S.a[z0 & 1], X.alpha, g, tb, in, z0);
@@ -749,31 +752,29 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 4 : 2)
     }
     const R* __restrict__ sa = S.a[k & 1];
     const R* __restrict__ sT = S.T[k & 1];
-    if (i <= nx && j < ny)
-      plane_face<0>(sa, sT, ph, g, X, fct, in, tx, ty, i, j, k, S.fx[0][ty][tx], S.fx[1][ty][tx],
-                    S.fx[2][ty][tx]);
-    if (i < nx && j <= ny)
-      plane_face<1>(sa, sT, ph, g, X, fct, in, tx, ty, i, j, k, S.fy[0][ty][tx], S.fy[1][ty][tx],
-                    S.fy[2][ty][tx]);
-    if (ty == 0) {
-      // high y-faces of the tile's last row
-      const int jj = blockIdx.y * kZY + kZY;
-      if (i < nx && jj <= ny)
-        plane_face<1>(sa, sT, ph, g, X, fct, in, tx, kZY, i, jj, k, S.fy[0][kZY][tx], S.fy[1][kZY][tx],
-                      S.fy[2][kZY][tx]);
-    } else if (ty == 1 && tx < kZY) {
-      // high x-faces of the tile's last column, one row per lane
-      const int ii = blockIdx.x * kZX + kZX, jj = blockIdx.y * kZY + tx;
-      if (ii <= nx && jj < ny)
-        plane_face<0>(sa, sT, ph, g, X, fct, in, kZX, tx, ii, jj, k, S.fx[0][tx][kZX],
-                      S.fx[1][tx][kZX], S.fx[2][tx][kZX]);
+    // in a second turn of the same code (see k_momentum): the high x-faces of the
+    // tile's last column, one row per lane of a warp, and the high y-faces of its last row
+#pragma unroll 1
+    for (int t = 0; t < (ty == 1 ? 2 : 1); ++t) {
+      const int lx = t ? kZX : tx, ly = t ? tx : ty;
+      const int fi = blockIdx.x * kZX + lx, fj = blockIdx.y * kZY + ly;
+      if (ly < kZY && fi <= nx && fj < ny)
+        plane_face<0, FCT>(sa, sT, ph, g, X, fct, in, lx, ly, fi, fj, k, S.fx[0][ly][lx], S.fx[1][ly][lx],
+                      S.fx[2][ly][lx]);
+    }
+#pragma unroll 1
+    for (int t = 0; t < (ty == 0 ? 2 : 1); ++t) {
+      const int ly = t ? kZY : ty, fj = blockIdx.y * kZY + ly;
+      if (i < nx && fj <= ny)
+        plane_face<1, FCT>(sa, sT, ph, g, X, fct, in, tx, ly, i, fj, k, S.fy[0][ly][tx], S.fy[1][ly][tx],
+                      S.fy[2][ly][tx]);
     }
     R fz1[3] = {R(0), R(0), R(0)};   // fluxes through the face between k and k + 1
     R gx = R(0), gy = R(0);
     if (col) {
       const R U = face_u<2>(X.u[2], g, false, i, j, k + 1);
       scal_flux(wa + 1, wt + 1, U, ph, fz1[0], fz1[1], fz1[2]);
-      if (fct.Rp) fz1[0] = fct_flux<2>(fct, g, k + 1 <= nz - 1, i, j, k + 1, U, wa[3], wa[4], fz1[0]);
+      if (FCT) fz1[0] = fct_flux<2>(fct, g, k + 1 <= nz - 1, i, j, k + 1, U, wa[3], wa[4], fz1[0]);
       if (qamp != R(0)) {
         gx = (sa[P::at(tx + 1, ty)] - sa[P::at(tx - 1, ty)]) * i2h;
         gy = (sa[P::at(tx, ty + 1)] - sa[P::at(tx, ty - 1)]) * i2h;
@@ -837,7 +838,9 @@ void launch_scalars(const Geo& g, const Phys& ph, const TBC& tb, Fields<R> X, Fi
   double qamp = ph.q_power != 0.0 ? 2.0 * ph.q_power / (M_PI * r2) : 0.0;
   double ir2 = ph.q_power != 0.0 ? 1.0 / r2 : 0.0;
   const ZRuns z = zmarch_runs(g, sizeof(R) == 4 ? 512 : 1024, sizeof(R) == 4 ? 24 : 16);
-  k_scalars<R><<<z.grid, dim3(kZX, kZY), 0, s>>>(
+  void (*kernel)(Geo, PhysR<R>, TBC, Fields<R>, Fields<R>, Fields<R>, const double*, R, R, R, R, R, R,
+                 FctRatios<R>, int) = fct_p ? k_scalars<true, R> : k_scalars<false, R>;
+  kernel<<<z.grid, dim3(kZX, kZY), 0, s>>>(
       g, make_physr<R>(ph, g), tb, X, Sn, Y, dt, (R)a, (R)b, (R)xc, (R)ph.q_y0, (R)qamp, (R)ir2,
       FctRatios<R>{fct_p, fct_m}, z.kz);
 }
@@ -1205,7 +1208,10 @@ __device__ __forceinline__ void mz_update(const PhysR<R>& ph, bool conc, R A, R 
   phi = V + fn + fM;
 }
 
-template <typename R>
+// FULL: with what only some steps need, the concentration's part of sigma and the
+// forces stored for the adjoint.  Without their code the float kernel takes 1629 ->
+// 1569 us at 256^3; the double one, 1446 -> 1457 us at 128 x 128 x 64, keeps it.
+template <bool FULL, typename R>
 __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 3 : 2)
     k_momentum(Geo g, PhysR<R> ph, TBC tb, Fields<R> X, const R* __restrict__ kappa,
                const R* __restrict__ M0, const R* __restrict__ M1, const R* __restrict__ M2,
@@ -1224,7 +1230,7 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 3 : 2)
   const int z1 = min(z0 + kz, nz);
   const bool in = zcols_interior(g, 3);
   const bool col = i < nx && j < ny;
-  const bool conc = X.c != nullptr;
+  const bool conc = FULL && X.c != nullptr;
   const R dt = (R)dtp[0];
   const R ih = ph.ih;
   // warm-up: u, v at z0-1 and z0; w at z0 and z0+1; alpha at z0-1 .. z0+1
@@ -1298,70 +1304,64 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 3 : 2)
     const R* __restrict__ mk = S.mu[mod3(k)];
     const R* __restrict__ mm = S.mu[mod3(k - 1)];
     const R* __restrict__ mp = S.mu[mod3(k + 1)];
+    // In-plane fluxes: those of the thread's own faces and, in a second turn of the
+    // same code by one warp of each, those on the tile's high (or low) side.  As
+    // separate code the sides made the loop body two thirds longer, and the warps
+    // waited for instructions more than for anything else: 256^3 float 1744 -> 1629 us,
+    // 128^3 double 2906 -> 2787 us.
     R F[2];
-    if (col) {
-      mz_centre<0>(Uk, mk, ph, tx, ty, F[0], F[1]);
-      S.c0[0][ty][tx + 1] = F[0];
-      S.c0[1][ty][tx + 1] = F[1];
-      mz_centre<1>(Vk, mk, ph, tx, ty, F[0], F[1]);
-      S.c1[0][ty + 1][tx] = F[0];
-      S.c1[1][ty + 1][tx] = F[1];
-    }
-    if (i < nx && j <= ny) {
-      mz_e0y(Uk, Vk, mk, ph, tx, ty, F);
-      S.e0y[0][ty][tx] = F[0];
-      S.e0y[1][ty][tx] = F[1];
-      mz_e2<1>(Wk, Vk, Vm, mk, mm, ph, tx, ty, F);
-      S.e2y[0][ty][tx] = F[0];
-      S.e2y[1][ty][tx] = F[1];
-    }
-    if (i <= nx && j < ny) {
-      mz_e1x(Uk, Vk, mk, ph, tx, ty, F);
-      S.e1x[0][ty][tx] = F[0];
-      S.e1x[1][ty][tx] = F[1];
-      mz_e2<0>(Wk, Uk, Um, mk, mm, ph, tx, ty, F);
-      S.e2x[0][ty][tx] = F[0];
-      S.e2x[1][ty][tx] = F[1];
-    }
-    // the tile's high (or low) sides
-    if (ty == 0) {
-      if (i < nx && y0 + kZY <= ny) {
-        mz_e0y(Uk, Vk, mk, ph, tx, kZY, F);
-        S.e0y[0][kZY][tx] = F[0];
-        S.e0y[1][kZY][tx] = F[1];
+#pragma unroll 1
+    for (int t = 0; t < (ty == 3 ? 2 : 1); ++t) {
+      const int lx = t ? -1 : tx, ly = t ? tx : ty;
+      if (t ? tx < kZY && y0 + tx < ny : col) {
+        mz_centre<0>(Uk, mk, ph, lx, ly, F[0], F[1]);
+        S.c0[0][ly][lx + 1] = F[0];
+        S.c0[1][ly][lx + 1] = F[1];
       }
-    } else if (ty == 1) {
-      if (i < nx) {
-        mz_centre<1>(Vk, mk, ph, tx, -1, F[0], F[1]);
-        S.c1[0][0][tx] = F[0];
-        S.c1[1][0][tx] = F[1];
+    }
+#pragma unroll 1
+    for (int t = 0; t < (ty == 1 ? 2 : 1); ++t) {
+      const int ly = t ? -1 : ty;
+      if (t ? i < nx : col) {
+        mz_centre<1>(Vk, mk, ph, tx, ly, F[0], F[1]);
+        S.c1[0][ly + 1][tx] = F[0];
+        S.c1[1][ly + 1][tx] = F[1];
       }
-    } else if (ty == 2) {
-      if (i < nx && y0 + kZY <= ny) {
-        mz_e2<1>(Wk, Vk, Vm, mk, mm, ph, tx, kZY, F);
-        S.e2y[0][kZY][tx] = F[0];
-        S.e2y[1][kZY][tx] = F[1];
+    }
+#pragma unroll 1
+    for (int t = 0; t < (ty == 0 ? 2 : 1); ++t) {
+      const int ly = t ? kZY : ty;
+      if (i < nx && y0 + ly <= ny) {
+        mz_e0y(Uk, Vk, mk, ph, tx, ly, F);
+        S.e0y[0][ly][tx] = F[0];
+        S.e0y[1][ly][tx] = F[1];
       }
-    } else if (ty == 3) {
-      const int r = tx & 7, q = tx >> 3;
-      if (q == 0) {
-        if (y0 + r < ny) {
-          mz_centre<0>(Uk, mk, ph, -1, r, F[0], F[1]);
-          S.c0[0][r][0] = F[0];
-          S.c0[1][r][0] = F[1];
-        }
-      } else if (q == 1) {
-        if (x0 + kZX <= nx && y0 + r < ny) {
-          mz_e1x(Uk, Vk, mk, ph, kZX, r, F);
-          S.e1x[0][r][kZX] = F[0];
-          S.e1x[1][r][kZX] = F[1];
-        }
-      } else if (q == 2) {
-        if (x0 + kZX <= nx && y0 + r < ny) {
-          mz_e2<0>(Wk, Uk, Um, mk, mm, ph, kZX, r, F);
-          S.e2x[0][r][kZX] = F[0];
-          S.e2x[1][r][kZX] = F[1];
-        }
+    }
+#pragma unroll 1
+    for (int t = 0; t < (ty == 2 ? 2 : 1); ++t) {
+      const int ly = t ? kZY : ty;
+      if (i < nx && y0 + ly <= ny) {
+        mz_e2<1>(Wk, Vk, Vm, mk, mm, ph, tx, ly, F);
+        S.e2y[0][ly][tx] = F[0];
+        S.e2y[1][ly][tx] = F[1];
+      }
+    }
+#pragma unroll 1
+    for (int t = 0; t < (ty == 4 ? 2 : 1); ++t) {
+      const int lx = t ? kZX : tx, ly = t ? tx : ty;
+      if (ly < kZY && x0 + lx <= nx && y0 + ly < ny) {
+        mz_e1x(Uk, Vk, mk, ph, lx, ly, F);
+        S.e1x[0][ly][lx] = F[0];
+        S.e1x[1][ly][lx] = F[1];
+      }
+    }
+#pragma unroll 1
+    for (int t = 0; t < (ty == 5 ? 2 : 1); ++t) {
+      const int lx = t ? kZX : tx, ly = t ? tx : ty;
+      if (ly < kZY && x0 + lx <= nx && y0 + ly < ny) {
+        mz_e2<0>(Wk, Uk, Um, mk, mm, ph, lx, ly, F);
+        S.e2x[0][ly][lx] = F[0];
+        S.e2x[1][ly][lx] = F[1];
       }
     }
     // z-direction fluxes above plane k
@@ -1383,7 +1383,7 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 3 : 2)
       // u on the x-face (i, j, k)
       if (g.bc[0] == WALL && i == 0) {
         us0[c] = R(0);
-        if (ph0) ph0[c] = R(0);
+        if (FULL && ph0) ph0[c] = R(0);
       } else {
         MZ_SUM(S.c0[0][ty][tx + 1] - S.c0[0][ty][tx], S.e0y[0][ty + 1][tx] - S.e0y[0][ty][tx],
                ez0h[0] - ez0[0], S.c0[1][ty][tx + 1] - S.c0[1][ty][tx],
@@ -1396,12 +1396,12 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 3 : 2)
         mz_update<0>(ph, conc, A, V, ak[e1 - 1], alR, mk[e1 - 1], mR, TL, TR, cL, cR, kL, kR, ML, M0[c], Uk[e3],
                      dt, us, phv);
         us0[c] = us;
-        if (ph0) ph0[c] = phv;
+        if (FULL && ph0) ph0[c] = phv;
       }
       // v on the y-face (i, j, k)
       if (g.bc[1] == WALL && j == 0) {
         us1[c] = R(0);
-        if (ph1) ph1[c] = R(0);
+        if (FULL && ph1) ph1[c] = R(0);
       } else {
         MZ_SUM(S.c1[0][ty + 1][tx] - S.c1[0][ty][tx], S.e1x[0][ty][tx + 1] - S.e1x[0][ty][tx],
                ez1h[0] - ez1[0], S.c1[1][ty + 1][tx] - S.c1[1][ty][tx],
@@ -1414,13 +1414,13 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 3 : 2)
         mz_update<1>(ph, conc, A, V, ak[e1 - P1::PX], alR, mk[e1 - P1::PX], mR, TL, TR, cL, cR, kL, kR, ML, M1[c],
                      Vk[e3], dt, us, phv);
         us1[c] = us;
-        if (ph1) ph1[c] = phv;
+        if (FULL && ph1) ph1[c] = phv;
       }
       // w on the z-face (i, j, k)
       const R M2R = M2[c];
       if (g.bc[2] == WALL && k == 0) {
         us2[c] = R(0);
-        if (ph2) ph2[c] = R(0);
+        if (FULL && ph2) ph2[c] = R(0);
       } else {
         MZ_SUM(cc2h[0] - cc2[0], S.e2x[0][ty][tx + 1] - S.e2x[0][ty][tx],
                S.e2y[0][ty + 1][tx] - S.e2y[0][ty][tx], cc2h[1] - cc2[1],
@@ -1428,7 +1428,7 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 3 : 2)
         mz_update<2>(ph, conc, A, V, am[e1], alR, mm[e1], mR, TL2, TR, cL2, cR, kL2, kR, ML2, M2R, Wk[e3], dt,
                      us, phv);
         us2[c] = us;
-        if (ph2) ph2[c] = phv;
+        if (FULL && ph2) ph2[c] = phv;
       }
       TL2 = TR;
       kL2 = kR;
@@ -1458,9 +1458,12 @@ void launch_momentum(const Geo& g, const Phys& ph, const TBC& tb, Fields<R> X, c
                      const R* M0, const R* M1, const R* M2, R* us0, R* us1, R* us2,
                      const double* dt, cudaStream_t s, R* const* phi) {
   const int smem = (int)sizeof(MomZ<R>);
-  cudaFuncSetAttribute(k_momentum<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  void (*kernel)(Geo, PhysR<R>, TBC, Fields<R>, const R*, const R*, const R*, const R*, R*, R*, R*,
+                 const double*, R*, R*, R*, int) =
+      sizeof(R) == 8 || X.c || phi ? k_momentum<true, R> : k_momentum<false, R>;
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   const ZRuns z = zmarch_runs(g, sizeof(R) == 4 ? 512 : 1024, sizeof(R) == 4 ? 24 : 16);
-  k_momentum<R><<<z.grid, dim3(kZX, kZY), smem, s>>>(
+  kernel<<<z.grid, dim3(kZX, kZY), smem, s>>>(
       g, make_physr<R>(ph, g), tb, X, kappa, M0, M1, M2, us0, us1, us2, dt,
       phi ? phi[0] : nullptr, phi ? phi[1] : nullptr, phi ? phi[2] : nullptr, z.kz);
 }
