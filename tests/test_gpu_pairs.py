@@ -1,10 +1,11 @@
-"""The finest level's sweeps taken two at a time (float, 2^23 cells and more): the
-V-cycles of one refinement from p = 0 against the oracle's in double.  Tolerance:
-a sweep rounds a value in about 8 float operations, 5e-7 of it; two or three
-cycles of at most 8 levels and 8 sweeps make about 128 of them in a row, 6e-5 if
-they all added up.  A neighbour missed along one edge of the 24-cell tiles in one
-sweep changes the result by percents there, above 1e-3 in the norm.  The coarsest solve takes few
-iterations, the same number in both.
+"""The finest level's sweeps taken two at a time (float, 2^23 cells and more) and the
+restriction of pairs of cells (float, every axis coarsened by two): the V-cycles
+of one refinement from p = 0 against the oracle's in double.  Tolerance: a sweep
+rounds a value in about 8 float operations, 5e-7 of it; two or three cycles of at
+most 8 levels and 8 sweeps make about 128 of them in a row, 6e-5 if they all added
+up.  A neighbour missed along one edge of the 24-cell tiles in one sweep changes
+the result by percents there, above 1e-3 in the norm.  The coarsest solve takes
+few iterations, the same number in both.
 """
 import numpy as np
 import pytest
@@ -26,6 +27,9 @@ W, P_ = cases.WALL, cases.PERIODIC
     (256, 256, 129, (P_, W, W), {"mg_levels": 3, "coarse_maxit": 4, "mg_pre": 1}),
     (260, 255, 130, (W, W, P_), {"mg_levels": 3, "coarse_maxit": 4, "mg_pre": 3, "mg_post": 1}),
     (272, 176, 176, (W, W, P_), {"mg_post": 0}),
+    # sweeps one by one; the restriction's pairs at the edges of small levels
+    (36, 20, 12, (W, P_, W), {}),
+    (72, 44, 36, (P_, W, P_), {}),
 ])
 def test_cycles_equal_oracle(nx, ny, nz, bc, kw):
     P = need_gpu()
