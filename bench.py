@@ -153,6 +153,10 @@ def load_peaks():
 
 
 # the sources of the forward kernels (the adjoint's files do not change them)
+# the mixed solve's forms by grid size (csrc/fvm_api.cu, fvm_mg.cu)
+RESIDUAL_UPDATE_CELLS = 1 << 19
+RESIDUAL_UPDATE_FLOPS_PER_CELL = 6   # FP64: two FMAs on the residual, one on its norm
+SWEEP_PAIR_CELLS = 1 << 23
 FORWARD_SOURCES = ("fvm_device.cuh", "fvm_internal.h", "fvm_mg.cu", "fvm_stage.cu")
 
 
@@ -541,8 +545,8 @@ def run_droplet(args, rank, world, local_rank):
     --droplet-steps steps (at most t = 0.12 s) with dt from the stability
     limits: steps, GPU time, the droplet's centroid displacement and
     migration speed, the largest velocity, the change of the phase volume
-    and the mirror asymmetry.  100 = 4 * 25 leaves a 25 x 25 coarsest level
-    to the one-CTA CG, which makes each step slow (tens of ms)."""
+    and the mirror asymmetry.  100 = 4 * 25 leaves a 25 x 25 coarsest level,
+    solved by a float inverse with double defect correction (3 ms a step)."""
     import numpy as np
     import torch
 
@@ -785,6 +789,11 @@ def run_ours(args, rank, world, local_rank):
                             f"{args.steps} profiled steps of the same workload"}
         if cls in FP64_FLOPS_PER_CELL:
             flops = FP64_FLOPS_PER_CELL[cls] * N
+            if cls == "residual64" and N >= RESIDUAL_UPDATE_CELLS:
+                # two of a solve's launches form the residual from p, the others
+                # update it with the float correction
+                full = min(nl, 2 * 3 * args.steps)
+                flops = (full * flops + (nl - full) * RESIDUAL_UPDATE_FLOPS_PER_CELL * N) / nl
             achieved = flops / per_launch_s / 1e12
             return dict(bound="alu", achieved=achieved, peak=fma64["tflops"],
                         peak_kind="measured FP64 FMA throughput of this GPU (fvm_fma_peak)",
@@ -794,6 +803,10 @@ def run_ours(args, rank, world, local_rank):
         if bpc is None:
             return None
         cpc = compulsory_bytes_per_cell(cls, True)
+        if cls == "gs_fine" and N >= SWEEP_PAIR_CELLS:
+            # sweeps per launch: all but the cycle's first left are taken in pairs,
+            # which still move each array once
+            bpc *= (2 * p.mg_pre - 1 + 2 * p.mg_post) / (p.mg_pre + p.mg_post)
         achieved = bpc * N / per_launch_s / 1e9
         traffic = traffic_for(cls, True, N)
         return dict(bound="hbm", achieved=achieved, peak=peak,

@@ -91,7 +91,9 @@ typedef struct {
   int mg_levels, mg_pre, mg_post;          /* hierarchy depth cap, V(pre,post)    */
   int mg_max_cycles, mg_fixed_cycles;      /* fixed > 0: exactly that many cycles */
   double mg_rtol;                          /* ||b - L p|| <= rtol ||b||           */
-  double coarse_rtol; int coarse_maxit;    /* CG on the coarsest level            */
+  double coarse_rtol; int coarse_maxit;    /* the coarsest level's solve: CG, or  */
+                                           /* an inverse up to 1000 cells when    */
+                                           /* coarse_maxit covers its cells       */
   int precision;                           /* fvm_precision                       */
   int mx_inner_cycles;                     /* float V-cycles per double refinement */
   int adjoint;                             /* 1: also reserve the buffers of      */

@@ -11,6 +11,9 @@
 //                       of fvm_tail.cu, one CTA
 //   k_residual_norm2    ||b - L x||^2 partial sums
 //   k_residual64        mixed form: r = b - L p in double, stored as float
+//   k_residual_update   r -= L e in float pairs after p += e (large grids)
+//   k_gs_pair           a sweep of each colour in one pass (float, large grids)
+//   k_restrict_pairs    float residual and restriction, two cells per load
 // The paper names no linear solver; this is the reading used throughout the
 // library: V(pre, post) cycles, red first before and black first after the
 // coarse correction so that the cycle is a symmetric operator.
@@ -611,8 +614,8 @@ __global__ void k_gs_addp(MGLevel<float> L, int colour, double* p, int store) {
 // ahead into L2; what is left is bound by instructions (about 150 per plane and
 // warp).  Rings of planes in shared memory filled by 8-byte asynchronous copies
 // (bound by L1) or by a bulk copy per row (about 12 cycles each) took half as long
-// again.  256^3: a pair 140 us as two sweeps, about 120 here; 512 x 512 x 256: 515 and
-// 430.  Below kPairCells, where most of a level stays in L2 and the planes in a
+// again.  256^3: a pair 140 us as two sweeps, 101 here (123 with the prolongation, 191
+// with p += e); 512 x 512 x 256: 515 and 430.  Below kPairCells, where most of a level stays in L2 and the planes in a
 // row count, the sweeps one by one are as fast or faster: melt pool step at
 // 256 x 256 x 128 29.3 ms both ways, 192^3 29.2 both, 160^3 18.5 against 18.8 with
 // pairs, 128^3 9.6 against 10.3; above, 224 x 224 x 192 36.0 against 35.1, 256^3 46.7
