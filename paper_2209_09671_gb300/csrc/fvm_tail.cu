@@ -1101,9 +1101,13 @@ void launch_tail_pack(const TailArgs<T>& A, cudaStream_t s) {
   overlap_launch(k_tail_pack<T>, dim3(kTailCTAs, A.nl, 2), 256, 0, s, A);
 }
 
+// The limits belong to the kernel, not to a launch, and contexts of other grids
+// may launch it from other host threads: they are always set to the same values
+// (with each grid's own size a thread could lower the limit between another
+// one's setting and launch, and that launch was refused).
 template <typename T>
 void launch_tail(const TailArgs<T>& A, size_t smem, cudaStream_t s) {
-  cudaFuncSetAttribute(k_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncSetAttribute(k_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTailSmem);
   cudaFuncSetAttribute(k_tail<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kTailCTAs);
