@@ -959,6 +959,14 @@ void graph_epilogue(fvm_ctx* c, double* p) {
   TIMED(c, FVM_K_MISC, 1, launch_sub_mean(p, N, c->scal + 2, s));
 }
 
+// Whether the sweeps' launch grids (blocks of 4 rows and 2 planes) are within
+// the 65535 blocks of an axis.  A larger grid solves by launches, which report
+// FVM_ECUDA: a launch refused inside the capture of a graph's loop would not
+// end well (see body_lost).
+bool sweeps_launch(const fvm_ctx* c) {
+  return (c->g.n[1] + 3) / 4 <= 65535 && (c->g.n[2] + 1) / 2 <= 65535;
+}
+
 // the solve graph for solution pointer p (built on first use, cached); null
 // when graphs are unavailable (the caller then runs the host loop)
 cudaGraphExec_t solve_graph(fvm_ctx* c, double* p, long* nk_fixed) {
@@ -967,8 +975,16 @@ cudaGraphExec_t solve_graph(fvm_ctx* c, double* p, long* nk_fixed) {
       *nk_fixed = c->gcache[q].nk;
       return c->gcache[q].exec;
     }
+  // an error of an earlier launch is for the caller to report, not for a graph
+  if (cudaPeekAtLastError() != cudaSuccess) return nullptr;
   cudaStream_t s = c->stream;
   const cudaStreamCaptureMode mode = cudaStreamCaptureModeThreadLocal;
+  // a capture in which a launch was refused is not kept: its graph would lack
+  // that kernel in every later solve
+  const auto end_capture = [&](cudaGraph_t* out) {
+    const bool refused = cudaPeekAtLastError() != cudaSuccess;
+    return cudaStreamEndCapture(s, out) == cudaSuccess && !refused;
+  };
   cudaGraph_t g = nullptr, tmp = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaGraphConditionalHandle h = 0;
@@ -977,6 +993,7 @@ cudaGraphExec_t solve_graph(fvm_ctx* c, double* p, long* nk_fixed) {
   size_t nleaves = 0;
   const long n0 = c->nlaunch;
   long n_body = 0;
+  bool body_lost = false;
   const bool whole = solve_is_tail(c);   // one launch: nothing to loop over
   bool ok = cudaGraphCreate(&g, 0) == cudaSuccess &&
             (whole || cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault) ==
@@ -993,7 +1010,7 @@ cudaGraphExec_t solve_graph(fvm_ctx* c, double* p, long* nk_fixed) {
     if (ok)
       for (size_t q = 0; q < nd; ++q) leaves[q] = deps[q];
     nleaves = nd;
-    if (cudaStreamEndCapture(s, &tmp) != cudaSuccess) ok = false;
+    if (!end_capture(&tmp)) ok = false;
   }
   if (ok && !whole) {
     // zeroed storage: the parameter union has no default constructor
@@ -1012,7 +1029,8 @@ cudaGraphExec_t solve_graph(fvm_ctx* c, double* p, long* nk_fixed) {
         const long nb0 = c->nlaunch;
         graph_body(c, p, h);
         n_body = c->nlaunch - nb0;
-        if (cudaStreamEndCapture(s, &tmp) != cudaSuccess) ok = false;
+        if (!end_capture(&tmp)) ok = false;
+        body_lost = !ok;
       }
     }
   }
@@ -1020,13 +1038,14 @@ cudaGraphExec_t solve_graph(fvm_ctx* c, double* p, long* nk_fixed) {
     ok = cudaStreamBeginCaptureToGraph(s, g, &cond, nullptr, 1, mode) == cudaSuccess;
     if (ok) {
       graph_epilogue(c, p);
-      if (cudaStreamEndCapture(s, &tmp) != cudaSuccess) ok = false;
+      if (!end_capture(&tmp)) ok = false;
     }
   }
   if (ok) ok = cudaGraphInstantiate(&exec, g, 0) == cudaSuccess;
   const long n_fixed = c->nlaunch - n0 - n_body;
   c->nlaunch = n0;
-  if (g) cudaGraphDestroy(g);
+  // (the runtime crashes when it destroys a graph whose body's capture failed)
+  if (g && !body_lost) cudaGraphDestroy(g);
   if (!ok) {
     cudaStreamCaptureStatus cs;
     if (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone)
@@ -1281,7 +1300,7 @@ fvm_status fvm_create(const fvm_params* prm, void* workspace, size_t bytes, void
       tb.Ls = ph.L[tb.s_axis];
     }
   }
-  c->graphs_ok = 1;
+  c->graphs_ok = sweeps_launch(c) ? 1 : 0;
   if (cudaMemsetAsync(c->ctl, 0, (1 + kRecords) * sizeof(SolveCtl) + sizeof(int) +
                                      sizeof(unsigned long long), c->stream) != cudaSuccess) {
     cudaGetLastError();

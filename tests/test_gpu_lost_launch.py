@@ -66,3 +66,22 @@ def test_two_threads_with_coarse_levels_of_different_size(precision):
     for s, *_ in jobs:
         s.close()
     assert not bad, bad[0]
+
+
+@pytest.mark.parametrize("precision", [cases.F64, cases.MIXED])
+def test_refused_launch_is_reported_by_every_solve(precision):
+    """300 000 rows exceed the sweeps' launch grid (65535 blocks of 4 rows):
+    the launch is refused on the host, and every solve on that pressure field
+    returns FVM_ECUDA, the later ones as well."""
+    P = need_gpu()
+    prm, alpha, rhs = _problem(4, 300000, 1, (W, W, P_), precision)
+    prm = prm.replace(coarse_maxit=10)
+    st = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(st):
+        s = P.Solver(prm, stream=st)
+        x = torch.zeros(prm.shape, dtype=torch.float64, device="cuda")
+        got = [s.fvm_poisson_solve(alpha, rhs, x, raise_on_error=False)["status"] for _ in range(3)]
+    torch.cuda.synchronize()
+    s.close()
+    assert got == [3, 3, 3]
