@@ -538,6 +538,16 @@ int coarse_post(const fvm_ctx* c) {
   return c->prm.mg_coarse_sweeps > 0 ? c->prm.mg_coarse_sweeps : c->prm.mg_post;
 }
 
+// without a cluster every level sweeps on its own and the coarsest takes
+// conjugate gradients on one CTA
+void check_tail(fvm_ctx* c) {
+  if (c->tail.first < 0) return;
+  if (c->mixed ? tail_schedulable<float>() : tail_schedulable<double>()) return;
+  c->tail = {-1, false, 0, 0};
+  c->pack = nullptr;
+  c->inv = nullptr;
+}
+
 // the two matrices of the coarsest level's float inverse, behind its scale
 float* tail_matrix(fvm_ctx* c, int np, int which) {
   return (float*)(c->inv + 256) + (size_t)which * np * np;
@@ -1255,6 +1265,7 @@ fvm_status fvm_create(const fvm_params* prm, void* workspace, size_t bytes, void
   c->ws = (char*)workspace;
   c->ws_bytes = bytes;
   plan_workspace(*prm, c);
+  check_tail(c);
   c->g = make_geo(*prm, c->shp[0]);
   Phys& ph = c->ph;
   for (int q = 0; q < 2; ++q) {
@@ -1921,6 +1932,7 @@ extern "C" fvm_status fvm_poisson_solve_noalloc(const fvm_params* prm, const voi
   c.ws = (char*)base;
   c.ws_bytes = kNoAllocScratchBytes;
   plan_noalloc(*prm, &c, (char*)base);
+  check_tail(&c);
   c.g = make_geo(*prm, c.shp[0]);
   noalloc_physics(prm, &c);
   cudaStream_t s = c.stream;

@@ -309,6 +309,9 @@ template <typename T>
 void launch_tail_pack(const TailArgs<T>& A, cudaStream_t s);
 template <typename T>
 void launch_tail(const TailArgs<T>& A, size_t smem, cudaStream_t s);
+// false where the device cannot hold the cluster: the levels then run one by one
+template <typename T>
+bool tail_schedulable();
 // CG on a coarsest level too large for the tail, vectors in global memory
 // (double in both precisions)
 template <typename T>

@@ -1106,31 +1106,52 @@ void launch_tail_pack(const TailArgs<T>& A, cudaStream_t s) {
 // (with each grid's own size a thread could lower the limit between another
 // one's setting and launch, and that launch was refused).
 template <typename T>
-void launch_tail(const TailArgs<T>& A, size_t smem, cudaStream_t s) {
+void tail_config(size_t smem, cudaStream_t s, cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at) {
   cudaFuncSetAttribute(k_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTailSmem);
   cudaFuncSetAttribute(k_tail<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  cudaLaunchConfig_t cfg = {};
+  cfg = {};
   cfg.gridDim = dim3(kTailCTAs);
   cfg.blockDim = dim3(kTailThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute at[2];
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].val.programmaticStreamSerializationAllowed = 1;
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = kTailCTAs;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
+  cfg.numAttrs = 1;
+}
+
+template <typename T>
+void launch_tail(const TailArgs<T>& A, size_t smem, cudaStream_t s) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at[2];
+  tail_config<T>(smem, s, cfg, at);
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.numAttrs = 2;
   cudaLaunchKernelEx(&cfg, k_tail<T>, A);
+}
+
+// whether the current device (or the part of it that this process may use) can
+// hold the cluster at all
+template <typename T>
+bool tail_schedulable() {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at[1];
+  tail_config<T>(kTailSmem, nullptr, cfg, at);
+  int clusters = 0;
+  if (cudaOccupancyMaxActiveClusters(&clusters, k_tail<T>, &cfg) == cudaSuccess) return clusters > 0;
+  cudaGetLastError();
+  return false;
 }
 
 #define FVM_TAIL_INST(T)                                                                        \
   template bool tail_layout<T>(const MGLevel<T>*, int, bool, TailArgs<T>&, size_t*, size_t*);   \
   template void launch_tail_inverse<T>(const TailArgs<T>&, float*, float*, double*, cudaStream_t); \
   template void launch_tail_pack<T>(const TailArgs<T>&, cudaStream_t);                          \
-  template void launch_tail<T>(const TailArgs<T>&, size_t, cudaStream_t);
+  template void launch_tail<T>(const TailArgs<T>&, size_t, cudaStream_t);                       \
+  template bool tail_schedulable<T>();
 
 FVM_TAIL_INST(double)
 FVM_TAIL_INST(float)
