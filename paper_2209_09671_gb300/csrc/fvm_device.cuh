@@ -210,6 +210,36 @@ __device__ __forceinline__ R sigma_of_T(R T, const Phys& ph) {
   return (R)ph.sigma0 + (R)ph.dsdT * (T - (R)ph.T0);
 }
 
+// A pair of phase values as the double kernels mix them: lo + t d from the smaller
+// value lo, t the fraction of the phase with the larger one.  Every term is
+// positive, so that the mixture keeps its digits wherever the interface is; taken
+// from the larger value, p0 + a (p1 - p0), the pair (7900, 1.2) kept 12 of 16 of
+// them in the light phase (a relative error of 5e-13 in rho).
+template <typename R>
+struct Mix {
+  R lo, d;
+  int heavy0;   // phase [0] has the larger value
+};
+
+template <typename R>
+inline Mix<R> make_mix(const double* p) {
+  const int heavy0 = p[0] > p[1];
+  return {(R)p[heavy0 ? 1 : 0], (R)(heavy0 ? p[0] - p[1] : p[1] - p[0]), heavy0};
+}
+
+// the fraction t of a phase fraction: a = clamp(alpha, 0, 1), or 1 - a
+template <typename R>
+__device__ __forceinline__ R part(R alpha, const Mix<R>& m);
+template <>
+__device__ __forceinline__ double part(double alpha, const Mix<double>& m) {
+  double t = clamp01(alpha);
+  // (volatile, so that the usual order does not pay for the subtraction)
+  if (m.heavy0) asm volatile("sub.rn.f64 %0, %1, %0;" : "+d"(t) : "d"(1.0));
+  return t;
+}
+template <>
+__device__ __forceinline__ float part(float alpha, const Mix<float>&) { return clamp01(alpha); }
+
 // Material and source constants in the working precision, so that float
 // kernels carry no double arithmetic or conversions.
 template <typename R>
@@ -221,7 +251,7 @@ struct PhysR {
   R L[3];
   R h, ih;
   R dsdc, c0, diff_c[2], eps_c;
-  R drho, dmu, dlam, drcp, ddiff;   // differences [1] - [0] of the pairs
+  Mix<R> mrho, mmu, mlam, mrcp, mdiff;   // the pairs again, as the double kernels mix them
 };
 
 template <typename R>
@@ -251,19 +281,19 @@ inline PhysR<R> make_physr(const Phys& ph, const Geo& g) {
   q.diff_c[0] = (R)ph.diff_c[0];
   q.diff_c[1] = (R)ph.diff_c[1];
   q.eps_c = (R)ph.eps_c;
-  q.drho = (R)(ph.rho[1] - ph.rho[0]);
-  q.dmu = (R)(ph.mu[1] - ph.mu[0]);
-  q.dlam = (R)(ph.lam[1] - ph.lam[0]);
-  q.drcp = (R)(ph.rcp[1] - ph.rcp[0]);
-  q.ddiff = (R)(ph.diff_c[1] - ph.diff_c[0]);
+  q.mrho = make_mix<R>(ph.rho);
+  q.mmu = make_mix<R>(ph.mu);
+  q.mlam = make_mix<R>(ph.lam);
+  q.mrcp = make_mix<R>(ph.rcp);
+  q.mdiff = make_mix<R>(ph.diff_c);
   return q;
 }
 
-// arithmetic mixture of a pair (dp: its difference [1] - [0])
+// arithmetic mixture of a pair (m: the same pair)
 template <typename R>
-__device__ __forceinline__ R mixr(R alpha, const R* pair, R dp) {
+__device__ __forceinline__ R mixr(R alpha, const R* pair, const Mix<R>& m) {
+  if (sizeof(R) == 8) return m.lo + part(alpha, m) * m.d;
   R a = clamp01(alpha);
-  if (sizeof(R) == 8) return pair[0] + a * dp;
   return a * pair[1] + (R(1) - a) * pair[0];
 }
 

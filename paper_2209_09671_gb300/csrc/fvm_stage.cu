@@ -653,7 +653,7 @@ __device__ __forceinline__ void scal_flux(const R* av, const R* tv, R U, const P
                                           R& Fa, R& FT, R& Df) {
   Fa = upwind_flux(U, av, ph.eps_a);
   FT = upwind_flux(U, tv, ph.eps_T);
-  const R lL = mixr(av[2], ph.lam, ph.dlam), lR = mixr(av[3], ph.lam, ph.dlam);
+  const R lL = mixr(av[2], ph.lam, ph.mlam), lR = mixr(av[3], ph.lam, ph.mlam);
   if (sizeof(R) == 8) {
     Df = quotient((lL * lR) * ((tv[3] - tv[2]) * (R(2) * ph.ih)), lL + lR);
   } else {
@@ -784,7 +784,7 @@ __global__ void __launch_bounds__(kZT, sizeof(R) == 4 ? 4 : 2)
     if (col) {
       const int c = (k * ny + j) * nx + i;
       const R al = wa[3];
-      const R rcp = mixr(al, ph.rcp, ph.drcp);
+      const R rcp = mixr(al, ph.rcp, ph.mrcp);
       R Ra, RT;
       if (sizeof(R) == 8) {
         Ra = -(((S.fx[0][ty][tx + 1] - S.fx[0][ty][tx]) +
@@ -949,7 +949,7 @@ __global__ void __launch_bounds__(kThreads)
   stage<3, F_EVEN, 0>(S.c, X.c, g, tb);
   stage<1, F_EVEN, 0>(S.D, X.alpha, g, tb);
   __syncthreads();
-  for (int e = flat_tid(); e < Tile<1>::N; e += kThreads) S.D[e] = mixr(S.D[e], ph.diff_c, ph.ddiff);
+  for (int e = flat_tid(); e < Tile<1>::N; e += kThreads) S.D[e] = mixr(S.D[e], ph.diff_c, ph.mdiff);
   const bool in = tile_interior(g, 3);
   __syncthreads();
   const R dt = (R)dtp[0];
@@ -1049,17 +1049,18 @@ __device__ __forceinline__ R cell_at(const R* __restrict__ a, const Geo& g, cons
 }
 
 // What the planes hold for the viscosity: mu(alpha) in float; in double the
-// clamped phase fraction, of which mu is linear (so that the mean over four
-// cells and the densities come from it in two operations)
+// fraction of the more viscous phase, of which mu is linear (so that the mean over
+// four cells and, when the heavier phase is the same one, the densities come from
+// it in two operations)
 template <typename R>
 __device__ __forceinline__ R mz_mu(R alpha, const PhysR<R>& ph) {
-  return sizeof(R) == 8 ? clamp01(alpha) : mixr(alpha, ph.mu, ph.dmu);
+  return sizeof(R) == 8 ? part(alpha, ph.mmu) : mixr(alpha, ph.mu, ph.mmu);
 }
 
 // viscous flux 2 mu du/dx of a face pair in a cell
 template <typename R>
 __device__ __forceinline__ R mz_visc(R mu, R du, const PhysR<R>& ph) {
-  if (sizeof(R) == 8) return ((R(2) * ph.ih * ph.dmu) * mu + R(2) * ph.ih * ph.mu[0]) * du;
+  if (sizeof(R) == 8) return ((R(2) * ph.ih * ph.mmu.d) * mu + R(2) * ph.ih * ph.mmu.lo) * du;
   return R(2) * mu * du * ph.ih;
 }
 
@@ -1095,7 +1096,7 @@ template <typename R>
 __device__ __forceinline__ void mz_edge(const R* v, R ut_lo, R ut_hi, R m0, R m1, R m2, R m3,
                                         const PhysR<R>& ph, R& Fa, R& Fv) {
   const R mue = sizeof(R) == 8
-                    ? (R(0.25) * ph.ih * ph.dmu) * ((m0 + m1) + (m2 + m3)) + ph.ih * ph.mu[0]
+                    ? (R(0.25) * ph.ih * ph.mmu.d) * ((m0 + m1) + (m2 + m3)) + ph.ih * ph.mmu.lo
                     : R(0.25) * (m0 + m1 + m2 + m3);
   const R Ue = R(0.5) * (ut_lo + ut_hi);
   Fa = upwind_flux(Ue, v, ph.eps_u);
@@ -1181,15 +1182,20 @@ __device__ __forceinline__ void mz_ez(const R* v, const R* Wu, const R* muu, con
   }
 
 // the forces on a D-face between cell L and cell R and the new face velocity
-// (mL, mR: the cells' viscosity measures, in double their clamped phase
-// fractions; sigma_f is then the linear sigma(c, T) of the mean T and c)
+// (mL, mR: the cells' viscosity measures, in double the fractions of the more
+// viscous phase; sigma_f is then the linear sigma(c, T) of the mean T and c)
 template <int D, typename R>
 __device__ __forceinline__ void mz_update(const PhysR<R>& ph, bool conc, R A, R V, R alL, R alR,
                                           R mL, R mR, R TL, R TR, R cL, R cR, R kL, R kR, R ML,
                                           R MR, R uf, R dt, R& us, R& phi) {
   const R ih = ph.ih;
   if (sizeof(R) == 8) {
-    const R rho_f = (R(0.5) * ph.drho) * (mL + mR) + ph.rho[0];
+    R tL = mL, tR = mR;
+    if (ph.mrho.heavy0 != ph.mmu.heavy0) {
+      tL = part(alL, ph.mrho);
+      tR = part(alR, ph.mrho);
+    }
+    const R rho_f = (R(0.5) * ph.mrho.d) * (tL + tR) + ph.mrho.lo;
     R sig_f = ph.dsdT * (R(0.5) * (TL + TR) - ph.T0) + ph.sigma0;
     if (conc) sig_f += ph.dsdc * (R(0.5) * (cL + cR) - ph.c0);
     const R fn = (sig_f * (R(-0.5) * ih)) * ((kL + kR) * (alR - alL));
@@ -1197,7 +1203,7 @@ __device__ __forceinline__ void mz_update(const PhysR<R>& ph, bool conc, R A, R 
     us = uf + dt * (A + quotient(phi, rho_f) + ph.g[D]);
     return;
   }
-  const R rho_f = R(0.5) * (mixr(alL, ph.rho, ph.drho) + mixr(alR, ph.rho, ph.drho));
+  const R rho_f = R(0.5) * (mixr(alL, ph.rho, ph.mrho) + mixr(alR, ph.rho, ph.mrho));
   const R sig_f = conc ? R(0.5) * (sigma_rc(TL, cL, ph) + sigma_rc(TR, cR, ph))
                        : R(0.5) * (sigma_r(TL, ph) + sigma_r(TR, ph));
   const R kap_f = R(0.5) * (kL + kR);
