@@ -113,11 +113,12 @@ __device__ __forceinline__ R clamp01(R a) {
 // The FP64 pipe of an SM takes 2 lanes a clock and runs double comparisons
 // too; the double kernels are bound by it, so signs and ranges are read from
 // the bit pattern with integer instructions (64 times the rate).
+// (NaN passes through, as in the general form; a negative zero becomes 0.)
 template <>
 __device__ __forceinline__ double clamp01(double a) {
-  const int hi = __double2hiint(a);
-  double r = (hi >= 0x3ff00000 && hi < 0x7ff00000) ? 1.0 : a;   // (not a NaN or an infinity)
-  return (hi < 0 && (unsigned)hi < 0xfff00000u) ? 0.0 : r;
+  const long long b = __double_as_longlong(a);
+  const double r = b >= 0x3ff0000000000000LL && b <= 0x7ff0000000000000LL ? 1.0 : a;
+  return b < 0 && (unsigned long long)b <= 0xfff0000000000000ULL ? 0.0 : r;
 }
 
 // a value below 0 (a zero's sign is as good as any where this is used)

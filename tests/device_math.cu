@@ -1,0 +1,26 @@
+// Entry points for tests/test_gpu_device_math.py: the device helpers of
+// fvm_device.cuh beside the instructions they replace, one value per thread.
+#include "fvm_device.cuh"
+
+using namespace fvm;
+
+namespace {
+
+template <typename F>
+__global__ void k_each(long long n, F f) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i < n) f(i);
+}
+
+template <typename F>
+int each(long long n, F f) {
+  k_each<<<(unsigned)((n + 255) / 256), 256>>>(n, f);
+  const cudaError_t e = cudaGetLastError();
+  return e != cudaSuccess ? (int)e : (int)cudaDeviceSynchronize();
+}
+
+}  // namespace
+
+extern "C" int dm_clamp01(long long n, const double* a, double* out) {
+  return each(n, [=] __device__(long long i) { out[i] = clamp01(a[i]); });
+}

@@ -1,0 +1,58 @@
+"""The arithmetic helpers of the double kernels (fvm_device.cuh), which stand
+in for comparisons, conversions, quotients and roots of the FP64 pipe: each
+against the plain operation, over all exponents and on both sides of every
+branch of the helper."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2209_09671_gb300 import _build
+from tests.gpu_util import need_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dm(tmp_path_factory):
+    need_gpu()
+    so = str(tmp_path_factory.mktemp("dm") / "device_math.so")
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "device_math.cu")
+    r = subprocess.run([_build.nvcc(), *_build.ARCH, *_build.FLAGS, "--extended-lambda", "-shared",
+                        "-I", _build.CSRC, "-I", os.path.join(os.path.dirname(_build.HERE), "include"),
+                        src, "-o", so], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return ctypes.CDLL(so)
+
+
+def _run(fn, ins, out_dtype=torch.float64):
+    """fn(n, inputs..., out) on the device; numpy in, numpy out."""
+    dev = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in ins]
+    out = torch.empty(dev[0].shape, dtype=out_dtype, device="cuda")
+    torch.cuda.synchronize()
+    assert fn(ctypes.c_longlong(dev[0].numel()), *[ctypes.c_void_p(t.data_ptr()) for t in dev],
+              ctypes.c_void_p(out.data_ptr())) == 0
+    return out.cpu().numpy()
+
+
+def _doubles(seed, per_exponent=8):
+    """Random mantissas at every exponent of both signs, with each exponent's
+    first and last mantissa, zeros, infinities and NaN."""
+    rng = np.random.default_rng(seed)
+    e = np.arange(2047, dtype=np.uint64)[:, None]
+    m = rng.integers(0, 1 << 52, (2047, per_exponent), dtype=np.uint64)
+    m[:, 0], m[:, 1] = 0, (1 << 52) - 1
+    b = ((e << np.uint64(52)) | m).ravel()
+    a = np.concatenate([b, b | np.uint64(1 << 63)]).view(np.float64)
+    return np.concatenate([a, [0.0, -0.0, np.inf, -np.inf, np.nan, -np.nan]])
+
+
+def test_clamp01(dm):
+    """0 below 0, 1 above 1, infinities included; NaN stays NaN."""
+    a = np.concatenate([_doubles(1), np.linspace(-1.0, 2.0, 3001), np.nextafter(1.0, [0.0, 2.0])])
+    got = _run(dm.dm_clamp01, [a])
+    want = np.where(a < 0.0, 0.0, np.where(a > 1.0, 1.0, a))
+    assert np.array_equal(got, want, equal_nan=True)
