@@ -24,3 +24,7 @@ int each(long long n, F f) {
 extern "C" int dm_clamp01(long long n, const double* a, double* out) {
   return each(n, [=] __device__(long long i) { out[i] = clamp01(a[i]); });
 }
+
+extern "C" int dm_root(long long n, const double* a, double* out) {
+  return each(n, [=] __device__(long long i) { out[i] = root(a[i]); });
+}

@@ -56,3 +56,27 @@ def test_clamp01(dm):
     got = _run(dm.dm_clamp01, [a])
     want = np.where(a < 0.0, 0.0, np.where(a > 1.0, 1.0, a))
     assert np.array_equal(got, want, equal_nan=True)
+
+
+U = 2.0 ** -53
+
+
+def _near(t):
+    """The numbers around t > 0: its neighbours and some more on both sides."""
+    b = np.float64(t).view(np.int64) + np.array([-3, -2, -1, 0, 1, 2, 3])
+    return np.concatenate([b.view(np.float64), t * np.linspace(0.5, 2.0, 301)])
+
+
+def test_root(dm):
+    """The approximate reciprocal root is good to 20 bits in its operand and in
+    its result: a relative error d of at most 3 2^-20.  After the step on it
+    the error is 3/2 d^2 + u (u = 2^-53, the rounding of the sum), which the last
+    step multiplies by d: 0.33 u; with its own rounding 1.4 u of the root."""
+    a = np.abs(np.concatenate([_doubles(2, 64), _near(2.0 ** -960), _near(2.0 ** 960)]))
+    got = _run(dm.dm_root, [a])
+    ok = np.isfinite(a)
+    want = np.sqrt(a[ok].astype(np.longdouble))
+    assert (np.abs(got[ok] - want) <= 1.4 * U * want).all()
+    assert np.array_equal(got[~ok], np.sqrt(a[~ok]), equal_nan=True)
+    edge = ok & ((a < 2.0 ** -960) | (a >= 2.0 ** 960))
+    assert np.array_equal(got[edge], np.sqrt(a[edge]))
