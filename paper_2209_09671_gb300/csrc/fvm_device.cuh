@@ -148,7 +148,7 @@ __device__ __forceinline__ double widen(float f) {
   const unsigned u = __float_as_uint(f), mag = u & 0x7fffffffu;
   double d = __hiloint2double((int)((u & 0x80000000u) | ((mag >> 3) + 0x38000000u)), (int)(u << 29));
   if (mag - 0x00800000u >= 0x7f000000u) {
-    d = 0.0;
+    d = __hiloint2double((int)(u & 0x80000000u), 0);
     if (mag != 0u) asm volatile("cvt.f64.f32 %0, %1;" : "=d"(d) : "f"(f));
   }
   return d;

@@ -28,3 +28,11 @@ extern "C" int dm_clamp01(long long n, const double* a, double* out) {
 extern "C" int dm_root(long long n, const double* a, double* out) {
   return each(n, [=] __device__(long long i) { out[i] = root(a[i]); });
 }
+
+// counts the float bit patterns whose widen() is not the conversion's
+extern "C" int dm_widen_all(unsigned long long* differ) {
+  return each(1LL << 32, [=] __device__(long long i) {
+    const float f = __uint_as_float((unsigned)i);
+    if (__double_as_longlong(widen(f)) != __double_as_longlong((double)f)) atomicAdd(differ, 1ULL);
+  });
+}

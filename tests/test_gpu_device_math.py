@@ -80,3 +80,11 @@ def test_root(dm):
     assert np.array_equal(got[~ok], np.sqrt(a[~ok]), equal_nan=True)
     edge = ok & ((a < 2.0 ** -960) | (a >= 2.0 ** 960))
     assert np.array_equal(got[edge], np.sqrt(a[edge]))
+
+
+def test_widen(dm):
+    """Every float, bit for bit."""
+    differ = torch.zeros(1, dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+    assert dm.dm_widen_all(ctypes.c_void_p(differ.data_ptr())) == 0
+    assert differ.item() == 0
