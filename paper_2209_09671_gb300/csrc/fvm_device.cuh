@@ -126,8 +126,12 @@ __device__ __forceinline__ bool is_negative(double a) { return __double2hiint(a)
 __device__ __forceinline__ bool is_negative(float a) { return __float_as_int(a) < 0; }
 
 // n / d to about a unit in the last place: the hardware's approximate
-// reciprocal (20 bits) and one step of third order, y (1 + e + e^2) with e =
-// 1 - d y, 4 FP64 operations instead of the about 10 of an IEEE division.  An
+// reciprocal y and the geometric series 1/d = y / (1 - e) = y (1 + e + e^2 + ...),
+// e = 1 - d y, cut after three terms (the hyperpower iteration of order three;
+// Altman, Pacific J. Math. 10, 1960), 4 FP64 operations instead of the about 10
+// of an IEEE division.  y is good to 20 bits in its operand and in its result,
+// |e| <= 3 2^-20, so that the cut leaves e^3 = 0.21 u (u = 2^-53); with the
+// roundings of the series' product and of the last one 2.3 u of the value.  An
 // operand outside [2^-960, 2^960] takes the division.
 __device__ __forceinline__ double quotient(double n, double d) {
   const unsigned u = (unsigned)__double2hiint(d) & 0x7fffffffu;
@@ -176,18 +180,19 @@ __device__ __forceinline__ float narrow<float>(double d) {
 }
 
 // sqrt(a) for a >= 0 to about a unit in the last place: the approximate
-// reciprocal root y and one Newton step on a y, with the rounding error of
-// that product (5 FP64 operations instead of about 15).  Operands outside
-// [2^-960, 2^960] take the root instruction.  A 0, which most cells (away from
-// the interface) pass, is returned first: inside that branch it cost the
-// 149 x 90 x 75 predictor 2.81 -> 2.93 ms.
+// reciprocal root y, whose error Newton's iteration for a^-1/2 (a y (1 + e/2), e =
+// 1 - a y^2) and then Newton's iteration for the root (z + (a - z^2) / (2 z), with y
+// for 1/z) square away: 5 FP64 operations instead of about 15.  With y good to d =
+// 3 2^-20, z is to 3/2 d^2 + u and the result to that times d and its rounding, 1.4 u.
+// Operands outside [2^-960, 2^960] take the root instruction.  A 0, which most
+// cells (away from the interface) pass, is returned first: inside that branch it
+// cost the 149 x 90 x 75 predictor 2.81 -> 2.93 ms.
 __device__ __forceinline__ double root(double a) {
   const int hi = __double2hiint(a);
   if ((hi | __double2loint(a)) == 0) return 0.0;
   if ((unsigned)(hi - 0x03f00000) >= 0x78000000u) return sqrt(a);
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-  // y refined once (error e -> 3/8 e^2, 2^-38), then the root from it
   const double ay = a * y;
   const double e = fma(-ay, y, 1.0);
   const double z = fma(0.5 * e, ay, ay);            // a y (1 + e/2)

@@ -29,6 +29,25 @@ extern "C" int dm_root(long long n, const double* a, double* out) {
   return each(n, [=] __device__(long long i) { out[i] = root(a[i]); });
 }
 
+extern "C" int dm_quotient(long long n, const double* a, const double* b, double* out) {
+  return each(n, [=] __device__(long long i) { out[i] = quotient(a[i], b[i]); });
+}
+
+// the plain division, root and conversion on the device
+extern "C" int dm_divide(long long n, const double* a, const double* b, double* out) {
+  return each(n, [=] __device__(long long i) { out[i] = a[i] / b[i]; });
+}
+extern "C" int dm_sqrt(long long n, const double* a, double* out) {
+  return each(n, [=] __device__(long long i) { out[i] = sqrt(a[i]); });
+}
+
+extern "C" int dm_narrow(long long n, const double* a, float* out) {
+  return each(n, [=] __device__(long long i) { out[i] = narrow<float>(a[i]); });
+}
+extern "C" int dm_to_float(long long n, const double* a, float* out) {
+  return each(n, [=] __device__(long long i) { out[i] = (float)a[i]; });
+}
+
 // counts the float bit patterns whose widen() is not the conversion's
 extern "C" int dm_widen_all(unsigned long long* differ) {
   return each(1LL << 32, [=] __device__(long long i) {

@@ -80,6 +80,36 @@ def test_root(dm):
     assert np.array_equal(got[~ok], np.sqrt(a[~ok]), equal_nan=True)
     edge = ok & ((a < 2.0 ** -960) | (a >= 2.0 ** 960))
     assert np.array_equal(got[edge], np.sqrt(a[edge]))
+    # (the root instruction is within u of the exact root)
+    assert (np.abs(got[ok] - _run(dm.dm_sqrt, [a])[ok]) <= 2.4 * U * want).all()
+
+
+def test_quotient(dm):
+    """|e| <= 3 2^-20 leaves e^3 = 0.21 u, the series' product and the last one
+    round by u each: 2.3 u of n / d.  A result below the normal numbers is rounded
+    once more, by half a unit of 2^-1074."""
+    d = np.concatenate([_doubles(3, 64), _near(2.0 ** -960), -_near(2.0 ** 960)])
+    rng = np.random.default_rng(4)
+    for scale in (None, 0, 500, -500):
+        n = rng.permutation(_doubles(5, 64))[np.arange(d.size) % 262000]
+        if scale is not None:   # a quotient of about 2^scale
+            n = np.ldexp(rng.uniform(1.0, 2.0, d.size), np.clip(np.frexp(d)[1] + scale, -1074, 1023))
+        got = _run(dm.dm_quotient, [n, d])
+        cuda = _run(dm.dm_divide, [n, d])
+        inside = (np.abs(d) >= 2.0 ** -960) & (np.abs(d) < 2.0 ** 960)
+        assert np.array_equal(got[~inside], cuda[~inside], equal_nan=True)
+        fin = inside & np.isfinite(n) & np.isfinite(cuda) & (np.abs(cuda) < 1.7e308)
+        assert fin.sum() > 1000
+        want = n[fin].astype(np.longdouble) / d[fin].astype(np.longdouble)
+        tol = 2.3 * U * np.abs(want) + 2.0 ** -1074
+        assert (np.abs(got[fin] - want) <= tol).all()
+        # (the division is within u of the exact quotient)
+        assert (np.abs(got[fin] - cuda[fin]) <= tol + U * np.abs(want)).all()
+        # infinities, NaN and overflow as the division has them (beyond the last
+        # numbers whose quotient the 2.3 u could take over the limit)
+        big = np.abs(n.astype(np.longdouble) / np.where(inside, d, 1.0).astype(np.longdouble))
+        sat = inside & ~(big <= np.longdouble(2.0) ** 1024 * (1.0 + 2.0 ** -50))
+        assert np.array_equal(got[sat], cuda[sat], equal_nan=True)
 
 
 def test_widen(dm):
@@ -88,3 +118,24 @@ def test_widen(dm):
     torch.cuda.synchronize()
     assert dm.dm_widen_all(ctypes.c_void_p(differ.data_ptr())) == 0
     assert differ.item() == 0
+
+
+def test_narrow(dm):
+    """Bit for bit: every exponent, the bits below a float's last one at 0, at
+    and around a tie and random, odd and even last bits; the numbers that round
+    to 2^128 and the subnormal ones among them."""
+    rng = np.random.default_rng(6)
+    e = np.arange(2048, dtype=np.uint64)[:, None, None]
+    top = np.concatenate([rng.integers(0, 1 << 23, 60, dtype=np.uint64),
+                          np.array([0, 1, 2, (1 << 23) - 2, (1 << 23) - 1], dtype=np.uint64)])[:, None]
+    low = np.concatenate([np.array([0, 1, (1 << 28) - 1, 1 << 28, (1 << 28) + 1, (1 << 29) - 1],
+                                   dtype=np.uint64), rng.integers(0, 1 << 29, 10, dtype=np.uint64)])
+    b = ((e << np.uint64(52)) | (top << np.uint64(29)) | low).ravel()
+    a = np.concatenate([b, b | np.uint64(1 << 63)]).view(np.float64)
+    got = _run(dm.dm_narrow, [a], torch.float32)
+    cuda = _run(dm.dm_to_float, [a], torch.float32)
+    assert np.array_equal(got.view(np.uint32), cuda.view(np.uint32))
+    with np.errstate(over="ignore", invalid="ignore"):
+        host = a.astype(np.float32)
+    num = ~np.isnan(a)
+    assert np.array_equal(got[num].view(np.uint32), host[num].view(np.uint32))
