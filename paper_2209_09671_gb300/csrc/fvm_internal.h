@@ -104,6 +104,18 @@ inline void overlap_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
   cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
+
+// Offset of the cell above one at offset o, in planes of nxy cells, n in all; the
+// last plane wraps to the first.  n may be as large as 2^31 - 1, so that o + nxy is
+// formed without a sign.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int plane_above(int o, int nxy, int n) {
+  const unsigned a = (unsigned)o + (unsigned)nxy;
+  return (int)(a >= (unsigned)n ? a - (unsigned)n : a);
+}
+
 #ifdef __CUDACC__
 // wait for the predecessor, and let the successor be scheduled
 __device__ __forceinline__ void dependency_wait() {

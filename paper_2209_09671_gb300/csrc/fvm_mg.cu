@@ -779,7 +779,7 @@ struct PairStep {
   __device__ __forceinline__ void march(int k0, int k1, int col, int nz, int nxy, int cnxy,
                                         bool out) const {
     const int n = nz * nxy;
-    const auto up = [&](int o) { return o + nxy >= n ? o + nxy - n : o + nxy; };
+    const auto up = [&](int o) { return plane_above(o, nxy, n); };
     const auto parent = [&](int k) {
       return PROLONG ? coarse_index(k < 0 ? k + nz : (k >= nz ? k - nz : k), L.f[2]) * cnxy : 0;
     };
