@@ -472,7 +472,7 @@ struct SweepFold {
   const MGLevel<T>* corr = nullptr;   // first sweep: the coarse correction of this level (prolongation)
   bool zero = false;                  // first sweep: x starts at 0 (zeroes the other colour)
   bool skip_first = false;            // first sweep: already taken (by the residual pass)
-  const T* xin = nullptr;             // second sweep: the first one's values are here (its colour only)
+  const T* xin = nullptr;             // second sweep: the first one's values are here (0 in its own colour)
   bool keep = false;                  // last sweep with addp: store x as well
   const int* gate = nullptr;          // first sweep: skipped on the device once *gate >= gate_min
   int gate_min = 0;
@@ -604,7 +604,7 @@ void coarsen_betas(fvm_ctx* c, MGLevel<T>* Ls) {
 // first sweep already taken (by k_residual64 in the mixed form, or skipped
 // because it would repeat the previous cycle's last sweep), or with that skip
 // decided on the device (FP64 solve graph: from the second cycle on).
-// kStartFirstAside: the first sweep was taken into c->y (colour 0 only).
+// kStartFirstAside: the first sweep was taken into c->y (colour 0; colour 1 is 0 there).
 enum { kStartAsIs = 0, kStartZero = 1, kStartFirstSwept = 2, kStartGated = 3, kStartFirstAside = 4 };
 
 // a cycle's first finest-level sweep repeats the previous cycle's last one

@@ -233,15 +233,15 @@ void launch_gs_prolong(const MGLevel<T>& F, const MGLevel<T>& C, int colour, cud
 // a sweep of `colour` from x = 0 that also zeroes the other colour
 template <typename T>
 void launch_gs_zero(const MGLevel<T>& L, int colour, cudaStream_t s);
-// a float sweep of `colour` that adds the new values of its cells and the
-// values of the other colour to the double p (p += x after the sweep); store:
-// the new values are written to x as well
 // Sweeps of colours `first` and 1 - first in one pass from L.x to L.x2 (see
 // k_gs_pair); C: apply the coarse correction first; p: add the result to it, and
 // store x2 only with `keep`.  pairs_fit: the grids it takes.
 bool pairs_fit(const Geo& g, int fx);
 void launch_gs_pair(const MGLevel<float>& L, const MGLevel<float>* C, int first, double* p,
                     bool keep, cudaStream_t s);
+// a float sweep of `colour` that adds the new values of its cells and the
+// values of the other colour to the double p (p += x after the sweep); store:
+// the new values are written to x as well
 void launch_gs_addp(const MGLevel<float>& L, int colour, double* p, bool store, cudaStream_t s);
 template <typename T>
 void launch_beta_coarsen(const MGLevel<T>& F, const MGLevel<T>& C, cudaStream_t s);
@@ -265,7 +265,12 @@ constexpr int kTailSmem = 220 * 1024;       // shared memory of a CTA
 constexpr int kTailCells32 = 512, kTailCells64 = 256;   // cells a CTA should have (float, double)
 constexpr int kTailCgCells = 64, kTailCgSingle = 400;    // the same for the coarsest level's CG
 constexpr int kTailInvCells = 32;           // the same for the coarsest level by a float inverse
-constexpr int kTailInvMax = 1000;           // cells of a coarsest level solved with one
+// Cells of a coarsest level solved with a float inverse.  It replaces only conjugate
+// gradients that the caller's iteration cap (1000 by default) does not cut short,
+// so that a larger limit changes nothing by default.  With a cap of 4000, six cycles
+// in double: 961 cells 0.96 ms; 1089 cells 12.0 ms by conjugate gradients, 1.36 with
+// the limit at 2048; 2025 cells 15.9 and 3.4 ms.
+constexpr int kTailInvMax = 1000;
 template <typename T>
 struct TailLevel {
   int n[3], f[3];              // cells per axis, coarsening factor to the next level
@@ -340,7 +345,7 @@ void launch_residual64(const Geo& g, const double* p, const double* b, float* co
                        float* e32 = nullptr, const float* w32 = nullptr, double* rd = nullptr,
                        const int* gate = nullptr);
 // rd -= L e (L.x) and the same outputs: r32 (L.b), ||r||^2, and with y the next
-// inner solve's first sweep (its colour 0 only)
+// inner solve's first sweep (colour 0; colour 1 is set to 0)
 void launch_residual_update(const MGLevel<float>& L, double* rd, float* y, double* partial,
                             double* out, cudaStream_t s);
 void launch_add_correction(long long n, double* p, const float* e, cudaStream_t s);

@@ -1012,7 +1012,7 @@ void launch_concentration(const Geo& g, const Phys& ph, Fields<R> X, Fields<R> S
 // of u, v and w are register windows of the thread's column, and the fluxes
 // through the z-facing sides of a control volume are carried from one plane
 // to the next.  Every flux is evaluated once: each thread takes those of its
-// own faces, four warps the ones on the tile's high (or low) side.
+// own faces, six of the eight warps one kind each on the tile's high (or low) side.
 template <typename R>
 struct MomZ {
   R u[3][Plane<3>::N];    // u planes (m mod 3)
