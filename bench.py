@@ -152,12 +152,14 @@ def load_peaks():
         return FALLBACK_HBM, "fallback"
 
 
-# the sources of the forward kernels (the adjoint's files do not change them)
 # the mixed solve's forms by grid size (csrc/fvm_api.cu, fvm_mg.cu)
 RESIDUAL_UPDATE_CELLS = 1 << 19
 RESIDUAL_UPDATE_FLOPS_PER_CELL = 6   # FP64: two FMAs on the residual, one on its norm
 SWEEP_PAIR_CELLS = 1 << 23
-FORWARD_SOURCES = ("fvm_device.cuh", "fvm_internal.h", "fvm_mg.cu", "fvm_stage.cu")
+# the sources that decide the forward kernels' traffic: the kernels, and the
+# forms that the solve takes of them (the adjoint's files do not change it)
+FORWARD_SOURCES = ("fvm_api.cu", "fvm_device.cuh", "fvm_internal.h", "fvm_mg.cu", "fvm_stage.cu",
+                   "fvm_tail.cu")
 
 
 def source_hash() -> str:
