@@ -354,7 +354,8 @@ __device__ void edge_flux(const AdjArgs& A, int i, int j, int k, int l, int q0) 
     off3<T_>(a3, b3, c3, -1);
     int a4 = a3, b4 = b3, c4 = c3;
     off3<D>(a4, b4, c4, -1);
-    // the mean of mu over the edge's four cells, mu linear in the phase fraction
+    // the mean of mu over the edge's four cells, mu linear in the phase fraction (the
+    // step adjoint is taken only with equal mu in both phases, so that this is exact)
     const double cs = (clamp01(val(A.X[3], r_even(g, i, j, k))) +
                        clamp01(val(A.X[3], r_even(g, a2, b2, c2)))) +
                       (clamp01(val(A.X[3], r_even(g, a3, b3, c3))) +
